@@ -106,7 +106,12 @@ struct mgmc_ctx {
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t exec = nullptr;
     int launches = 0;
-    size_t coarse_smem = 0;   // dynamic shared memory of the coarse-grid kernel
+    CoarsePlan plan{};        // shared-memory plan, phases and coarsest-grid matrices of the coarse kernel
+    int4* coarse_ops = nullptr;
+    int coarse_nops = 0;
+    unsigned char* coarse_image = nullptr;
+    double* gain = nullptr;
+    double* e0 = nullptr;
     bool fused = false;   // 2D, nu1 = nu2 = 1: fused tile kernels on the grids above coarse_max_n
     bool recursive = false;   // W-cycle or radius-2 grids: general kernels, cycle enqueued recursively
     // recursive path, 2D: grids 0..small_top run in one k_cycle_small launch per visit of
@@ -180,6 +185,30 @@ V* upload(mgmc_ctx* h, const std::vector<V>& v, mgmc_status& st)
     return p;
 }
 
+// The coarse kernel's phases: the V-cycle on grids top .. 0.  Flags of a sweep: bit 0
+// backward, bit 1 not pre-drawn; of a low-rank step: bit 0 backward, bit 1 no smoothing
+// before it, bit 2 forms d_{l-1}; of a prolongation: bit 1 draws the backward sweep's normals.
+void coarse_phases(const mgmc_ctx* h, std::vector<int4>& ops)
+{
+    const int nu1 = h->cfg.nu1, nu2 = h->cfg.nu2;
+    for (int l = h->top; l >= 1; --l) {
+        for (int j = 0; j < nu1; ++j) {
+            ops.push_back(make_int4(kOpSweep, l, 2 * j, j > 0 ? 2 : 0));
+            ops.push_back(make_int4(kOpLowrank, l, 2 * j, j == nu1 - 1 ? 4 : 0));
+        }
+        if (nu1 == 0) ops.push_back(make_int4(kOpLowrank, l, 0, 2 | 4));
+        ops.push_back(make_int4(kOpRestrict, l, 0, 0));
+    }
+    ops.push_back(make_int4(kOpCoarsest, 0, 0, 0));
+    for (int l = 1; l <= h->top; ++l) {
+        ops.push_back(make_int4(kOpProlong, l, 1, (l == h->top && h->plan.shared_z && nu2 > 0) ? 2 : 0));
+        for (int j = 0; j < nu2; ++j) {
+            ops.push_back(make_int4(kOpSweep, l, 2 * j + 1, 1 | (j > 0 ? 2 : 0)));
+            ops.push_back(make_int4(kOpLowrank, l, 2 * j + 1, 1));
+        }
+    }
+}
+
 template <typename T>
 mgmc_status build_device_levels(mgmc_ctx* h, const HostProblem& hp)
 {
@@ -238,16 +267,16 @@ mgmc_status build_device_levels(mgmc_ctx* h, const HostProblem& hp)
                 for (int t = 1; t < D.ncoef; ++t) coef[(size_t)t * D.alloc + e] = (T)a[hp.C + t];
             }
             D.coef = upload(h, coef, st);
-            if (R == 2 && sizeof(T) == 8) {
-                std::vector<double> aux((size_t)D.alloc * 2, 0.0);
-                for (long long s2 = 0; s2 < HL.N; ++s2) {
-                    const long long e = off(s2);
-                    const double aii = HL.st[(size_t)s2 * hp.NS + hp.C];
-                    aux[(size_t)e] = 1.0 / aii;
-                    aux[(size_t)D.alloc + (size_t)e] = std::sqrt(aii);
-                }
-                D.inv_sqrt25 = upload(h, aux, st);
+        }
+        if (sizeof(T) == 8 && (R == 2 || l <= h->top)) {
+            std::vector<T> aux((size_t)D.alloc * 2, T(0));
+            for (long long s2 = 0; s2 < HL.N; ++s2) {
+                const long long e = off(s2);
+                const double aii = HL.st[(size_t)s2 * hp.NS + hp.C];
+                aux[(size_t)e] = (T)(1.0 / aii);
+                aux[(size_t)D.alloc + (size_t)e] = (T)std::sqrt(aii);
             }
+            D.isq = upload(h, aux, st);
         }
         if (hp.m > 0) {
             // rows of B grouped by grid row, sorted by x index
@@ -303,6 +332,11 @@ mgmc_status build_device_levels(mgmc_ctx* h, const HostProblem& hp)
         HostLevel& HL = const_cast<HostLevel&>(hp.lev[l]);
         for (int dir = 0; dir < 2; ++dir) {
             std::vector<T> gt(HL.gval[dir].begin(), HL.gval[dir].end());
+            if (l <= h->top) {   // read by the coarse kernel with one thread per row: columns contiguous
+                const size_t rows = HL.gsite[dir].size();
+                for (size_t r = 0; r < rows; ++r)
+                    for (int k = 0; k < hp.m; ++k) gt[(size_t)k * rows + r] = (T)HL.gval[dir][r * hp.m + k];
+            }
             D.gT[dir] = upload(h, gt, st);
         }
         fused_extras(HL, hp, l);
@@ -331,15 +365,6 @@ mgmc_status build_device_levels(mgmc_ctx* h, const HostProblem& hp)
             D.g_ss[dir] = upload(h, gss, st);
         }
         if (st != MGMC_OK) return fail(st, "device upload failed");
-    }
-    {
-        std::vector<int> nl;
-        for (int l = 0; l < hp.n_levels; ++l) nl.push_back(hp.lev[l].n);
-        h->coarse_smem =
-            (size_t)coarse_smem_elems(d, nl.data(), h->top, h->top == hp.n_levels - 1 && hp.disc == 0) * sizeof(T);
-        cudaError_t e = coarse_prepare<T>(d, h->coarse_smem);
-        if (e != cudaSuccess)
-            return fail(MGMC_ERR_CUDA, std::string("coarse kernel set-up: ") + cudaGetErrorString(e));
     }
     // general path: residual field of every smoothed grid, low-rank scratch
     if (!h->fused) {
@@ -405,7 +430,51 @@ mgmc_status build_device_levels(mgmc_ctx* h, const HostProblem& hp)
     h->levels_dev = h->buf.get(dbytes);
     if (!h->levels_dev) return fail(MGMC_ERR_OOM, "allocator returned NULL");
     CUDA_TRY(cudaMemcpyAsync(h->levels_dev, levels.data(), dbytes, cudaMemcpyHostToDevice, h->buf.stream));
+    if (!h->recursive && !h->cfg.gibbs) {
+        cudaError_t e = coarse_prepare<T>(d, kCoarseSmemLimit);
+        if (e != cudaSuccess)
+            return fail(MGMC_ERR_CUDA, std::string("coarse kernel set-up: ") + cudaGetErrorString(e));
+        std::vector<int4> ops;
+        coarse_phases(h, ops);
+        h->coarse_ops = upload(h, ops, st);
+        h->coarse_nops = (int)ops.size();
+        if (!hp.gain0.empty()) h->gain = upload(h, hp.gain0, st);
+        if (!hp.e0.empty()) h->e0 = upload(h, hp.e0, st);
+        if (st != MGMC_OK) return fail(st, "device upload failed");
+    }
     return MGMC_OK;
+}
+
+// the coarse kernel's job of one chain (device pointers of its handle)
+template <typename T>
+CoarseJob<T> coarse_job(const mgmc_ctx* c)
+{
+    CoarseJob<T> J{};
+    J.levels = (const DevLevel<T>*)c->levels_dev;
+    J.P = c->P_dev;
+    J.chol = c->chol;
+    J.gain = c->gain;
+    J.e0 = c->e0;
+    J.ops = c->coarse_ops;
+    J.image = c->coarse_image;
+    J.plan = c->plan;
+    J.n_ops = c->coarse_nops;
+    J.top = c->top;
+    J.is_finest = c->top == c->L - 1 ? 1 : 0;
+    J.n0 = c->n0;
+    return J;
+}
+
+
+// Compute threads of the coarse kernel: a colour of a 31^2 grid has 256 sites, of a 63^2 grid 1024
+int coarse_cta(const mgmc_ctx* h)
+{
+    if (h->coarse_threads > 0) return h->coarse_threads;
+    int nmax = 0;
+    const std::vector<const mgmc_ctx*> chains =
+        h->is_batch() ? std::vector<const mgmc_ctx*>(h->sub.begin(), h->sub.end()) : std::vector<const mgmc_ctx*>{h};
+    for (const mgmc_ctx* c : chains) nmax = std::max(nmax, c->fp32() ? c->lf[c->top].n : c->ld[c->top].n);
+    return nmax > 31 ? 512 : 256;
 }
 
 // The 2D nu1 = nu2 = 1 cycle of one chain or of a batch: every phase is one
@@ -431,13 +500,7 @@ void enqueue_cycle_batch(mgmc_ctx* h, cudaStream_t s, int& launches)
         launch_lowrank_batch<T>((const LowrankJob<T>*)h->jobs_lrd[d], h->njob_lrd[d], h->per_lrd[d], h->nblk_lrd[d],
                                 true, s, launches);
     }
-    // one CTA per chain: 1024 threads while the chains leave SMs free (latency-bound
-    // grids), 256 once several chains share an SM
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-    const int coarse_threads =
-        h->coarse_threads > 0 ? h->coarse_threads : ((!h->is_batch() || nc <= 2 * sms) ? 1024 : 256);
-    launch_coarse_batch<T>((const CoarseJob<T>*)h->jobs_coarse, nc, coarse_threads, h->batch_coarse_smem, s, launches);
+    launch_coarse<T>((const CoarseJob<T>*)h->jobs_coarse, nc, 2, coarse_cta(h), h->batch_coarse_smem, s, launches);
     for (int d = h->n_depth - 1; d >= 0; --d) {
         if (prof && d == 0) cudaEventRecordWithFlags(h->ev[2], s, cudaEventRecordExternal);
         if (d == 0 && h->stream_fine)
@@ -595,8 +658,8 @@ void enqueue_cycle(mgmc_ctx* h, cudaStream_t s, int& launches)
         if (h->cfg.nu1 == 0) launch_lowrank<T>(D, P, -1, 0u, true, s, launches);
         launch_restrict<T>(D, lv[l - 1], s, launches);
     }
-    launch_coarse<T>((const DevLevel<T>*)h->levels_dev, h->cfg.dim, h->top, h->top == Lf, P, h->chol, h->n0,
-                     h->cfg.nu1, h->cfg.nu2, h->coarse_smem, s, launches);
+    launch_coarse<T>((const CoarseJob<T>*)h->jobs_coarse, 1, h->cfg.dim, coarse_cta(h), h->batch_coarse_smem, s,
+                     launches);
     for (int l = h->top + 1; l <= Lf; ++l) {
         const DevLevel<T>& D = lv[l];
         launch_prolong<T>(lv[l - 1], D, s, launches);
@@ -806,7 +869,7 @@ mgmc_status mgmc_create(const mgmc_config* cfg_in, const mgmc_allocator* alloc, 
     HostProblem hp;
     int code = MGMC_OK;
     std::string err = build_hierarchy(hp, cfg.dim, cfg.n, cfg.n_levels, cfg.scale_hd, cfg.disc, kappa2, kappa2_const, m,
-                                      obs_site, obs_w, nnz_per_obs, Gamma, y, &code);
+                                      obs_site, obs_w, nnz_per_obs, Gamma, y, kCoarseGainMax, &code);
     if (!err.empty()) return fail((mgmc_status)code, err);
 
     mgmc_ctx* h = new mgmc_ctx();
@@ -819,18 +882,26 @@ mgmc_status mgmc_create(const mgmc_config* cfg_in, const mgmc_allocator* alloc, 
         h->buf.alloc = *alloc;
         h->buf.use_cuda_malloc = false;
     }
-    // grids inside the single-CTA coarse kernel: n <= coarse_max_n, and the state and
-    // right-hand side of all of them must fit in shared memory
+    // grids inside the single-CTA coarse kernel: n <= coarse_max_n, as many as its
+    // shared-memory plan holds
     int cmax = cfg.coarse_max_n > 0 ? cfg.coarse_max_n : (cfg.dim == 2 ? 63 : 15);
     h->top = 0;
     {
         const size_t esz = cfg.precision == MGMC_FP32 ? 4 : 8;
-        const size_t budget = 200 * 1024;
-        std::vector<int> nl;
-        for (int l = 0; l < h->L; ++l) nl.push_back(hp.lev[l].n);
+        std::vector<int> nl, nnz, grows;
+        for (int l = 0; l < h->L; ++l) {
+            nl.push_back(hp.lev[l].n);
+            nnz.push_back((int)hp.lev[l].bsite.size());
+            grows.push_back((int)(hp.lev[l].gsite[0].size() + hp.lev[l].gsite[1].size()));
+        }
         for (int l = 0; l < h->L && l < kCoarseMaxLevels; ++l) {
-            size_t bytes = (size_t)coarse_smem_elems(cfg.dim, nl.data(), l, l == h->L - 1 && cfg.disc == 0) * esz;
-            if (hp.lev[l].n <= cmax && bytes + 16384 <= budget) h->top = l;
+            CoarsePlan p;
+            if (l > 0 && hp.lev[l].n > cmax) break;
+            if (!coarse_plan(cfg.dim, nl.data(), l, l == h->L - 1 && cfg.disc == 0, m, nnz.data(), grows.data(), esz,
+                             kCoarseSmemLimit, &p))
+                break;
+            h->top = l;
+            h->plan = p;
         }
     }
     // the Gibbs sampler sweeps the finest grid with the unfused kernels, outside the coarse
@@ -885,6 +956,22 @@ mgmc_status mgmc_create(const mgmc_config* cfg_in, const mgmc_allocator* alloc, 
     if (!h->P_dev) return cleanup(fail(MGMC_ERR_OOM, "allocator returned NULL"));
     if (cudaMemcpyAsync(h->P_dev, &h->P, sizeof(DevProblem), cudaMemcpyHostToDevice, h->buf.stream) != cudaSuccess)
         return cleanup(fail(MGMC_ERR_CUDA, "upload failed"));
+    if (!h->recursive && !cfg.gibbs) {
+        h->coarse_image = (unsigned char*)h->buf.get((size_t)h->plan.img_bytes);
+        if (!h->coarse_image) return cleanup(fail(MGMC_ERR_OOM, "allocator returned NULL"));
+        cudaError_t e;
+        if (h->fp32()) {
+            const CoarseJob<float>* j = upload(h, std::vector<CoarseJob<float>>{coarse_job<float>(h)}, st);
+            e = st == MGMC_OK ? coarse_image<float>(j, h->coarse_image, cfg.dim, h->buf.stream) : cudaErrorUnknown;
+            h->jobs_coarse = (void*)j;
+        } else {
+            const CoarseJob<double>* j = upload(h, std::vector<CoarseJob<double>>{coarse_job<double>(h)}, st);
+            e = st == MGMC_OK ? coarse_image<double>(j, h->coarse_image, cfg.dim, h->buf.stream) : cudaErrorUnknown;
+            h->jobs_coarse = (void*)j;
+        }
+        h->batch_coarse_smem = (size_t)h->plan.smem_bytes;
+        if (e != cudaSuccess) return cleanup(fail(MGMC_ERR_CUDA, "coarse-grid image set-up failed"));
+    }
     // QoI (finest-level padded offsets)
     h->n_qoi = n_qoi;
     {
@@ -1356,13 +1443,13 @@ mgmc_status build_batch_tables(mgmc_ctx* h)
     std::vector<CycleState*> csl;
     size_t smem = 0;
     for (mgmc_ctx* c : chains) {
-        cj.push_back({(const DevLevel<T>*)c->levels_dev, c->top, c->top == c->L - 1 ? 1 : 0, c->P_dev, c->chol, c->n0});
+        cj.push_back(coarse_job<T>(c));
         const DevLevel<T>& Fh = levels_of<T>(c)[c->L - 1];
         qj.push_back({Fh.x, c->n_qoi, c->q_site, c->q_w, c->cs});
         pj.push_back({Fh.x, Fh.n, Fh.pitch, Fh.base});
         h->pack_max_n = std::max(h->pack_max_n, Fh.n);
         csl.push_back(c->cs);
-        smem = std::max(smem, c->coarse_smem);
+        smem = std::max(smem, (size_t)c->plan.smem_bytes);
     }
     h->jobs_coarse = upload(h, cj, st);
     h->jobs_qoi = upload(h, qj, st);
@@ -1370,8 +1457,7 @@ mgmc_status build_batch_tables(mgmc_ctx* h)
     h->cs_list = upload(h, csl, st);
     h->batch_coarse_smem = smem;
     if (st != MGMC_OK) return fail(st, "batch table upload failed");
-    cudaError_t e = coarse_prepare_batch<T>(smem);
-    if (e == cudaSuccess) e = tile_prepare_batch<T>();
+    cudaError_t e = tile_prepare_batch<T>();
     if (e != cudaSuccess) return fail(MGMC_ERR_CUDA, std::string("batch kernel set-up: ") + cudaGetErrorString(e));
     apply_band_min(h);
     (void)nc;

@@ -63,9 +63,10 @@ struct DevLevel {
     // the squared shifted Laplacian: offsets o = (dx+2) + 5 (dy+2), centre 12, slot t >= 1
     // = a(i, i + o_{12+t}); two halo rows and columns around the interior)
     int rad;
-    // FP64 25-point grids: 1 / a_ii at [e] and sqrt(a_ii) at [alloc + e] (correctly rounded on
-    // the host), so that a site update needs neither a division nor a square root
-    const double* inv_sqrt25;
+    // FP64 25-point grids and the grids inside the coarse kernel: 1 / a_ii at [e] and
+    // sqrt(a_ii) at [alloc + e] (rounded once from FP64 on the host), so that a site update
+    // needs neither a division nor a square root
+    const T* isq;
     // B_l rows grouped by grid row (finest level; used by the residual norm)
     const int* brow_ptr;    // [n^(dim-1) + 1]
     const int* bent_i;      // x index of the entry
@@ -76,7 +77,7 @@ struct DevLevel {
     const long long* bcol_site;   // padded element offset
     const double* bcol_w;
     const int* bcol_ss;           // grids inside the coarse kernel: shared-memory index of the site
-    const int* bcol_dense;        // coarsest grid: dense site index
+    const int* bcol_dense;        // coarsest grid: dense site index (k_coarsest_slot)
     const int* g_ss[2];           // grids inside the coarse kernel: shared-memory index of G's sites
     // G_l on its support, per direction (0 forward, 1 backward)
     int g_rows[2];
@@ -92,7 +93,8 @@ struct DevLevel {
     const int* tile_loc;          // local site of the entry, lx | ly << 16, relative to the tile origin
     const int* tile_ent;          // index t of the entry in the column lists bcol_*
     double* zparts;               // [nnz] w_t * theta(site_t), written by the tile kernels
-    const T* gT[2];               // G_l(dir) in the path precision, [rows * m]
+    const T* gT[2];               // G_l(dir) in the path precision, [rows * m] (grids inside the
+                                  // coarse kernel: k-major, [m * rows])
     int h_rows;                   // H = P^T A_l G_l(forward) on the coarse grid
     const long long* h_site;      // coarse padded offsets
     const T* hT;                  // [rows * m]

@@ -17,8 +17,8 @@ void launch_restrict(const DevLevel<T>& F, const DevLevel<T>& C, cudaStream_t st
 template <typename T>
 void launch_coarsest_slot(const DevLevel<T>& L, const DevProblem& P, const double* chol, int n0, unsigned slot,
                           cudaStream_t st, int& launches);
-// the small grids of the general path (2D) in one CTA: a list of phases {code, level, slot,
-// flags} the host builds from the cycle's recursion (kernels.cu, k_cycle_small)
+// phases {code, grid, slot, flags} of the kernels that run several grids in one CTA, listed by
+// the host from the cycle's recursion (coarse.cu; kernels.cu: k_cycle_small)
 enum { kOpSweep = 0, kOpLowrank = 1, kOpRestrict = 2, kOpZero = 3, kOpCoarsest = 4, kOpProlong = 5 };
 constexpr int kSmallCycleThreads = 512;
 constexpr int kSmallMaxLevels = 16;   // grids 0..top held by the kernel (top < 16)
@@ -29,14 +29,45 @@ void launch_cycle_small(const DevLevel<T>* levels_dev, int top, const DevProblem
                         const int4* ops, int n_ops, double* zb, cudaStream_t st, int& launches);
 template <typename T>
 void launch_prolong(const DevLevel<T>& C, const DevLevel<T>& F, cudaStream_t st, int& launches);
-// one chain of a batched coarse-grid launch
+// shared-memory plan of the coarse kernel (coarse.cu), offsets in elements of the path precision
+constexpr int kCoarseMaxLevels = 8;   // grids it holds at most (their descriptors are staged)
+constexpr int kCoarseGainMax = 64;    // coarsest unknowns up to which the gain matrix is used
+struct CoarsePlan {
+    int x_off[kCoarseMaxLevels];   // grid l's blocks: state, right-hand side, 1/a_ii, coefficients
+    int sa_off[kCoarseMaxLevels];  // its sqrt(a_ii) block (-1: none)
+    int zf[kCoarseMaxLevels];      // normals of the forward / backward sweep
+    int zb[kCoarseMaxLevels];
+    int g_off[kCoarseMaxLevels];   // byte offsets of the staged rows of G and their sites (-1: in global memory)
+    int gs_off[kCoarseMaxLevels];
+    int ent0[kCoarseMaxLevels];    // first staged observation entry
+    int nent;                      // staged observation entries
+    int stage_ent;                 // 0: the entries are read from global memory
+    int ent_off;                   // byte offset of the entries
+    int shared_z;                  // 1: the top grid's two sweeps share zf[top] = zb[top], no sqrt(a_ii) block
+    int img_bytes;                 // the static image is the first img_bytes
+    int lr_off;                    // byte offset of the low-rank area
+    int smem_bytes;
+    int pad;
+};
+// g_rows_of_level: rows of G of both directions together
+bool coarse_plan(int dim, const int* n_of_level, int top, bool top_is_fd_finest, int m, const int* nnz_of_level,
+                 const int* g_rows_of_level, size_t elem, size_t limit, CoarsePlan* out);
+// dynamic shared memory the coarse kernel may use: 227 KB less its static part
+constexpr size_t kCoarseSmemLimit = 232448 - 6144;
+// one chain of a coarse-grid launch
 template <typename T>
 struct CoarseJob {
     const DevLevel<T>* levels;   // device descriptors of grids 0 .. L-1
+    const DevProblem* P;
+    const double* chol;          // Cholesky factor of the coarsest operator (n0 > kCoarseGainMax)
+    const double* gain;          // [n0][2 n0 + m] rows [A~_0^-1 | A~_0^-1 B_0 Gamma^-1 | L_0^-T], or NULL
+    const double* e0;            // [m][n0] columns of B_0 Gamma^-1 (n0 > kCoarseGainMax)
+    const int4* ops;             // phases {code, grid, slot, flags}
+    const unsigned char* image;  // static part of the shared memory (coarse_image)
+    CoarsePlan plan;
+    int n_ops;
     int top;
     int is_finest;
-    const DevProblem* P;
-    const double* chol;
     int n0;
 };
 // one chain of a batched QoI launch
@@ -49,29 +80,18 @@ struct QoiJob {
     CycleState* cs;
 };
 template <typename T>
-cudaError_t coarse_prepare_batch(size_t smem_bytes);
-template <typename T>
-void launch_coarse_batch(const CoarseJob<T>* jobs, int n, int threads, size_t smem_bytes, cudaStream_t st,
-                         int& launches);
-template <typename T>
 void launch_qoi_batch(const QoiJob<T>* jobs, int n, cudaStream_t st, int& launches);
 void launch_set_cycle_batch(CycleState* const* cs, int n, unsigned long long seed, unsigned long long cycle, int noise,
                             double* qoi, long long n_steps, cudaStream_t st);
 
-// the V-cycle of grids 0..top in one CTA with shared-memory state (coarse.cu)
-// grids a coarse kernel holds at most (their descriptors are staged in shared memory)
-constexpr int kCoarseMaxLevels = 8;
-// coarsest grids with at most this many unknowns are solved by one warp from a factor
-// staged in shared memory
-constexpr int kCoarsestWarp = 32;
-// elements of the coarse kernel's dynamic shared memory; top_is_fd_finest: the top
-// grid is the finest grid in its 5/7-point finite-difference form (one operator field)
-long long coarse_smem_elems(int dim, const int* n_of_level, int top, bool top_is_fd_finest);
+// the V-cycle of grids 0..top of n chains, one CTA each, with shared-memory state (coarse.cu)
 template <typename T>
 cudaError_t coarse_prepare(int dim, size_t smem_bytes);
 template <typename T>
-void launch_coarse(const DevLevel<T>* levels_dev, int dim, int top, bool is_finest, const DevProblem& P,
-                   const double* chol, int n0, int nu1, int nu2, size_t smem_bytes, cudaStream_t st, int& launches);
+cudaError_t coarse_image(const CoarseJob<T>* job, unsigned char* image, int dim, cudaStream_t st);
+template <typename T>
+void launch_coarse(const CoarseJob<T>* jobs, int n, int dim, int threads, size_t smem_bytes, cudaStream_t st,
+                   int& launches);
 template <typename T>
 void launch_qoi(const DevLevel<T>& L, int n_qoi, const long long* q_site, const double* q_w, const DevProblem& P,
                 cudaStream_t st, int& launches);

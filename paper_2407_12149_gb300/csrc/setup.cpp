@@ -462,7 +462,7 @@ std::string fine_operator(HostProblem& hp, int dim, int n, int scale_hd, int dis
 
 std::string build_hierarchy(HostProblem& hp, int dim, int n, int n_levels, int scale_hd, int disc, const double* kappa2,
                             double kappa2_const, int m, const int32_t* obs_site, const double* obs_w,
-                            int nnz_per_obs, const double* Gamma, const double* y, int* code)
+                            int nnz_per_obs, const double* Gamma, const double* y, int gain_max, int* code)
 {
     *code = MGMC_ERR_ARG;
     hp.dim = dim;
@@ -611,6 +611,37 @@ std::string build_hierarchy(HostProblem& hp, int dim, int n, int n_levels, int s
         if (!cholesky_lower(n0, A0, hp.chol0)) {
             *code = MGMC_ERR_NOT_SPD;
             return "coarsest posterior operator is not positive definite";
+        }
+        // E = B_0 Gamma^-1 by columns
+        std::vector<double> E((size_t)m * n0, 0.0);
+        for (int k = 0; k < m; ++k)
+            for (int t = L0.bptr[k]; t < L0.bptr[k + 1]; ++t)
+                for (int c = 0; c < m; ++c)
+                    E[(size_t)c * n0 + (size_t)L0.bsite[t]] += L0.bw[t] * hp.Gamma_inv[(size_t)k * m + c];
+        if (n0 <= gain_max) {
+            const std::vector<double>& Lc = hp.chol0;
+            const int len = 2 * n0 + m;
+            hp.gain0.assign((size_t)n0 * len, 0.0);
+            std::vector<double> r((size_t)n0);
+            auto back = [&]() {   // r <- L^-T r
+                for (int i = n0 - 1; i >= 0; --i) {
+                    for (int t = i + 1; t < n0; ++t) r[i] -= Lc[(size_t)t * n0 + i] * r[t];
+                    r[i] /= Lc[(size_t)i * n0 + i];
+                }
+            };
+            for (int c = 0; c < len; ++c) {
+                for (int i = 0; i < n0; ++i)
+                    r[i] = c < n0 ? (i == c ? 1.0 : 0.0) : c < n0 + m ? E[(size_t)(c - n0) * n0 + i] : (i == c - n0 - m ? 1.0 : 0.0);
+                if (c < n0 + m)
+                    for (int i = 0; i < n0; ++i) {   // r <- L^-1 r
+                        for (int t = 0; t < i; ++t) r[i] -= Lc[(size_t)i * n0 + t] * r[t];
+                        r[i] /= Lc[(size_t)i * n0 + i];
+                    }
+                back();
+                for (int i = 0; i < n0; ++i) hp.gain0[(size_t)i * len + c] = r[i];
+            }
+        } else {
+            hp.e0 = E;
         }
     }
     *code = MGMC_OK;

@@ -39,6 +39,9 @@ struct HostProblem {
     bool gamma_diag = true;
     int n0 = 0;
     std::vector<double> chol0;       // Cholesky factor of A~_0 (lower, row-major)
+    // coarsest sample as one product (n0 <= gain_max): rows [A~_0^-1 | A~_0^-1 B_0 Gamma^-1 | L_0^-T];
+    // larger coarsest grids: the columns of B_0 Gamma^-1, [m][n0]
+    std::vector<double> gain0, e0;
     double f_norm = 0.0;             // ||f_L||_2
 };
 
@@ -46,7 +49,7 @@ struct HostProblem {
 // the mgmc_status to return.
 std::string build_hierarchy(HostProblem& hp, int dim, int n, int n_levels, int scale_hd, int disc, const double* kappa2,
                             double kappa2_const, int m, const int32_t* obs_site, const double* obs_w,
-                            int nnz_per_obs, const double* Gamma, const double* y, int* code);
+                            int nnz_per_obs, const double* Gamma, const double* y, int gain_max, int* code);
 
 // The finest grid's operator alone: hp.dim, NS, C, n_levels and lev[] must be set
 // (build_hierarchy does this); fills lev[n_levels - 1].st.

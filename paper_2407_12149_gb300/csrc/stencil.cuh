@@ -60,13 +60,13 @@ __device__ __forceinline__ double coef25_at(const DevLevel<double>& L, long long
 __device__ __forceinline__ double update25(const DevLevel<double>& L, long long e, double z)
 {
     double acc = L.f ? L.f[e] : 0.0;
-    acc += L.inv_sqrt25[L.alloc + e] * z;
+    acc += L.isq[L.alloc + e] * z;
 #pragma unroll
     for (int o = 0; o < 25; ++o) {
         if (o == 12) continue;
         acc -= coef25_at(L, e, o) * L.x[e + off25(o, L.pitch)];
     }
-    return acc * L.inv_sqrt25[e];
+    return acc * L.isq[e];
 }
 
 // ---------------------------------------------------------------------------
