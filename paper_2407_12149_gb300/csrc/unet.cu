@@ -11,10 +11,14 @@
 // ReLU, a 1x1 output convolution.  Loss: mean squared error on the n x n
 // interior; optimiser: Adam (Kingma & Ba 2015).
 //
-// Every 3x3 convolution is an im2col + tcgen05 GEMM (tc_gemm.cu):
+// The 3x3 convolutions run as implicit GEMMs on the tensor cores (tc_conv.cu); the first
+// layer (3 input channels) and narrow ones (c0 = 8) as im2col + tcgen05 GEMM (tc_gemm.cu),
+// with the same order of sums:
 //   forward      Y[P][co]      = relu(Xcol[P][9ci] W[co][9ci]^T + b)
 //   data grad    dXcol[P][9ci] = dZ[P][co] Wt[9ci][co]^T, then col2im
 //   weight grad  dWt[9ci][co]  = XcolT[9ci][P] dZT[co][P]^T (split over P, fixed-order sum)
+// Everything else is bound by memory: each kernel moves 8 channels (16 or 32 bytes) per
+// thread, since every channel count is a multiple of 8.
 // All reductions (bias gradients, loss) run in a fixed order: results are
 // deterministic.  This file also holds the exported GEMM entry point.
 #include <cuda_bf16.h>
@@ -29,6 +33,7 @@
 
 #include "../../include/mgmc.h"
 #include "common.cuh"
+#include "tc_conv.cuh"
 #include "tc_gemm.cuh"
 
 namespace mgmc {
@@ -37,7 +42,7 @@ namespace {
 using bf16 = __nv_bfloat16;
 
 constexpr int kLayers = 14;
-constexpr int kRedBlocks = 256;   // partial-sum blocks of the column reductions
+constexpr int kRedBlocks = 608;   // partial-sum blocks of the column reductions (4 per SM)
 
 struct LayerDef {
     int level, cin, cout;
@@ -90,6 +95,29 @@ __global__ void k_im2col(const bf16* __restrict__ x, int B, int H, int cin, bf16
     }
 }
 
+// k_im2col of 3 channels (ldo = 32): one pixel's row of 27 values and 5 zeros per thread
+__global__ void k_im2col3(const bf16* __restrict__ x, int B, int H, bf16* __restrict__ out)
+{
+    const long long P = (long long)B * H * H;
+    for (long long p = gtid(); p < P; p += gstride()) {
+        const int j = (int)(p % H), i = (int)((p / H) % H);
+        const bf16* img = x + p * 3;
+        __align__(16) bf16 v[32];
+#pragma unroll
+        for (int t = 0; t < 9; ++t) {
+            const int dy = t / 3 - 1, dx = t % 3 - 1;
+            const bool in = (unsigned)(i + dy) < (unsigned)H && (unsigned)(j + dx) < (unsigned)H;
+            const bf16* s = img + ((long long)dy * H + dx) * 3;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) v[3 * t + c] = in ? s[c] : __float2bfloat16(0.f);
+        }
+#pragma unroll
+        for (int c = 27; c < 32; ++c) v[c] = __float2bfloat16(0.f);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) reinterpret_cast<uint4*>(out + p * 32)[q] = reinterpret_cast<const uint4*>(v)[q];
+    }
+}
+
 // out[c][r] = in[r][c] for r < R, c < C (32 x 32 tiles through shared memory)
 __global__ void k_transpose(const bf16* __restrict__ in, long long R, int C, long long ldi, bf16* __restrict__ out,
                             long long ldo)
@@ -110,38 +138,92 @@ __global__ void k_transpose(const bf16* __restrict__ in, long long R, int C, lon
     }
 }
 
-// dz = bf16(dy * (y > 0)); part[block][c] = sum of dz over the block's rows (C divides 256)
-__global__ void k_relu_bwd(const float* __restrict__ dy, const bf16* __restrict__ y, long long P, int C,
-                           bf16* __restrict__ dz, float* __restrict__ part)
+// 8 BF16 values
+struct Bf8 {
+    __nv_bfloat162 h[4];
+};
+__device__ __forceinline__ Bf8 ld8(const bf16* p)
 {
-    __shared__ float red[256];
-    const int c = threadIdx.x % C, r0 = threadIdx.x / C, rs = blockDim.x / C;
-    const long long rows = (P + gridDim.x - 1) / gridDim.x;
-    const long long rb = blockIdx.x * rows, re = min(P, rb + rows);
-    float acc = 0.f;
-    for (long long r = rb + r0; r < re; r += rs) {
-        const long long e = r * C + c;
-        const bf16 v = __float2bfloat16(__bfloat162float(y[e]) > 0.f ? dy[e] : 0.f);
-        dz[e] = v;
-        acc += __bfloat162float(v);
+    const uint4 v = *reinterpret_cast<const uint4*>(p);
+    return *reinterpret_cast<const Bf8*>(&v);
+}
+__device__ __forceinline__ void st8(bf16* p, const Bf8& v) { *reinterpret_cast<uint4*>(p) = *reinterpret_cast<const uint4*>(&v); }
+__device__ __forceinline__ void unpack8(const Bf8& v, float* f)
+{
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float2 t = __bfloat1622float2(v.h[q]);
+        f[2 * q] = t.x;
+        f[2 * q + 1] = t.y;
     }
-    red[threadIdx.x] = acc;
+}
+__device__ __forceinline__ Bf8 pack8(const float* f)
+{
+    Bf8 v;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v.h[q] = __floats2bfloat162_rn(f[2 * q], f[2 * q + 1]);
+    return v;
+}
+__device__ __forceinline__ void ldf8(const float* p, float* f)
+{
+    *reinterpret_cast<float4*>(f) = *reinterpret_cast<const float4*>(p);
+    *reinterpret_cast<float4*>(f + 4) = *reinterpret_cast<const float4*>(p + 4);
+}
+__device__ __forceinline__ void stf8(float* p, const float* f)
+{
+    *reinterpret_cast<float4*>(p) = *reinterpret_cast<const float4*>(f);
+    *reinterpret_cast<float4*>(p + 4) = *reinterpret_cast<const float4*>(f + 4);
+}
+
+// sums over a block's rows of 8 channels per thread: thread (r0, c8) holds acc; out[8 c8 ..] for the rows' total
+__device__ __forceinline__ void block_colsum(float (*red)[256], const float* acc, int groups, float* out)
+{
+#pragma unroll
+    for (int q = 0; q < 8; ++q) red[q][threadIdx.x] = acc[q];
     __syncthreads();
-    if (threadIdx.x < C) {
+    const int C = 8 * groups;
+    for (int c = threadIdx.x; c < C; c += blockDim.x) {
         float s = 0.f;
-        for (int k = 0; k < rs; ++k) s += red[k * C + threadIdx.x];
-        part[(long long)blockIdx.x * C + threadIdx.x] = s;
+        for (int k = c >> 3; k < (int)blockDim.x; k += groups) s += red[c & 7][k];
+        out[c] = s;
     }
 }
 
-// out[c] = sum over nb blocks of part[b][c] (fixed order)
+// dz = bf16(dy * (y > 0)); part[block][c] = sum of dz over the block's rows (C divides 2048)
+__global__ void k_relu_bwd(const float* __restrict__ dy, const bf16* __restrict__ y, long long P, int C,
+                           bf16* __restrict__ dz, float* __restrict__ part)
+{
+    __shared__ float red[8][256];
+    const int groups = C / 8, c8 = threadIdx.x % groups, r0 = threadIdx.x / groups, rs = blockDim.x / groups;
+    const long long rows = (P + gridDim.x - 1) / gridDim.x;
+    const long long rb = blockIdx.x * rows, re = min(P, rb + rows);
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+    for (long long r = rb + r0; r < re; r += rs) {
+        const long long e = r * C + 8 * c8;
+        float d[8], f[8];
+        ldf8(dy + e, d);
+        unpack8(ld8(y + e), f);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) d[q] = f[q] > 0.f ? d[q] : 0.f;
+        const Bf8 v = pack8(d);
+        st8(dz + e, v);
+        unpack8(v, f);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc[q] += f[q];
+    }
+    block_colsum(red, acc, groups, part + (long long)blockIdx.x * C);
+}
+
+// out[c] = sum over nb blocks of part[b][c] (fixed order): one warp per column
 __global__ void k_colsum(const float* __restrict__ part, int nb, int C, float* __restrict__ out)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = (int)(gtid() >> 5), lane = threadIdx.x & 31;
     if (c >= C) return;
     float s = 0.f;
-    for (int b = 0; b < nb; ++b) s += part[(long long)b * C + c];
-    out[c] = s;
+    for (int b = lane; b < nb; b += 32) s += part[(long long)b * C + c];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) out[c] = s;
 }
 
 // dx[p][c] (+)= sum over taps of dcol[p'][tap cin + c], p' = (i - ky + 1, j - kx + 1)
@@ -168,30 +250,46 @@ __global__ void k_col2im(const float* __restrict__ dcol, int ldc, int B, int H, 
 // 2x2 average pool of x [B][2H][2H][C] into y [B][H][H][C]
 __global__ void k_pool_fwd(const bf16* __restrict__ x, int B, int H, int C, bf16* __restrict__ y)
 {
-    const long long n = (long long)B * H * H * C;
+    const int G = C / 8;
+    const long long n = (long long)B * H * H * G;
     const int W2 = 2 * H;
     for (long long it = gtid(); it < n; it += gstride()) {
-        const int c = (int)(it % C);
-        const long long q = it / C;
+        const int c = 8 * (int)(it % G);
+        const long long q = it / G;
         const int j = (int)(q % H), i = (int)((q / H) % H);
         const long long b = q / ((long long)H * H);
-        auto at = [&](int a, int bb) { return __bfloat162float(x[((b * W2 + 2 * i + a) * W2 + 2 * j + bb) * C + c]); };
-        y[it] = __float2bfloat16(0.25f * (at(0, 0) + at(1, 0) + at(0, 1) + at(1, 1)));
+        float f[4][8];
+#pragma unroll
+        for (int a = 0; a < 2; ++a)
+#pragma unroll
+            for (int bb = 0; bb < 2; ++bb)
+                unpack8(ld8(x + ((b * W2 + 2 * i + a) * W2 + 2 * j + bb) * C + c), f[2 * bb + a]);
+        float o[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) o[t] = 0.25f * (f[0][t] + f[1][t] + f[2][t] + f[3][t]);
+        st8(y + q * C + c, pack8(o));
     }
 }
 
 // dx [B][2H][2H][C] (+)= dy [B][H][H][C] / 4
 __global__ void k_pool_bwd(const float* __restrict__ dy, int B, int H, int C, float* __restrict__ dx, int accumulate)
 {
-    const int W2 = 2 * H;
-    const long long n = (long long)B * W2 * W2 * C;
+    const int W2 = 2 * H, G = C / 8;
+    const long long n = (long long)B * W2 * W2 * G;
     for (long long it = gtid(); it < n; it += gstride()) {
-        const int c = (int)(it % C);
-        const long long q = it / C;
+        const int c = 8 * (int)(it % G);
+        const long long q = it / G;
         const int j = (int)(q % W2), i = (int)((q / W2) % W2);
         const long long b = q / ((long long)W2 * W2);
-        const float v = 0.25f * dy[((b * H + i / 2) * H + j / 2) * C + c];
-        dx[it] = accumulate ? dx[it] + v : v;
+        float v[8], o[8];
+        ldf8(dy + ((b * H + i / 2) * H + j / 2) * C + c, v);
+        if (accumulate) ldf8(dx + q * C + c, o);
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            const float a = 0.25f * v[t];
+            o[t] = accumulate ? o[t] + a : a;
+        }
+        stf8(dx + q * C + c, o);
     }
 }
 
@@ -199,14 +297,14 @@ __global__ void k_pool_bwd(const float* __restrict__ dy, int B, int H, int C, fl
 __global__ void k_upcat(const bf16* __restrict__ low, int ca, const bf16* __restrict__ skip, int cb, int B, int H,
                         bf16* __restrict__ u)
 {
-    const int C = ca + cb, h = H / 2;
-    const long long n = (long long)B * H * H * C;
+    const int C = ca + cb, h = H / 2, G = C / 8;
+    const long long n = (long long)B * H * H * G;
     for (long long it = gtid(); it < n; it += gstride()) {
-        const int c = (int)(it % C);
-        const long long p = it / C;
+        const int c = 8 * (int)(it % G);
+        const long long p = it / G;
         const int j = (int)(p % H), i = (int)((p / H) % H);
         const long long b = p / ((long long)H * H);
-        u[it] = c < ca ? low[((b * h + i / 2) * h + j / 2) * ca + c] : skip[p * cb + (c - ca)];
+        st8(u + p * C + c, c < ca ? ld8(low + ((b * h + i / 2) * h + j / 2) * ca + c) : ld8(skip + p * cb + (c - ca)));
     }
 }
 
@@ -214,21 +312,29 @@ __global__ void k_upcat(const bf16* __restrict__ low, int ca, const bf16* __rest
 __global__ void k_upcat_bwd(const float* __restrict__ du, int ca, int cb, int B, int H, float* __restrict__ dlow,
                             float* __restrict__ dskip)
 {
-    const int C = ca + cb, h = H / 2;
-    const long long nl = (long long)B * h * h * ca, ns = (long long)B * H * H * cb;
+    const int C = ca + cb, h = H / 2, ga = ca / 8, gb = cb / 8;
+    const long long nl = (long long)B * h * h * ga, ns = (long long)B * H * H * gb;
     for (long long it = gtid(); it < nl + ns; it += gstride()) {
         if (it < nl) {
-            const int c = (int)(it % ca);
-            const long long q = it / ca;
+            const int c = 8 * (int)(it % ga);
+            const long long q = it / ga;
             const int j = (int)(q % h), i = (int)((q / h) % h);
             const long long b = q / ((long long)h * h);
-            auto at = [&](int a, int bb) { return du[((b * H + 2 * i + a) * H + 2 * j + bb) * C + c]; };
-            dlow[it] = at(0, 0) + at(1, 0) + at(0, 1) + at(1, 1);
+            float f[4][8], o[8];
+#pragma unroll
+            for (int a = 0; a < 2; ++a)
+#pragma unroll
+                for (int bb = 0; bb < 2; ++bb) ldf8(du + ((b * H + 2 * i + a) * H + 2 * j + bb) * C + c, f[2 * bb + a]);
+#pragma unroll
+            for (int t = 0; t < 8; ++t) o[t] = f[0][t] + f[1][t] + f[2][t] + f[3][t];
+            stf8(dlow + q * ca + c, o);
         } else {
             const long long e = it - nl;
-            const int c = (int)(e % cb);
-            const long long p = e / cb;
-            dskip[e] = du[p * C + ca + c];
+            const int c = 8 * (int)(e % gb);
+            const long long p = e / gb;
+            float f[8];
+            ldf8(du + p * C + ca + c, f);
+            stf8(dskip + p * cb + c, f);
         }
     }
 }
@@ -239,7 +345,12 @@ __global__ void k_out_fwd(const bf16* __restrict__ x, long long P, int C, const 
 {
     for (long long p = gtid(); p < P; p += gstride()) {
         float s = 0.f;
-        for (int c = 0; c < C; ++c) s += w[c] * __bfloat162float(x[p * C + c]);
+        for (int c = 0; c < C; c += 8) {
+            float f[8];
+            unpack8(ld8(x + p * C + c), f);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) s += w[c + q] * f[q];
+        }
         out[p] = s + b[0];
     }
 }
@@ -276,23 +387,59 @@ __global__ void k_loss(const float* __restrict__ out, const float* __restrict__ 
 __global__ void k_out_bwd(const float* __restrict__ dout, const bf16* __restrict__ x, long long P, int C,
                           const float* __restrict__ w, float* __restrict__ dx, float* __restrict__ part)
 {
+    __shared__ float red[8][256];
+    __shared__ float tot[256];
+    const int groups = C / 8, c8 = threadIdx.x % groups, r0 = threadIdx.x / groups, rs = blockDim.x / groups;
     const long long rows = (P + gridDim.x - 1) / gridDim.x;
     const long long rb = blockIdx.x * rows, re = min(P, rb + rows);
-    for (long long e = rb * C + threadIdx.x; e < re * C; e += blockDim.x) dx[e] = dout[e / C] * w[e % C];
-    for (int c = threadIdx.x; c <= C; c += blockDim.x) {
+    float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, wc[8], sum = 0.f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) wc[q] = w[8 * c8 + q];
+#pragma unroll 2
+    for (long long r = rb + r0; r < re; r += rs) {
+        const float d = dout[r];
+        float f[8], o[8];
+        unpack8(ld8(x + r * C + 8 * c8), f);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            o[q] = d * wc[q];
+            acc[q] += d * f[q];
+        }
+        stf8(dx + r * C + 8 * c8, o);
+        sum += d;
+    }
+    float* out = part + (long long)blockIdx.x * (C + 1);
+    tot[threadIdx.x] = c8 == 0 ? sum : 0.f;
+    block_colsum(red, acc, groups, out);   // its barrier also covers tot
+    if (threadIdx.x == 0) {
         float s = 0.f;
-        for (long long r = rb; r < re; ++r) s += c < C ? dout[r] * __bfloat162float(x[r * C + c]) : dout[r];
-        part[(long long)blockIdx.x * (C + 1) + c] = s;
+        for (int k = 0; k < (int)blockDim.x; k += groups) s += tot[k];
+        out[C] = s;
     }
 }
 
-// g[co K + k] = dwt[k][co]  (weight gradient in the [cout][3][3][cin] order)
-__global__ void k_wt_to_flat(const float* __restrict__ dwt, int K, int Co, float* __restrict__ g)
+// g[co K + k] = sum over `splits` partials of part[z][k][co], z ascending (weight gradient in the
+// [cout][3][3][cin] order): 32 x 32 tiles through shared memory
+__global__ void k_wt_to_flat(const float* __restrict__ part, int splits, int Kp, int K, int Co, float* __restrict__ g)
 {
-    const long long n = (long long)K * Co;
-    for (long long it = gtid(); it < n; it += gstride()) {
-        const int k = (int)(it % K), co = (int)(it / K);
-        g[it] = dwt[(long long)k * Co + co];
+    __shared__ float t[32][33];
+    const int k0 = blockIdx.x * 32, c0 = blockIdx.y * 32;
+    const long long count = (long long)Kp * Co;
+    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+        const int k = k0 + r, c = c0 + threadIdx.x;
+        float acc = 0.f;
+        if (k < K && c < Co) {
+            const float* p = part + (long long)k * Co + c;
+            acc = p[0];
+#pragma unroll 8
+            for (int z = 1; z < splits; ++z) acc += p[z * count];
+        }
+        t[r][threadIdx.x] = acc;
+    }
+    __syncthreads();
+    for (int r = threadIdx.y; r < 32; r += blockDim.y) {
+        const int c = c0 + r, k = k0 + threadIdx.x;
+        if (c < Co && k < K) g[(long long)c * K + k] = t[threadIdx.x][r];
     }
 }
 
@@ -484,6 +631,15 @@ mgmc_status refresh_bf16(UnetCtx* u)
     return MGMC_OK;
 }
 
+void im2col(UnetCtx* u, const bf16* x, int B, int Hs, int l)
+{
+    const long long P = (long long)B * Hs * Hs;
+    if (u->L[l].cin == 3)
+        k_im2col3<<<grid_for(P), 256, 0, u->stream>>>(x, B, Hs, u->col);
+    else
+        k_im2col<<<grid_for(P * 9), 256, 0, u->stream>>>(x, B, Hs, u->L[l].cin, u->col, u->Kp[l]);
+}
+
 // forward pass of B samples whose inputs are at `input` ([B][H][H][3] BF16)
 mgmc_status forward(UnetCtx* u, int B, const bf16* input)
 {
@@ -495,19 +651,25 @@ mgmc_status forward(UnetCtx* u, int B, const bf16* input)
         const LayerDef& D = u->L[l];
         const int s = D.level, Hs = u->Hs(s);
         const long long P = u->Ps(s, B);
-        if (l == 2) k_pool_fwd<<<grid_for(P * u->L[1].cout), 256, 0, st>>>(u->act[1], B, Hs, u->L[1].cout, u->p0);
-        if (l == 4) k_pool_fwd<<<grid_for(P * u->L[3].cout), 256, 0, st>>>(u->act[3], B, Hs, u->L[3].cout, u->p1);
-        if (l == 6) k_pool_fwd<<<grid_for(P * u->L[5].cout), 256, 0, st>>>(u->act[5], B, Hs, u->L[5].cout, u->p2);
+        if (l == 2) k_pool_fwd<<<grid_for(P * u->L[1].cout / 8), 256, 0, st>>>(u->act[1], B, Hs, u->L[1].cout, u->p0);
+        if (l == 4) k_pool_fwd<<<grid_for(P * u->L[3].cout / 8), 256, 0, st>>>(u->act[3], B, Hs, u->L[3].cout, u->p1);
+        if (l == 6) k_pool_fwd<<<grid_for(P * u->L[5].cout / 8), 256, 0, st>>>(u->act[5], B, Hs, u->L[5].cout, u->p2);
         if (l == 8)
-            k_upcat<<<grid_for(P * D.cin), 256, 0, st>>>(u->act[7], u->L[7].cout, u->act[5], u->L[5].cout, B, Hs,
+            k_upcat<<<grid_for(P * D.cin / 8), 256, 0, st>>>(u->act[7], u->L[7].cout, u->act[5], u->L[5].cout, B, Hs,
                                                        u->u2);
         if (l == 10)
-            k_upcat<<<grid_for(P * D.cin), 256, 0, st>>>(u->act[9], u->L[9].cout, u->act[3], u->L[3].cout, B, Hs,
+            k_upcat<<<grid_for(P * D.cin / 8), 256, 0, st>>>(u->act[9], u->L[9].cout, u->act[3], u->L[3].cout, B, Hs,
                                                        u->u1);
         if (l == 12)
-            k_upcat<<<grid_for(P * D.cin), 256, 0, st>>>(u->act[11], u->L[11].cout, u->act[1], u->L[1].cout, B, Hs,
+            k_upcat<<<grid_for(P * D.cin / 8), 256, 0, st>>>(u->act[11], u->L[11].cout, u->act[1], u->L[1].cout, B, Hs,
                                                        u->u0);
-        k_im2col<<<grid_for(P * 9), 256, 0, st>>>(u->layer_in(l), B, Hs, D.cin, u->col, u->Kp[l]);
+        if (tc_conv_ok(D.cin, D.cout)) {
+            if (tc_conv_fwd(u->layer_in(l), B, Hs, D.cin, u->Wb[l], D.cout, u->theta + u->boff[l], u->act[l], u->status,
+                            st) != cudaSuccess)
+                rc = unet_fail(MGMC_ERR_CUDA, "convolution launch failed");
+            continue;
+        }
+        im2col(u, u->layer_in(l), B, Hs, l);
         rc = gemm(u, u->col, u->Kp[l], u->Wb[l], u->Kp[l], u->act[l], P, D.cout, u->K[l],
                   kEpiBias | kEpiRelu | kEpiBF16, u->theta + u->boff[l], 1);
     }
@@ -528,21 +690,35 @@ mgmc_status conv_backward(UnetCtx* u, int l, int B, const bf16* input, float* dx
     const int s = D.level, Hs = u->Hs(s);
     const long long P = u->Ps(s, B);
     k_relu_bwd<<<kRedBlocks, 256, 0, st>>>(u->dact[l], u->act[l], P, D.cout, u->dz, u->part);
-    k_colsum<<<(D.cout + 255) / 256, 256, 0, st>>>(u->part, kRedBlocks, D.cout, u->grad + u->boff[l]);
+    k_colsum<<<(D.cout + 7) / 8, 256, 0, st>>>(u->part, kRedBlocks, D.cout, u->grad + u->boff[l]);
+    const long long tiles = (u->Kp[l] + 127) / 128;  // N = cout <= 256 is one tile
+    // the weight gradient's pixel ranges, for ~2 CTAs per SM
+    const int splits = (int)std::max(1LL, std::min(304LL / tiles, (P + 2047) / 2048));
+    if (tc_conv_ok(D.cin, D.cout)) {
+        // the split of tc_gemm_plan
+        const long long kb = (P + 63) / 64, per = (kb + std::min<long long>(splits, kb) - 1) / std::min<long long>(splits, kb);
+        const int ns = (int)((kb + per - 1) / per);
+        if ((size_t)ns * u->Kp[l] * D.cout > u->wpart_elems)
+            return unet_fail(MGMC_ERR_STATE, "split-K scratch too small");
+        UNET_CUDA(tc_conv_wgrad(u->layer_in(l), u->dz, B, Hs, D.cin, D.cout, ns, per * 64, u->wpart, u->status, st));
+        k_wt_to_flat<<<dim3((unsigned)((u->K[l] + 31) / 32), (unsigned)((D.cout + 31) / 32)), dim3(32, 32), 0, st>>>(
+            u->wpart, ns, u->Kp[l], u->K[l], D.cout, u->grad + u->woff[l]);
+        if (dx) UNET_CUDA(tc_conv_dgrad(u->dz, B, Hs, D.cin, u->Wt[l], D.cout, dx, u->status, st));
+        UNET_CUDA(cudaGetLastError());
+        return MGMC_OK;
+    }
     const dim3 tb(32, 8);
     k_transpose<<<dim3((unsigned)((P + 31) / 32), (unsigned)((D.cout + 31) / 32)), tb, 0, st>>>(u->dz, P, D.cout,
                                                                                                D.cout, u->dzT, P);
     const bf16* x = l == 0 ? input : u->layer_in(l);
-    k_im2col<<<grid_for(P * 9), 256, 0, st>>>(x, B, Hs, D.cin, u->col, u->Kp[l]);
+    im2col(u, x, B, Hs, l);
     k_transpose<<<dim3((unsigned)((P + 31) / 32), (unsigned)((u->Kp[l] + 31) / 32)), tb, 0, st>>>(
         u->col, P, u->Kp[l], u->Kp[l], u->colT, P);
-    // weight gradient dWt[Kp][co] = colT[Kp][P] dzT[co][P]^T, split over P for ~2 CTAs per SM
-    const long long tiles = (u->Kp[l] + 127) / 128;  // N = cout <= 256 is one tile
-    const int splits = (int)std::max(1LL, std::min(304LL / tiles, (P + 2047) / 2048));
+    // weight gradient dWt[Kp][co] = colT[Kp][P] dzT[co][P]^T
     mgmc_status rc = gemm(u, u->colT, (int)P, u->dzT, (int)P, u->dwt, u->Kp[l], D.cout, P, kEpiF32, nullptr, splits);
     if (rc != MGMC_OK) return rc;
-    k_wt_to_flat<<<grid_for((long long)u->K[l] * D.cout), 256, 0, st>>>(u->dwt, u->K[l], D.cout,
-                                                                        u->grad + u->woff[l]);
+    k_wt_to_flat<<<dim3((unsigned)((u->K[l] + 31) / 32), (unsigned)((D.cout + 31) / 32)), dim3(32, 32), 0, st>>>(
+        u->dwt, 1, u->Kp[l], u->K[l], D.cout, u->grad + u->woff[l]);
     if (dx) {
         rc = gemm(u, u->dz, D.cout, u->Wt[l], D.cout, u->dcol, P, u->Kp[l], D.cout, kEpiF32, nullptr, 1);
         if (rc != MGMC_OK) return rc;
@@ -565,13 +741,13 @@ mgmc_status loss_grad(UnetCtx* u, int B, const bf16* input, const float* target)
     const float scale = 2.0f / (float)((long long)B * u->n * u->n);
     k_loss<<<kRedBlocks, 256, 0, st>>>(u->out, target, B, u->H, u->n, scale, u->dout, u->part + kLossOff);
     k_out_bwd<<<kRedBlocks, 256, 0, st>>>(u->dout, u->act[13], P0, u->c0, u->wout_r, u->dact[13], u->part);
-    k_colsum<<<1, 256, 0, st>>>(u->part, kRedBlocks, u->c0 + 1, u->grad + u->out_w);
+    k_colsum<<<(u->c0 + 8) / 8, 256, 0, st>>>(u->part, kRedBlocks, u->c0 + 1, u->grad + u->out_w);
     const int c1 = u->L[2].cout, c2 = u->L[4].cout, c3 = u->L[6].cout, c0 = u->c0;
     auto pb = [&](int s, float* dy, float* dxx, int C) {  // pool of level s-1 -> s, backward
-        k_pool_bwd<<<grid_for(u->Ps(s - 1, B) * C), 256, 0, st>>>(dy, B, u->Hs(s), C, dxx, 1);
+        k_pool_bwd<<<grid_for(u->Ps(s - 1, B) * C / 8), 256, 0, st>>>(dy, B, u->Hs(s), C, dxx, 1);
     };
     auto ub = [&](int s, int ca, int cb, float* dlow, float* dskip) {
-        k_upcat_bwd<<<grid_for(u->Ps(s, B) * (ca + cb)), 256, 0, st>>>(u->du, ca, cb, B, u->Hs(s), dlow, dskip);
+        k_upcat_bwd<<<grid_for(u->Ps(s, B) * (ca + cb) / 8), 256, 0, st>>>(u->du, ca, cb, B, u->Hs(s), dlow, dskip);
     };
     if ((rc = conv_backward(u, 13, B, input, u->dact[12])) != MGMC_OK) return rc;
     if ((rc = conv_backward(u, 12, B, input, u->du)) != MGMC_OK) return rc;

@@ -59,6 +59,31 @@ def test_forward_matches_oracle(torch_mod):
     assert np.abs(got - ref).max() <= 5e-2 * rms, np.abs(got - ref).max() / rms
 
 
+@pytest.mark.parametrize("n,c0,batch", [(31, 16, 3), (31, 32, 1), (63, 16, 5), (127, 16, 1)])
+def test_implicit_convolutions_match_oracle(torch_mod, n, c0, batch):
+    """Every convolution kernel at its edges: 16-, 32- and 64-channel chunks, tiles of one to
+    eight images (4 x 4 bottom grids, a batch that does not fill them), lines (128 wide), output
+    channels below the tile.  Bounds as in the tests beside it."""
+    torch = torch_mod
+    net, theta, xr, xbits, t = _setup(torch, n, c0, batch=batch, seed=4)
+    got = net.predict(xbits, precision="fp64").cpu().numpy().reshape(batch, n, n)
+    ref = U.forward(theta, xr, c0, bf16=True)[0][:, :n, :n]
+    rel = np.linalg.norm(got - ref) / np.linalg.norm(ref)
+    assert rel <= 1e-2, rel
+    tg = torch.tensor(t.reshape(batch, n * n), dtype=torch.float32).cuda()
+    loss, g = net.gradient(xbits, tg, batch)
+    lo, go = U.loss_and_grad(theta, xr, t, c0, bf16=True)
+    assert abs(loss - lo) <= 1e-2 * lo
+    o = 0
+    for name, _, ci, co in U.layer_table(c0) + [("out", 0, c0, 1)]:
+        nw = co * 9 * ci if name != "out" else c0
+        for sl in (slice(o, o + nw), slice(o + nw, o + nw + co)):
+            err = np.linalg.norm(g[sl] - go[sl]) / max(np.linalg.norm(go[sl]), 1e-12)
+            assert err <= 5e-2, (name, err)
+        o += nw + co
+    net.close()
+
+
 @pytest.mark.parametrize("batch", [2, 4])
 def test_gradient_matches_oracle(torch_mod, batch):
     """batch 4 splits the weight-gradient GEMMs of the finest level over pixels."""
