@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/mgmc.h"
+#include "normal64.cuh"
 
 namespace mgmc {
 
@@ -159,18 +160,7 @@ __device__ __forceinline__ uint4 noise_counter(const CycleState& cs, unsigned pa
 
 // Box-Muller pair from one Philox block: u = (top 53 bits + 1/2) 2^-53,
 // z0 = r cos(2 pi u2), z1 = r sin(2 pi u2), r = sqrt(-2 ln u1).
-__device__ __forceinline__ void normal_pair(const uint4 w, double& z0, double& z1)
-{
-    unsigned long long k1 = (((unsigned long long)w.x << 32) | w.y) >> 11;
-    unsigned long long k2 = (((unsigned long long)w.z << 32) | w.w) >> 11;
-    double u1 = ((double)k1 + 0.5) * 0x1p-53;
-    double u2 = ((double)k2 + 0.5) * 0x1p-53;
-    double r = sqrt(-2.0 * log(u1));
-    double s, c;
-    sincospi(2.0 * u2, &s, &c);
-    z0 = r * c;
-    z1 = r * s;
-}
+__device__ __forceinline__ void normal_pair(const uint4 w, double& z0, double& z1) { n64::pair53(w, z0, z1); }
 
 // The same draws in FP32: u is the FP32 rounding of (k + 1/2) 2^-53, formed from
 // the two 32-bit halves so that the full 53-bit value is used.  The angle is
@@ -199,15 +189,8 @@ __device__ __forceinline__ void normal_pair(const uint4 w, float& z0, float& z1)
 // angle, accurate logarithm and reciprocal-square-root radius as normal_pair.
 __device__ __forceinline__ void normal_quad(const uint4 w, double& z0, double& z1, double& z2, double& z3)
 {
-    const double r0 = sqrt(-2.0 * log(((double)w.x + 0.5) * 0x1p-32));
-    const double r1 = sqrt(-2.0 * log(((double)w.z + 0.5) * 0x1p-32));
-    double s, c;
-    sincospi(2.0 * (((double)w.y + 0.5) * 0x1p-32), &s, &c);
-    z0 = r0 * c;
-    z1 = r0 * s;
-    sincospi(2.0 * (((double)w.w + 0.5) * 0x1p-32), &s, &c);
-    z2 = r1 * c;
-    z3 = r1 * s;
+    n64::pair32(w.x, w.y, z0, z1);
+    n64::pair32(w.z, w.w, z2, z3);
 }
 __device__ __forceinline__ void normal_quad(const uint4 w, float& z0, float& z1, float& z2, float& z3)
 {
@@ -228,12 +211,7 @@ __device__ __forceinline__ void normal_quad(const uint4 w, float& z0, float& z1,
 // transforming only the two words it needs (the same operations as normal_quad)
 __device__ __forceinline__ void normal_half(const uint4 w, int px, double& z0, double& z1)
 {
-    const unsigned wa = px ? w.z : w.x, wb = px ? w.w : w.y;
-    const double r = sqrt(-2.0 * log(((double)wa + 0.5) * 0x1p-32));
-    double s, c;
-    sincospi(2.0 * (((double)wb + 0.5) * 0x1p-32), &s, &c);
-    z0 = r * c;
-    z1 = r * s;
+    n64::pair32(px ? w.z : w.x, px ? w.w : w.y, z0, z1);
 }
 __device__ __forceinline__ void normal_half(const uint4 w, int px, float& z0, float& z1)
 {
