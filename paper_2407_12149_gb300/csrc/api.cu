@@ -97,6 +97,9 @@ struct mgmc_ctx {
     int n_qoi = 0;
     long long* q_site = nullptr;
     double* q_w = nullptr;
+    double* q_part = nullptr;   // partial sums and ticket of the QoI launch
+    int* q_ticket = nullptr;
+    int max_qoi = 0;            // most QoI sites of a chain
     void* x_stage = nullptr;
     double* u = nullptr;
     double* partial = nullptr;
@@ -517,7 +520,7 @@ void enqueue_cycle_batch(mgmc_ctx* h, cudaStream_t s, int& launches)
         launch_lowrank_batch<T>((const LowrankJob<T>*)h->jobs_lru[d], h->njob_lru[d], h->per_lru[d], h->nblk_lru[d],
                                 false, s, launches);
     }
-    launch_qoi_batch<T>((const QoiJob<T>*)h->jobs_qoi, nc, s, launches);
+    launch_qoi_batch<T>((const QoiJob<T>*)h->jobs_qoi, nc, h->max_qoi, s, launches);
 }
 
 // The phases of one visit of grid l <= small_top and everything below it, with the slots
@@ -621,7 +624,7 @@ void enqueue_cycle(mgmc_ctx* h, cudaStream_t s, int& launches)
         h->small_next = 0;
         std::vector<int> visit((size_t)h->L, 0);
         enqueue_level<T>(h, h->L - 1, visit, s, launches);
-        launch_qoi<T>(levels_of<T>(h)[h->L - 1], h->n_qoi, h->q_site, h->q_w, h->P, s, launches);
+        launch_qoi_batch<T>((const QoiJob<T>*)h->jobs_qoi, 1, h->max_qoi, s, launches);
         return;
     }
     auto& lv = levels_of<T>(h);
@@ -643,7 +646,7 @@ void enqueue_cycle(mgmc_ctx* h, cudaStream_t s, int& launches)
             if (prof && j == 0) cudaEventRecordWithFlags(h->ev[3], s, cudaEventRecordExternal);
             launch_lowrank<T>(D, P, 1, (unsigned)(2 * j + 1), false, s, launches);
         }
-        launch_qoi<T>(D, h->n_qoi, h->q_site, h->q_w, P, s, launches);
+        launch_qoi_batch<T>((const QoiJob<T>*)h->jobs_qoi, 1, h->max_qoi, s, launches);
         return;
     }
     for (int l = Lf; l > h->top; --l) {
@@ -670,7 +673,7 @@ void enqueue_cycle(mgmc_ctx* h, cudaStream_t s, int& launches)
             launch_lowrank<T>(D, P, 1, (unsigned)(2 * j + 1), false, s, launches);
         }
     }
-    launch_qoi<T>(lv[Lf], h->n_qoi, h->q_site, h->q_w, P, s, launches);
+    launch_qoi_batch<T>((const QoiJob<T>*)h->jobs_qoi, 1, h->max_qoi, s, launches);
 }
 
 mgmc_status ensure_graph(mgmc_ctx* h)
@@ -989,6 +992,8 @@ mgmc_status mgmc_create(const mgmc_config* cfg_in, const mgmc_allocator* alloc, 
         }
         h->q_site = upload(h, qs, st);
         h->q_w = upload(h, qw, st);
+        h->q_part = upload(h, std::vector<double>(kQoiMaxCtas, 0.0), st);
+        h->q_ticket = upload(h, std::vector<int>(1, 0), st);
     }
     // staging and mean-solve scratch
     size_t esz = h->fp32() ? 4 : 8;
@@ -1003,6 +1008,14 @@ mgmc_status mgmc_create(const mgmc_config* cfg_in, const mgmc_allocator* alloc, 
     if (h->fused) {
         st = h->fp32() ? build_batch_tables<float>(h) : build_batch_tables<double>(h);
         if (st != MGMC_OK) return cleanup(st);
+    } else {
+        h->max_qoi = h->n_qoi;
+        auto job = [&](auto* x) {
+            using T = std::remove_pointer_t<decltype(x)>;
+            return upload(h, std::vector<QoiJob<T>>{{x, h->n_qoi, h->q_site, h->q_w, h->cs, h->q_part, h->q_ticket}}, st);
+        };
+        h->jobs_qoi = h->fp32() ? (void*)job(h->lf[h->L - 1].x) : (void*)job(h->ld[h->L - 1].x);
+        if (st != MGMC_OK) return cleanup(fail(st, "device upload failed"));
     }
     if (cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
         return cleanup(fail(MGMC_ERR_CUDA, "stream creation failed"));
@@ -1445,7 +1458,8 @@ mgmc_status build_batch_tables(mgmc_ctx* h)
     for (mgmc_ctx* c : chains) {
         cj.push_back(coarse_job<T>(c));
         const DevLevel<T>& Fh = levels_of<T>(c)[c->L - 1];
-        qj.push_back({Fh.x, c->n_qoi, c->q_site, c->q_w, c->cs});
+        qj.push_back({Fh.x, c->n_qoi, c->q_site, c->q_w, c->cs, c->q_part, c->q_ticket});
+        h->max_qoi = std::max(h->max_qoi, c->n_qoi);
         pj.push_back({Fh.x, Fh.n, Fh.pitch, Fh.base});
         h->pack_max_n = std::max(h->pack_max_n, Fh.n);
         csl.push_back(c->cs);

@@ -998,7 +998,16 @@ bool coarse_plan(int dim, const int* n_of_level, int top, bool top_is_fd_finest,
     return false;
 }
 
-// F^T theta of every chain's finest grid, then step += 1, cycle += 1 (one CTA per chain)
+__host__ __device__ inline int qoi_ctas(int n_qoi)
+{
+    const int c = (n_qoi + 1023) / 1024;
+    return c < 1 ? 1 : (c > kQoiMaxCtas ? kQoiMaxCtas : c);
+}
+
+// F^T theta of every chain's finest grid, then step += 1, cycle += 1.  Up to 16 CTAs per
+// chain: products and conversions are FP64, a few hundred cycles per warp and site each, so a
+// QoI of thousands of sites takes several SMs (one CTA: 60 us for 16 641 sites, 16 CTAs:
+// about 6 us).  The partial sums are added by the chain's last CTA in CTA order.
 template <typename T>
 __global__ void k_qoi_batch(const QoiJob<T>* __restrict__ jobs)
 {
@@ -1006,13 +1015,17 @@ __global__ void k_qoi_batch(const QoiJob<T>* __restrict__ jobs)
     pdl_launch_dependents();
     // the QoI sites and weights never change: the first kQoiPre of each thread are loaded
     // before the wait on the preceding launch, the state after it (same summation order)
-    constexpr int kQoiPre = 8;
-    const QoiJob<T> J = jobs[blockIdx.x];
+    constexpr int kQoiPre = 4;
+    const QoiJob<T> J = jobs[blockIdx.y];
+    // the chain's own number of CTAs: its sum does not depend on the other chains of a launch
+    const int nb = qoi_ctas(J.n_qoi);
+    if ((int)blockIdx.x >= nb) return;
+    const int t0 = blockIdx.x * blockDim.x + threadIdx.x, st = nb * blockDim.x;
     long long site[kQoiPre];
     double w[kQoiPre];
 #pragma unroll
     for (int r = 0; r < kQoiPre; ++r) {
-        const int t = threadIdx.x + r * blockDim.x;
+        const int t = t0 + r * st;
         site[r] = t < J.n_qoi ? J.q_site[t] : 0;
         w[r] = t < J.n_qoi ? J.q_w[t] : 0.0;
     }
@@ -1020,23 +1033,30 @@ __global__ void k_qoi_batch(const QoiJob<T>* __restrict__ jobs)
     double acc = 0.0;
 #pragma unroll
     for (int r = 0; r < kQoiPre; ++r)
-        if (threadIdx.x + r * blockDim.x < J.n_qoi) acc += w[r] * (double)J.x[site[r]];
-    for (int t = threadIdx.x + kQoiPre * blockDim.x; t < J.n_qoi; t += blockDim.x)
-        acc += J.q_w[t] * (double)J.x[J.q_site[t]];
+        if (t0 + r * st < J.n_qoi) acc += w[r] * (double)J.x[site[r]];
+    for (int t = t0 + kQoiPre * st; t < J.n_qoi; t += st) acc += J.q_w[t] * (double)J.x[J.q_site[t]];
     part[threadIdx.x] = acc;
     __syncthreads();
-    for (int st = blockDim.x / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st) part[threadIdx.x] += part[threadIdx.x + st];
+    for (int h = blockDim.x / 2; h > 0; h >>= 1) {
+        if (threadIdx.x < h) part[threadIdx.x] += part[threadIdx.x + h];
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        CycleState* cs = J.cs;
-        double q = part[0];
-        if (cs->qoi) cs->qoi[cs->step] = q;
-        if (!isfinite(q)) atomicOr(&cs->status, kStatusNumeric);
-        cs->step += 1;
-        cs->cycle += 1;
+    if (threadIdx.x != 0) return;
+    double q = part[0];
+    if (nb > 1) {
+        J.part[blockIdx.x] = q;
+        __threadfence();
+        if (atomicAdd(J.ticket, 1) != nb - 1) return;
+        __threadfence();
+        q = 0.0;
+        for (int b = 0; b < nb; ++b) q += __ldcg(J.part + b);
+        *J.ticket = 0;
     }
+    CycleState* cs = J.cs;
+    if (cs->qoi) cs->qoi[cs->step] = q;
+    if (!isfinite(q)) atomicOr(&cs->status, kStatusNumeric);
+    cs->step += 1;
+    cs->cycle += 1;
 }
 
 __global__ void k_set_cycle_batch(CycleState* const* cs, int n, unsigned long long seed, unsigned long long cycle,
@@ -1085,9 +1105,9 @@ void launch_coarse(const CoarseJob<T>* jobs, int n, int dim, int threads, size_t
 }
 
 template <typename T>
-void launch_qoi_batch(const QoiJob<T>* jobs, int n, cudaStream_t st, int& launches)
+void launch_qoi_batch(const QoiJob<T>* jobs, int n, int max_qoi, cudaStream_t st, int& launches)
 {
-    launch_pdl(k_qoi_batch<T>, dim3((unsigned)n), dim3(256), 0, st, jobs);
+    launch_pdl(k_qoi_batch<T>, dim3((unsigned)qoi_ctas(max_qoi), (unsigned)n), dim3(256), 0, st, jobs);
     ++launches;
 }
 
@@ -1103,7 +1123,7 @@ template cudaError_t coarse_image<float>(const CoarseJob<float>*, unsigned char*
 template cudaError_t coarse_image<double>(const CoarseJob<double>*, unsigned char*, int, cudaStream_t);
 template void launch_coarse<float>(const CoarseJob<float>*, int, int, int, size_t, cudaStream_t, int&);
 template void launch_coarse<double>(const CoarseJob<double>*, int, int, int, size_t, cudaStream_t, int&);
-template void launch_qoi_batch<float>(const QoiJob<float>*, int, cudaStream_t, int&);
-template void launch_qoi_batch<double>(const QoiJob<double>*, int, cudaStream_t, int&);
+template void launch_qoi_batch<float>(const QoiJob<float>*, int, int, cudaStream_t, int&);
+template void launch_qoi_batch<double>(const QoiJob<double>*, int, int, cudaStream_t, int&);
 
 }  // namespace mgmc

@@ -10,7 +10,7 @@
 // which ends in the exact coarsest Cholesky sample (Sec. 3.5), and back up:
 //   k_prolong                              : theta += P psi_{l-1}
 //   k_sweep_colour  (reverse colours), k_lowrank_v + k_lowrank_apply (backward G)
-// and k_qoi_advance records F^T theta and advances the cycle counter.
+// and k_qoi_batch (coarse.cu) records F^T theta and advances the cycle counter.
 //
 // Low-rank bookkeeping: the right-hand side of level l is kept as
 // f_l = fdense_l + B_l Gamma^-1 d_l with a dense field fdense_l and an m-vector
@@ -529,31 +529,6 @@ __global__ void __launch_bounds__(kSmallCycleThreads)
     }
 }
 
-// The whole V-cycle below (and including) level `top`, one CTA.
-// levels[0..top] are the device descriptors, index = paper level.
-// F^T theta of the finest level into qoi[step]; then step += 1, cycle += 1.
-template <typename T>
-__global__ void k_qoi_advance(DevLevel<T> L, int n_qoi, const long long* q_site, const double* q_w, DevProblem P)
-{
-    __shared__ double part[256];
-    double acc = 0.0;
-    for (int t = threadIdx.x; t < n_qoi; t += blockDim.x) acc += q_w[t] * (double)L.x[q_site[t]];
-    part[threadIdx.x] = acc;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) part[threadIdx.x] += part[threadIdx.x + s];
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        CycleState* cs = P.cs;
-        double q = part[0];
-        if (cs->qoi) cs->qoi[cs->step] = q;
-        if (!isfinite(q)) atomicOr(&cs->status, kStatusNumeric);
-        cs->step += 1;
-        cs->cycle += 1;
-    }
-}
-
 __global__ void k_set_cycle(CycleState* cs, unsigned long long seed, unsigned long long cycle, unsigned chain,
                             int noise, double* qoi)
 {
@@ -772,14 +747,6 @@ void launch_cycle_small(const DevLevel<T>* levels_dev, int top, const DevProblem
     ++launches;
 }
 
-template <typename T>
-void launch_qoi(const DevLevel<T>& L, int n_qoi, const long long* q_site, const double* q_w, const DevProblem& P,
-                cudaStream_t st, int& launches)
-{
-    k_qoi_advance<T><<<1, 256, 0, st>>>(L, n_qoi, q_site, q_w, P);
-    ++launches;
-}
-
 void launch_set_cycle(CycleState* cs, unsigned long long seed, unsigned long long cycle, unsigned chain, int noise,
                       double* qoi, cudaStream_t st)
 {
@@ -832,8 +799,6 @@ void launch_resid(const DevLevel<T>& L, const DevProblem& P, double* u, double* 
                                           cudaStream_t, int&);                                                   \
     template void launch_cycle_small<T>(const DevLevel<T>*, int, const DevProblem&, const double*, int,            \
                                         const int4*, int, double*, cudaStream_t, int&);                          \
-    template void launch_qoi<T>(const DevLevel<T>&, int, const long long*, const double*, const DevProblem&,      \
-                                cudaStream_t, int&);                                                             \
     template void launch_pack<T>(const DevLevel<T>&, T*, bool, cudaStream_t);                               \
     template void launch_pack_batch<T>(const PackJob<T>*, void* const*, int, int, bool, cudaStream_t);         \
     template void launch_resid<T>(const DevLevel<T>&, const DevProblem&, double*, double*, int, double*,         \

@@ -78,9 +78,12 @@ struct QoiJob {
     const long long* q_site;
     const double* q_w;
     CycleState* cs;
+    double* part;                // [kQoiMaxCtas] partial sums
+    int* ticket;                 // CTAs of the launch that have finished (0 between launches)
 };
+constexpr int kQoiMaxCtas = 16;
 template <typename T>
-void launch_qoi_batch(const QoiJob<T>* jobs, int n, cudaStream_t st, int& launches);
+void launch_qoi_batch(const QoiJob<T>* jobs, int n, int max_qoi, cudaStream_t st, int& launches);
 void launch_set_cycle_batch(CycleState* const* cs, int n, unsigned long long seed, unsigned long long cycle, int noise,
                             double* qoi, long long n_steps, cudaStream_t st);
 
@@ -92,9 +95,6 @@ cudaError_t coarse_image(const CoarseJob<T>* job, unsigned char* image, int dim,
 template <typename T>
 void launch_coarse(const CoarseJob<T>* jobs, int n, int dim, int threads, size_t smem_bytes, cudaStream_t st,
                    int& launches);
-template <typename T>
-void launch_qoi(const DevLevel<T>& L, int n_qoi, const long long* q_site, const double* q_w, const DevProblem& P,
-                cudaStream_t st, int& launches);
 void launch_set_cycle(CycleState* cs, unsigned long long seed, unsigned long long cycle, unsigned chain, int noise,
                       double* qoi, cudaStream_t st);
 template <typename T>
