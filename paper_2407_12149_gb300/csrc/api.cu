@@ -132,6 +132,7 @@ struct mgmc_ctx {
     std::vector<void*> maps_fwd, maps_bwd;   // TileMaps per tile job, per depth
     std::vector<int> njob_tile, nblk_tile, njob_lrd, nblk_lrd, njob_lru, nblk_lru;
     std::vector<int> per_tile, per_lrd, per_lru;
+    std::vector<int> cl_lrd, cl_lru;   // cluster size of the low-rank launches (1: none)
     // FP32 finest grids: the streaming kernels (stream2d.cu) instead of depth-0 tiles
     bool stream_fine = false;
     bool fine0 = true;    // the depth-0 grids have the 5-point finite-difference form
@@ -501,7 +502,7 @@ void enqueue_cycle_batch(mgmc_ctx* h, cudaStream_t s, int& launches)
                                  s, launches);
         if (prof && d == 0) cudaEventRecordWithFlags(h->ev[1], s, cudaEventRecordExternal);
         launch_lowrank_batch<T>((const LowrankJob<T>*)h->jobs_lrd[d], h->njob_lrd[d], h->per_lrd[d], h->nblk_lrd[d],
-                                true, s, launches);
+                                h->cl_lrd[d], true, s, launches);
     }
     launch_coarse<T>((const CoarseJob<T>*)h->jobs_coarse, nc, 2, coarse_cta(h), h->batch_coarse_smem, s, launches);
     for (int d = h->n_depth - 1; d >= 0; --d) {
@@ -518,7 +519,7 @@ void enqueue_cycle_batch(mgmc_ctx* h, cudaStream_t s, int& launches)
                                  launches);
         if (prof && d == 0) cudaEventRecordWithFlags(h->ev[3], s, cudaEventRecordExternal);
         launch_lowrank_batch<T>((const LowrankJob<T>*)h->jobs_lru[d], h->njob_lru[d], h->per_lru[d], h->nblk_lru[d],
-                                false, s, launches);
+                                h->cl_lru[d], false, s, launches);
     }
     launch_qoi_batch<T>((const QoiJob<T>*)h->jobs_qoi, nc, h->max_qoi, s, launches);
 }
@@ -1404,6 +1405,17 @@ mgmc_status build_batch_tables(mgmc_ctx* h)
                 h->s9_grid.back() = stream9_grid(strips);
             }
         }
+        // grids without z partials: the blocks of a low-rank job are one cluster, of one size
+        // for all jobs of the launch
+        const bool zst = (d == 0 && h->stream_fine) || s9;
+        int cld = 1, clu = 1;
+        for (mgmc_ctx* c : chains) {
+            const int l = c->L - 1 - d;
+            if (l <= c->top || c->m == 0) continue;
+            const DevLevel<T>& Lh = levels_of<T>(c)[l];
+            cld = std::max(cld, lowrank_cluster(std::max(Lh.g_rows[0], Lh.h_rows)));
+            clu = std::max(clu, lowrank_cluster(Lh.g_rows[1]));
+        }
         for (mgmc_ctx* c : chains) {
             const int l = c->L - 1 - d;
             if (l <= c->top) continue;
@@ -1419,15 +1431,18 @@ mgmc_status build_batch_tables(mgmc_ctx* h)
             if (!make_tile_maps<T>(Lh, Ch, false, &mf.back()) || !make_tile_maps<T>(Lh, Ch, true, &mb.back()))
                 return fail(MGMC_ERR_CUDA, "TMA descriptor encoding failed");
             if (c->m > 0) {
-                int rd = std::max(Lh.g_rows[0], Lh.h_rows);
                 DevLevel<T> Lz = Lh;
-                if ((d == 0 && h->stream_fine) || s9) Lz.zparts = nullptr;   // the low-rank kernel reads the state
-                ld.push_back({Lz, Ch, c->P, bd, lowrank_blocks(rd)});
-                bd += lowrank_blocks(rd);
-                lu.push_back({Lz, Ch, c->P, bu, lowrank_blocks(Lh.g_rows[1])});
-                bu += lowrank_blocks(Lh.g_rows[1]);
+                if (zst) Lz.zparts = nullptr;   // the low-rank kernel reads the state
+                const int nd = zst ? cld : lowrank_blocks(std::max(Lh.g_rows[0], Lh.h_rows));
+                const int nu = zst ? clu : lowrank_blocks(Lh.g_rows[1]);
+                ld.push_back({Lz, Ch, c->P, bd, nd});
+                bd += nd;
+                lu.push_back({Lz, Ch, c->P, bu, nu});
+                bu += nu;
             }
         }
+        h->cl_lrd.push_back(zst ? cld : 1);
+        h->cl_lru.push_back(zst ? clu : 1);
         // common block count of the jobs of one launch (0: they differ)
         auto common = [](const auto& v, auto count) {
             int per = v.empty() ? 0 : count(v[0]);

@@ -883,122 +883,142 @@ __global__ void __launch_bounds__(TileGeom<T, FINE, BWD>::NT, 3)
 // The same step when m <= kLrReg and every thread holds at most one row of G
 // (and of H): all loads that do not depend on v -- the thread's G/H row, its
 // site and the value there, B^T G, d, the Cholesky diagonal -- are issued before
-// z and v are formed.  The static ones (G/H rows, sites, B^T G, column pointers,
-// L_Gamma) are issued before the wait on the preceding launch (pdl_wait), so
+// z and v are formed.  What set-up fixed (G/H rows, sites, B^T G, column pointers,
+// L_Gamma) is loaded, and the low-rank noise L_Gamma z' drawn, before the wait on the
+// preceding launch (pdl_wait; the cycle state changes only in a cycle's last launch), so
 // after it only the state, f, d and the z partials are fetched: one round trip.
-// The sums run in the same order as the general path.  Both forms call
-// pdl_wait themselves.
+// An FP64 instruction or conversion costs a warp about 70 cycles on this GPU and does not
+// overlap with its next one, so z and B^T G v take four lanes per observation and v is
+// rounded to the path precision once, not by every thread that applies it.
+// Streamed grids keep no partials: every CTA of a job reads the state at the observation
+// entries, which other CTAs of the job update.  Those CTAs are one cluster, and no CTA writes
+// the state before all have read it (state_read / state_free).
+// Both forms call pdl_wait themselves.
+// Measured (GB300): eight 1023^2 FP32 chains, 4 cycles (40 of these launches) 1524 -> 1402 us,
+// 1023^2 FP64 chain, 2 cycles 1410 -> 1341 us.
 constexpr int kLrReg = 16;
-// entries of a column of B whose sites are loaded before the wait (point observations have 4)
-constexpr int kLrEnt = 4;
 
-// z_k = (B^T theta)_k from the z partials of the tile kernels, or (streamed finest
-// grid, no partials) from the state itself: the same products w_t theta(site_t),
-// rounded before they are summed, in the same order
+// z_k = (B^T theta)_k, by four lanes (lane p of the observation takes the entries p, p + 4, ..):
+// from the z partials of the tile kernels, or (streamed grids, no partials) from the
+// state itself, the products w_t theta(site_t) rounded before they are summed
 template <typename T>
-__device__ __forceinline__ double lowrank_z(const DevLevel<T>& L, const T* x, int k)
+__device__ __forceinline__ double lowrank_z4(const DevLevel<T>& L, const T* x, int k, int p, bool on)
 {
     double acc = 0.0;
-    if (L.zparts)
-        for (int t = L.bcol_ptr[k]; t < L.bcol_ptr[k + 1]; ++t) acc += L.zparts[t];
-    else
-        for (int t = L.bcol_ptr[k]; t < L.bcol_ptr[k + 1]; ++t) acc += __dmul_rn(L.bcol_w[t], (double)x[L.bcol_site[t]]);
+    if (on) {
+        const int t1 = L.bcol_ptr[k + 1];
+        if (L.zparts)
+            for (int t = L.bcol_ptr[k] + p; t < t1; t += 4) acc += L.zparts[t];
+        else
+            for (int t = L.bcol_ptr[k] + p; t < t1; t += 4) acc += __dmul_rn(L.bcol_w[t], (double)x[L.bcol_site[t]]);
+    }
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 2);
     return acc;
+}
+
+// cluster barrier around the update of a state that all CTAs of the cluster read
+__device__ __forceinline__ void state_read() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void state_free() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
+
+// L_Gamma z' of one observation; zp: the standard normals z' (in shared memory)
+__device__ __forceinline__ double lowrank_lz(const DevProblem& P, const double* zp, int k)
+{
+    if (P.gamma_diag) return P.LG[k * P.m + k] * zp[k];
+    double lz = 0.0;
+    for (int t = 0; t <= k; ++t) lz += P.LG[k * P.m + t] * zp[t];
+    return lz;
 }
 
 template <typename T>
 __device__ __forceinline__ void lowrank_fused_short(const DevLevel<T>& L, const DevLevel<T>& C, const DevProblem& P,
-                                                    int down, int blk, double* z, double* zp, double* v)
+                                                    int down, int blk, double* z, double* zp, double* v, T* vt)
 {
     const int m = P.m;
     const int dir = down ? 0 : 1;
     const unsigned slot = down ? 0u : 1u;
     T* x = down ? L.x2 : L.x;
     const int r0 = blk * blockDim.x + threadIdx.x;
-    const int k0 = threadIdx.x;
+    // observation k, lane p of its four
+    const int k = threadIdx.x >> 2, p = threadIdx.x & 3;
     const bool hg = r0 < L.g_rows[dir];
     const bool hh = down && r0 < L.h_rows;
-    const bool hk = k0 < m;
+    const bool hk = k < m;
     const bool hb = down && blk == 0 && hk;
+    // the draws first: their chain is the longest
+    if ((int)threadIdx.x < m) zp[threadIdx.x] = P.cs->noise ? lowrank_normal<T>(*P.cs, L.level, slot, threadIdx.x) : 0.0;
     T gr[kLrReg], hr[kLrReg];
-    double bg[kLrReg];
+    double bg[kLrReg / 4];
 #pragma unroll
-    for (int k = 0; k < kLrReg; ++k) {
-        gr[k] = (hg && k < m) ? L.gT[dir][(long long)r0 * m + k] : T(0);
-        hr[k] = (hh && k < m) ? L.hT[(long long)r0 * m + k] : T(0);
-        bg[k] = (hb && k < m) ? L.BtG[k0 * m + k] : 0.0;
+    for (int t = 0; t < kLrReg; ++t) {
+        gr[t] = (hg && t < m) ? L.gT[dir][(long long)r0 * m + t] : T(0);
+        hr[t] = (hh && t < m) ? L.hT[(long long)r0 * m + t] : T(0);
     }
+#pragma unroll
+    for (int t = 0; t < kLrReg / 4; ++t) bg[t] = (hb && p + 4 * t < m) ? L.BtG[k * m + p + 4 * t] : 0.0;
     const long long gs = hg ? L.g_site[dir][r0] : 0;
     const long long hs = hh ? L.h_site[r0] : 0;
-    int t0 = 0, t1 = 0;
-    double lgk = 0.0;
-    if (hk) {
-        t0 = L.bcol_ptr[k0];
-        t1 = L.bcol_ptr[k0 + 1];
-        if (P.gamma_diag) lgk = P.LG[k0 * m + k0];
-    }
-    // without z partials (streamed finest grid) the state is read at the entries of
-    // column k0 of B: their sites and weights are static
+    // the lane's first entry of the column (point observations have four); static
     const bool zst = L.zparts == nullptr;
-    long long es[kLrEnt];
-    double ew[kLrEnt];
-#pragma unroll
-    for (int u = 0; u < kLrEnt; ++u) {
-        const bool has = hk && zst && t0 + u < t1;
-        es[u] = has ? L.bcol_site[t0 + u] : 0;
-        ew[u] = has ? L.bcol_w[t0 + u] : 0.0;
+    int t0 = 0, t1 = 0;
+    if (hk) {
+        t0 = L.bcol_ptr[k] + p;
+        t1 = L.bcol_ptr[k + 1];
     }
+    const bool he = zst && t0 < t1;
+    const long long es = he ? L.bcol_site[t0] : 0;
+    const double ew = he ? L.bcol_w[t0] : 0.0;
+    __syncthreads();
+    const double lz = (hk && p == 0) ? lowrank_lz(P, zp, k) : 0.0;
     // everything below depends on the preceding launches
     pdl_wait();
-    const CycleState cs = *P.cs;
-    const double dk = hk ? L.d[k0] : 0.0;
+    const double dk = (hk && p == 0) ? L.d[k] : 0.0;
     const T xv = hg ? x[gs] : T(0);
     const T fv = hh ? C.f[hs] : T(0);
-    if (hk) {
+    if ((int)threadIdx.x < ((4 * m + 31) & ~31)) {
         double acc = 0.0;
         if (zst) {
-#pragma unroll
-            for (int u = 0; u < kLrEnt; ++u)
-                if (t0 + u < t1) acc += __dmul_rn(ew[u], (double)x[es[u]]);
-            for (int t = t0 + kLrEnt; t < t1; ++t) acc += __dmul_rn(L.bcol_w[t], (double)x[L.bcol_site[t]]);
+            if (he) acc = __dmul_rn(ew, (double)x[es]);
+            for (int t = t0 + 4; t < t1; t += 4) acc += __dmul_rn(L.bcol_w[t], (double)x[L.bcol_site[t]]);
         } else {
-            for (int t = t0; t < t1; ++t) acc += L.zparts[t];
+            for (int t = t0; t < t1; t += 4) acc += L.zparts[t];
         }
-        z[k0] = acc;
-        zp[k0] = cs.noise ? lowrank_normal<T>(cs, L.level, slot, k0) : 0.0;
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        if (hk && p == 0) {
+            const double vk = acc - dk - lz;
+            vt[k] = (T)vk;
+            v[k] = vk;
+            z[k] = acc;
+        }
     }
     __syncthreads();
-    if (hk) {
-        double lz = 0.0;
-        if (cs.noise) {
-            if (P.gamma_diag)
-                lz = lgk * zp[k0];
-            else
-                for (int t = 0; t <= k0; ++t) lz += P.LG[k0 * m + t] * zp[t];
-        }
-        v[k0] = z[k0] - dk - lz;
+    if (zst) {
+        state_read();
+        state_free();
     }
-    __syncthreads();
     if (hg) {
         T acc = T(0);
 #pragma unroll
-        for (int k = 0; k < kLrReg; ++k)
-            if (k < m) acc += gr[k] * (T)v[k];
+        for (int t = 0; t < kLrReg; ++t)
+            if (t < m) acc += gr[t] * vt[t];
         x[gs] = xv - acc;
     }
     if (hh) {
         T acc = T(0);
 #pragma unroll
-        for (int k = 0; k < kLrReg; ++k)
-            if (k < m) acc += hr[k] * (T)v[k];
+        for (int t = 0; t < kLrReg; ++t)
+            if (t < m) acc += hr[t] * vt[t];
         C.f[hs] = fv + acc;
     }
-    if (hb) {
+    if (down && blk == 0 && (int)threadIdx.x < ((4 * m + 31) & ~31)) {
         double acc = 0.0;
 #pragma unroll
-        for (int k = 0; k < kLrReg; ++k)
-            if (k < m) acc += bg[k] * v[k];
-        L.dnext[k0] = dk - z[k0] + acc;
+        for (int t = 0; t < kLrReg / 4; ++t)
+            if (hk && p + 4 * t < m) acc += bg[t] * v[p + 4 * t];
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        if (hk && p == 0) L.dnext[k] = dk - z[k] + acc;
     }
 }
 
@@ -1009,53 +1029,58 @@ __device__ __forceinline__ void lowrank_fused_body(const DevLevel<T>& L, const D
     __shared__ double z[kMaxObs];
     __shared__ double zp[kMaxObs];
     __shared__ double v[kMaxObs];
+    __shared__ T vt[kMaxObs];
     const int m = P.m;
     const int dir = down ? 0 : 1;
     const unsigned slot = down ? 0u : 1u;
     const int stride = nblk * blockDim.x;
     if (m <= kLrReg && L.g_rows[dir] <= stride && (!down || L.h_rows <= stride)) {
-        lowrank_fused_short<T>(L, C, P, down, blk, z, zp, v);
+        lowrank_fused_short<T>(L, C, P, down, blk, z, zp, v, vt);
         return;
     }
+    for (int k = threadIdx.x; k < m; k += blockDim.x)
+        zp[k] = P.cs->noise ? lowrank_normal<T>(*P.cs, L.level, slot, k) : 0.0;
+    __syncthreads();
+    const int kq = threadIdx.x >> 2, p = threadIdx.x & 3;   // 256 threads: four lanes for each of up to 64 observations
+    const double lz = (kq < m && p == 0) ? lowrank_lz(P, zp, kq) : 0.0;
     pdl_wait();
-    const CycleState cs = *P.cs;
     T* x = down ? L.x2 : L.x;
-    for (int k = threadIdx.x; k < m; k += blockDim.x) {
-        z[k] = lowrank_z<T>(L, x, k);
-        zp[k] = cs.noise ? lowrank_normal<T>(cs, L.level, slot, k) : 0.0;
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < m; k += blockDim.x) {
-        double lz = 0.0;
-        if (cs.noise) {
-            if (P.gamma_diag)
-                lz = P.LG[k * m + k] * zp[k];
-            else
-                for (int t = 0; t <= k; ++t) lz += P.LG[k * m + t] * zp[t];
+    {
+        const double acc = lowrank_z4<T>(L, x, kq, p, kq < m);
+        if (kq < m && p == 0) {
+            const double vk = acc - L.d[kq] - lz;
+            vt[kq] = (T)vk;
+            v[kq] = vk;
+            z[kq] = acc;
         }
-        v[k] = z[k] - L.d[k] - lz;
     }
     __syncthreads();
+    if (!L.zparts) {
+        state_read();
+        state_free();
+    }
     const T* Gm = L.gT[dir];
     for (int r = blk * blockDim.x + threadIdx.x; r < L.g_rows[dir]; r += stride) {
         T acc = T(0);
-        for (int k = 0; k < m; ++k) acc += Gm[(long long)r * m + k] * (T)v[k];
+        for (int k = 0; k < m; ++k) acc += Gm[(long long)r * m + k] * vt[k];
         long long s = L.g_site[dir][r];
         x[s] = x[s] - acc;
     }
     if (!down) return;
     for (int r = blk * blockDim.x + threadIdx.x; r < L.h_rows; r += stride) {
         T acc = T(0);
-        for (int k = 0; k < m; ++k) acc += L.hT[(long long)r * m + k] * (T)v[k];
+        for (int k = 0; k < m; ++k) acc += L.hT[(long long)r * m + k] * vt[k];
         long long s = L.h_site[r];
         C.f[s] = C.f[s] + acc;
     }
-    if (blk == 0)
-        for (int k = threadIdx.x; k < m; k += blockDim.x) {
-            double acc = 0.0;
-            for (int t = 0; t < m; ++t) acc += L.BtG[k * m + t] * v[t];
-            L.dnext[k] = L.d[k] - z[k] + acc;
-        }
+    if (blk == 0) {
+        double acc = 0.0;
+        if (kq < m)
+            for (int t = p; t < m; t += 4) acc += L.BtG[kq * m + t] * v[t];
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        if (kq < m && p == 0) L.dnext[kq] = L.d[kq] - z[kq] + acc;
+    }
 }
 
 // batched: job j owns blocks [block0, block0 + nblocks)
@@ -1077,6 +1102,12 @@ int lowrank_blocks(int rows)
     if (blocks < 1) blocks = 1;
     if (blocks > 64) blocks = 64;
     return blocks;
+}
+int lowrank_cluster(int rows)
+{
+    int c = 1;
+    while (c < 8 && 256 * c < rows) c *= 2;
+    return c;
 }
 namespace {
 
@@ -1190,11 +1221,12 @@ void launch_tile_batch(const TileJob<T>* jobs, const TileMaps* maps, int njobs, 
 }
 
 template <typename T>
-void launch_lowrank_batch(const LowrankJob<T>* jobs, int njobs, int per, int nblocks, bool down, cudaStream_t st,
-                          int& launches)
+void launch_lowrank_batch(const LowrankJob<T>* jobs, int njobs, int per, int nblocks, int cluster, bool down,
+                          cudaStream_t st, int& launches)
 {
     if (nblocks <= 0) return;
-    launch_pdl(k_lowrank_fused_batch<T>, dim3((unsigned)nblocks), dim3(256), 0, st, jobs, njobs, per, down ? 1 : 0);
+    launch_pdl_cluster(k_lowrank_fused_batch<T>, dim3((unsigned)nblocks), dim3(256), 0, (unsigned)cluster, st, jobs, njobs,
+                       per, down ? 1 : 0);
     ++launches;
 }
 
@@ -1203,7 +1235,7 @@ void launch_lowrank_batch(const LowrankJob<T>* jobs, int njobs, int per, int nbl
     template cudaError_t tile_prepare_batch<T>();                                                                 \
     template void launch_tile_batch<T>(const TileJob<T>*, const TileMaps*, int, int, int, bool, bool, bool,       \
                                        cudaStream_t, int&);                                                       \
-    template void launch_lowrank_batch<T>(const LowrankJob<T>*, int, int, int, bool, cudaStream_t, int&);
+    template void launch_lowrank_batch<T>(const LowrankJob<T>*, int, int, int, int, bool, cudaStream_t, int&);
 
 MGMC_TILE_INST(float)
 MGMC_TILE_INST(double)

@@ -46,10 +46,13 @@ bool make_tile_maps(const DevLevel<T>& L, const DevLevel<T>& C, bool bwd, TileMa
 template <typename T>
 void launch_tile_batch(const TileJob<T>* jobs, const TileMaps* maps, int njobs, int per, int ntiles, bool fine,
                        bool bwd, bool x_zero, cudaStream_t st, int& launches);
-// per: the common block count of every job (0 if they differ)
+// per: the common block count of every job (0 if they differ).  cluster: 1, or -- grids without
+// z partials -- the block count of every job, launched as one cluster
 template <typename T>
-void launch_lowrank_batch(const LowrankJob<T>* jobs, int njobs, int per, int nblocks, bool down, cudaStream_t st,
-                          int& launches);
+void launch_lowrank_batch(const LowrankJob<T>* jobs, int njobs, int per, int nblocks, int cluster, bool down,
+                          cudaStream_t st, int& launches);
 int lowrank_blocks(int rows);
+// blocks of a job whose blocks form a cluster: 1, 2, 4 or 8, one row of G per thread while it lasts
+int lowrank_cluster(int rows);
 
 }  // namespace mgmc
