@@ -122,7 +122,7 @@ struct mgmc_ctx {
     int small_top = -1;
     int4* small_ops = nullptr;
     double* small_z = nullptr;   // normals of one sweep of the largest 25-point grid held
-    std::vector<int> small_off, small_cnt;
+    std::vector<int> small_off, small_cnt, small_pre;
     int small_next = 0;
     DevProblem* P_dev = nullptr;   // device copy of P (batched launches)
     // batch handle: per-chain handles and the job tables of the batched launches
@@ -560,6 +560,23 @@ void plan_small(mgmc_ctx* h, int l, std::vector<int>& visit, std::vector<int4>& 
         h->small_off.push_back((int)ops.size());
         small_phases(h, l, visit, ops);
         h->small_cnt.push_back((int)ops.size() - h->small_off.back());
+        // places of the normals drawn at the launch's start (see k_cycle_small): the low-rank and
+        // coarsest ones first, then the site normals of the smallest grids, while they fit
+        int pre = 0;
+        for (int pass = 0; pass < 2; ++pass)
+            for (size_t q = (size_t)h->small_off.back(); q < ops.size(); ++q) {
+                int4& op = ops[q];
+                const int n = h->fp32() ? h->lf[op.y].n : h->ld[op.y].n;
+                const int rad = h->fp32() ? h->lf[op.y].rad : h->ld[op.y].rad;
+                int need = 0;
+                if (pass == 0 && op.x == kOpLowrank && h->m > 0 && (op.w & 3) != 2) need = h->m;
+                if (pass == 0 && op.x == kOpCoarsest && h->gain) need = h->n0;
+                if (pass == 1 && op.x == kOpSweep && !h->fp32() && rad == 2 && n <= kSmallPreN) need = n * n;
+                if (need == 0 || pre + need > kSmallMaxPre) continue;
+                op.w |= (pre + 1) << 8;
+                pre += need;
+            }
+        h->small_pre.push_back(pre);
         return;
     }
     ++visit[(size_t)l];
@@ -580,8 +597,8 @@ void enqueue_level(mgmc_ctx* h, int l, std::vector<int>& visit, cudaStream_t s, 
     if (l <= h->small_top) {
         // this visit's phase list (built at creation in the same visit order)
         const int k = h->small_next++;
-        launch_cycle_small<T>((const DevLevel<T>*)h->levels_dev, h->small_top, P, h->chol, h->n0,
-                              h->small_ops + h->small_off[k], h->small_cnt[k], h->small_z, s, launches);
+        launch_cycle_small<T>((const DevLevel<T>*)h->levels_dev, h->small_top, P, h->chol, h->gain, h->n0,
+                              h->small_ops + h->small_off[k], h->small_cnt[k], h->small_pre[k], h->small_z, s, launches);
         return;
     }
     const int v = visit[(size_t)l]++;
@@ -943,6 +960,9 @@ mgmc_status mgmc_create(const mgmc_config* cfg_in, const mgmc_allocator* alloc, 
         for (int l = 0; l < h->L && l < kSmallMaxLevels; ++l)
             if (hp.lev[l].n <= thr) h->small_top = l;
         if (h->small_top >= 1) {
+            if (!hp.gain0.empty()) h->gain = upload(h, hp.gain0, st);
+            const cudaError_t e = h->fp32() ? cycle_small_prepare<float>() : cycle_small_prepare<double>();
+            if (e != cudaSuccess) return cleanup(fail(MGMC_ERR_CUDA, "small-grid kernel set-up failed"));
             std::vector<int> visit((size_t)h->L, 0);
             std::vector<int4> ops;
             plan_small(h, h->L - 1, visit, ops);

@@ -128,6 +128,15 @@ __device__ __forceinline__ void draw25_pair(const DevLevel<double>& L, const Cyc
     if (i0 + 2 < n) zb[(long long)j * n + i0 + 2] = z1;
 }
 
+// draw25_pair's sites set to zero (no noise)
+__device__ __forceinline__ void zero25_pair(const DevLevel<double>& L, double* zb, int item)
+{
+    const int nq = (L.n + 3) >> 2, rq = item >> 1, i0 = 4 * (rq % nq) + (item & 1), j = rq / nq;
+    if (i0 >= L.n) return;
+    zb[j * L.n + i0] = 0.0;
+    if (i0 + 2 < L.n) zb[j * L.n + i0 + 2] = 0.0;
+}
+
 __device__ __forceinline__ void sweep25_site(const DevLevel<double>& L, const CycleState& cs, int colour,
                                              unsigned slot, long long t)
 {
@@ -204,6 +213,28 @@ __device__ void coarsest_slot_body(const DevLevel<T>& L, const DevProblem& P, co
     }
 }
 
+// The same sample as one product with the rows of the gain matrix [A~_0^-1 | A~_0^-1 B_0 Gamma^-1 |
+// L_0^-T], eight lanes a row; zc: the standard normals, vec: scratch of 2 n0 + m doubles
+template <typename T>
+__device__ void coarsest_gain_body(const DevLevel<T>& L, int m, const double* gain, int n0, const double* zc, double* vec)
+{
+    const int n = L.n, len = 2 * n0 + m;
+    for (int s = threadIdx.x; s < len; s += blockDim.x)
+        vec[s] = s < n0 ? (L.f ? (double)L.f[site_offset(2, L.pitch, L.plane, L.base, s % n, s / n, 0)] : 0.0)
+                        : (s < n0 + m ? L.d[s - n0] : zc[s - n0 - m]);
+    __syncthreads();
+    for (int q = threadIdx.x; q < ((8 * n0 + 31) & ~31); q += blockDim.x) {
+        const int s = q >> 3, p = q & 7;
+        double acc = 0.0;
+        if (s < n0)
+            for (int t = p; t < len; t += 8) acc = fma(gain[s * len + t], vec[t], acc);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 4);
+        if (p == 0 && s < n0) L.x[site_offset(2, L.pitch, L.plane, L.base, s % n, s / n, 0)] = (T)acc;
+    }
+}
+
 template <typename T>
 __global__ void k_coarsest_slot(DevLevel<T> L, DevProblem P, const double* __restrict__ chol, int n0,
                                 unsigned slot)
@@ -263,14 +294,15 @@ __device__ __forceinline__ T prolong_site(const DevLevel<T>& C, int fi, int fj, 
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ void lowrank_v_body(const DevLevel<T>& L, const DevProblem& P, const CycleState& cs,
-                                               int dir, unsigned slot, int want_dnext, double* z, double* zp)
+                                               int dir, unsigned slot, int want_dnext, double* z, double* zp,
+                                               const double* drawn = nullptr)
 {
     const int m = P.m;
     for (int k = threadIdx.x; k < m; k += blockDim.x) {
         double acc = 0.0;
         for (int t = L.bcol_ptr[k]; t < L.bcol_ptr[k + 1]; ++t) acc += L.bcol_w[t] * (double)L.x[L.bcol_site[t]];
         z[k] = acc;
-        zp[k] = (dir >= 0 && cs.noise) ? lowrank_normal<T>(cs, L.level, slot, k) : 0.0;
+        zp[k] = (dir >= 0 && cs.noise) ? (drawn ? drawn[k] : lowrank_normal<T>(cs, L.level, slot, k)) : 0.0;
     }
     __syncthreads();
     for (int k = threadIdx.x; k < m; k += blockDim.x) {
@@ -404,18 +436,120 @@ __global__ void k_prolong(DevLevel<T> C, DevLevel<T> F)
 // visit of grid `top` -- with the V- or W-cycle recursion below it, in the order and
 // with the noise slots of the per-launch path -- and the CTA runs them one after the
 // other, a barrier after each phase (and between colours).  Every phase evaluates the
-// per-site functions of the per-launch kernels (the two agree to rounding: the compiler
-// may contract their multiply-adds differently); one launch replaces the hundreds of
-// small launches the coarse visits of a W-cycle need.
+// per-site operations of the per-launch kernels (the two agree to rounding); one launch
+// replaces the hundreds of small launches the coarse visits of a W-cycle need.
+//
+// What bounds it: a W-cycle visits the smallest grids most often (a 63^2 visit: 840 phases,
+// three quarters of them on 7^2 and 3^2), so the latency of a phase of a few sites, which is
+// memory latency and the chain of FP64 instructions (about 70 cycles each, not overlapping
+// inside a warp).  Hence
+//  - the fields of the grids 0..s_top (15^2 and below) live in shared memory for the whole
+//    launch: their descriptors' pointers are redirected to the copies, low-rank data and
+//    d_l included where they fit;
+//  - a 25-point site of a small grid is summed by up to eight lanes (three products and
+//    three additions instead of 24 products in a row), as many as keep one warp per
+//    scheduler busy;
+//  - the low-rank and coarsest normals of all phases and the site normals of grids <= 7^2
+//    are drawn in one parallel phase at the start;
+//  - the coarsest sample is the product with the gain matrix (setup.hpp).
+// Measured (GB300, 255^2, squared operator): W-cycle 3524 -> 2532 us (two of these launches).
 // ---------------------------------------------------------------------------
-// The descriptors of grids 0..top and (up to kSmallMaxOps) the phase list are staged in
-// shared memory first, so that a phase's data loads do not wait on two dependent global
-// loads (the phase, then the descriptor fields) each time.
+// one 25-point site by LPS lanes (consecutive lanes of a warp; the group's first lane
+// has the result): x_i <- (f_i + sqrt(a_ii) z - sum_{j != i} a_ij x_j) / a_ii
+template <int LPS>
+__device__ __forceinline__ double update25_lanes(const DevLevel<double>& L, long long e, double z, int lane, bool on)
+{
+    double acc = 0.0;
+    if (on) {
+        if (lane == 0) acc = fma(L.isq[L.alloc + e], z, L.f ? L.f[e] : 0.0);
+#pragma unroll
+        for (int q = 0; q < 24 / LPS; ++q) {
+            const int t = lane + LPS * q, o = t + (t >= 12 ? 1 : 0);
+            acc = fma(-coef25_at(L, e, o), L.x[e + off25(o, L.pitch)], acc);
+        }
+    }
+#pragma unroll
+    for (int s = 1; s < LPS; s <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
+    return on ? acc * L.isq[e] : 0.0;
+}
+
+// the sites of one colour, LPS lanes each; z(i, j): the site's normal
+template <int LPS, typename Z>
+__device__ __forceinline__ void colour25(const DevLevel<double>& L, int c, Z&& z)
+{
+    const int sites = (int)colour25_sites(L.n, c);
+    const int lane = threadIdx.x & (LPS - 1);
+    for (int t0 = 0; t0 < sites; t0 += blockDim.x / LPS) {
+        const int t = t0 + threadIdx.x / LPS;
+        // whole warps stay together for the shuffles
+        if (t0 + (int)(threadIdx.x & ~31u) / LPS >= sites) break;
+        const bool on = t < sites;
+        int i = 0, j = 0;
+        if (on) colour25_site(L.n, c, t, i, j);
+        const long long e = site_offset(2, L.pitch, L.plane, L.base, i, j, 0);
+        const double x = update25_lanes<LPS>(L, e, on && lane == 0 ? z(i, j) : 0.0, lane, on);
+        if (on && lane == 0) L.x[e] = x;
+    }
+}
+
+// r = f - A x of a 25-point grid, LPS lanes per site
+template <int LPS>
+__device__ __forceinline__ void residual25(const DevLevel<double>& L)
+{
+    const int N = L.n * L.n, lane = threadIdx.x & (LPS - 1);
+    for (int t0 = 0; t0 < N; t0 += blockDim.x / LPS) {
+        const int t = t0 + threadIdx.x / LPS;
+        if (t0 + (int)(threadIdx.x & ~31u) / LPS >= N) break;
+        const bool on = t < N;
+        const long long e = on ? site_offset(2, L.pitch, L.plane, L.base, t % L.n, t / L.n, 0) : 0;
+        double acc = 0.0;
+        if (on) {
+            if (lane == 0) acc = fma(-L.coef[e], L.x[e], L.f ? L.f[e] : 0.0);
+#pragma unroll
+            for (int q = 0; q < 24 / LPS; ++q) {
+                const int u = lane + LPS * q, o = u + (u >= 12 ? 1 : 0);
+                acc = fma(-coef25_at(L, e, o), L.x[e + off25(o, L.pitch)], acc);
+            }
+        }
+#pragma unroll
+        for (int s = 1; s < LPS; s <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
+        if (on && lane == 0) L.res[e] = acc;
+    }
+}
+
+// a global array's copy in the shared arena (16-byte granules); NULL when it does not fit
+struct Arena {
+    unsigned char* base;
+    unsigned used, size;
+    template <typename V>
+    __device__ __forceinline__ V* take(long long count)
+    {
+        const unsigned bytes = (unsigned)((count * sizeof(V) + 15) / 16 * 16);
+        if (used + bytes > size) return nullptr;
+        V* p = reinterpret_cast<V*>(base + used);
+        used += bytes;
+        return p;
+    }
+};
+// redirect `ptr` to a copy in the arena (kept in global memory when it does not fit)
+template <typename V>
+__device__ __forceinline__ void to_shared(Arena& ar, V*& ptr, long long count)
+{
+    if (!ptr) return;
+    using M = typename std::remove_const<V>::type;
+    M* p = ar.take<M>(count);
+    if (!p) return;
+    for (long long q = threadIdx.x; q < count; q += blockDim.x) p[q] = ptr[q];
+    ptr = p;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kSmallCycleThreads)
     k_cycle_small(const DevLevel<T>* __restrict__ lv_g, int top, DevProblem P, const double* __restrict__ chol,
-                  int n0, const int4* __restrict__ ops_g, int n_ops, double* __restrict__ zb)
+                  const double* __restrict__ gain_g, int n0, const int4* __restrict__ ops_g, int n_ops, int n_pre,
+                  unsigned arena_bytes, double* __restrict__ zb)
 {
+    extern __shared__ __align__(16) unsigned char smem_dyn[];
     __shared__ double r[MGMC_MAX_COARSEST];
     __shared__ double g[kMaxObs];
     __shared__ double z[kMaxObs];
@@ -433,35 +567,117 @@ __global__ void __launch_bounds__(kSmallCycleThreads)
     __syncthreads();
     const CycleState cs = *P.cs;
     const int m = P.m;
+    auto op_at = [&](int q) { return q < kSmallMaxOps ? ops_s[q] : ops_g[q]; };
+    // the pre-drawn normals, then the copies of the small grids' arrays
+    Arena ar{smem_dyn, 0u, arena_bytes};
+    double* const pre = ar.take<double>(n_pre);
+    const double* gain = gain_g;
+    T* top_x = lv[top].x;   // the visit's result goes back here
+    __syncthreads();
+    {
+        // the same pointers in every thread: each keeps its own view, thread 0 stores it
+        for (int l = 0; l <= top; ++l) {
+            DevLevel<T> L = lv[l];
+            if (L.n > kSmallSharedN) break;
+            // all of a grid's fields or none
+            const unsigned mark = ar.used;
+            const long long fields = 3 + (L.coef ? L.ncoef : 0) + (L.diag ? 1 : 0) + (L.isq ? 2 : 0);
+            if (mark + fields * ((L.alloc * sizeof(T) + 15) / 16 * 16) > ar.size) break;
+            const long long cf = L.coef ? L.ncoef * L.alloc : 0;
+            to_shared(ar, L.x, L.alloc);
+            to_shared(ar, L.f, L.alloc);
+            if (L.res) to_shared(ar, L.res, L.alloc);
+            to_shared(ar, L.coef, cf);
+            to_shared(ar, L.diag, L.alloc);
+            to_shared(ar, L.isq, 2 * L.alloc);
+            __syncthreads();
+            if (threadIdx.x == 0) lv[l] = L;
+            __syncthreads();
+        }
+        if (gain && n0 <= 16) to_shared(ar, gain, (long long)n0 * (2 * n0 + m));
+        if (m > 0) {
+            for (int l = 0; l <= top; ++l) {
+                DevLevel<T> L = lv[l];
+                if (L.n > kSmallSharedN) break;
+                const int nnz = L.bcol_ptr[m];
+                to_shared(ar, L.bcol_site, nnz);
+                to_shared(ar, L.bcol_w, nnz);
+                to_shared(ar, L.bcol_ptr, m + 1);
+                if (l < top) to_shared(ar, L.d, m);
+                if (L.lrv) to_shared(ar, L.lrv, 2 * m);
+                to_shared(ar, L.BtG, (long long)m * m);
+                for (int dir = 0; dir < 2; ++dir) {
+                    to_shared(ar, L.g_site[dir], L.g_rows[dir]);
+                    to_shared(ar, L.g_val[dir], (long long)L.g_rows[dir] * m);
+                }
+                __syncthreads();
+                if (threadIdx.x == 0) lv[l] = L;
+                __syncthreads();
+            }
+            if (threadIdx.x == 0)
+                for (int l = 1; l <= top; ++l) lv[l].dnext = lv[l - 1].d;
+        }
+    }
+    // the normals that do not depend on the state: phase q's at pre + (flags >> 8), one pair per item
     for (int q = 0; q < n_ops; ++q) {
-        const int4 op = q < kSmallMaxOps ? ops_s[q] : ops_g[q];
+        const int4 op = op_at(q);
+        const int off = (op.w >> 8) - 1;
+        if (off < 0) continue;
+        const DevLevel<T>& L = lv[op.y];
+        if (op.x == kOpLowrank) {
+            for (int k = (threadIdx.x + 32 * q) % blockDim.x; k < m; k += blockDim.x)
+                pre[off + k] = cs.noise ? lowrank_normal<T>(cs, L.level, (unsigned)op.z, k) : 0.0;
+        } else if (op.x == kOpCoarsest) {
+            for (int s = (threadIdx.x + 32 * q) % blockDim.x; 2 * s < n0; s += blockDim.x) {
+                double z0 = 0.0, z1 = 0.0;
+                if (cs.noise) draw_pair<double>(cs, (unsigned)s, 2u, 0, (unsigned)op.z, z0, z1);
+                pre[off + 2 * s] = z0;
+                if (2 * s + 1 < n0) pre[off + 2 * s + 1] = z1;
+            }
+        } else if constexpr (std::is_same<T, double>::value) {
+            const int items = L.n * ((L.n + 3) >> 2) * 2;
+            for (int it = (threadIdx.x + 32 * q) % blockDim.x; it < items; it += blockDim.x) {
+                if (cs.noise)
+                    draw25_pair(L, cs, (unsigned)op.z, pre + off, it);
+                else
+                    zero25_pair(L, pre + off, it);
+            }
+        }
+    }
+    __syncthreads();
+    for (int q = 0; q < n_ops; ++q) {
+        const int4 op = op_at(q);
         const DevLevel<T>& L = lv[op.y];
         const long long N = (long long)L.n * L.n;
+        const int off = (op.w >> 8) - 1;   // pre-drawn normals, or -1
         switch (op.x) {
         case kOpSweep: {
             const unsigned slot = (unsigned)op.z;
-            const int dir = op.w;
+            const int dir = op.w & 1;
             const int nq = (L.n + 3) >> 2;
             bool done = false;
             if constexpr (std::is_same<T, double>::value) {
                 if (L.rad == 2) {
                     // the sweep's normals first, for all sites at once (one draw per pair), then
                     // the nine classes read them: the colour phases carry no Box-Muller transform
-                    if (cs.noise) {
+                    const double* zs = off >= 0 ? pre + off : zb;
+                    if (off < 0 && cs.noise) {
                         const long long items = (long long)L.n * nq * 2;
                         for (long long it = threadIdx.x; it < items; it += blockDim.x) draw25_pair(L, cs, slot, zb, it);
                         __syncthreads();
                     }
+                    const bool have = off >= 0 || cs.noise;
+                    auto zz = [&](int i, int j) { return have ? zs[(long long)j * L.n + i] : 0.0; };
+                    // lanes per site: sites x lanes near 128, one warp per scheduler
+                    const int lps = L.n <= 7 ? 8 : L.n <= 15 ? 4 : 1;
                     for (int ci = 0; ci < 9; ++ci) {
                         const int c = dir == 0 ? ci : 8 - ci;
-                        const long long sites = colour25_sites(L.n, c);
-                        for (long long t = threadIdx.x; t < sites; t += blockDim.x) {
-                            int i, j;
-                            colour25_site(L.n, c, t, i, j);
-                            const double zz = cs.noise ? zb[(long long)j * L.n + i] : 0.0;
-                            const long long e = site_offset(2, L.pitch, L.plane, L.base, i, j, 0);
-                            L.x[e] = update25(L, e, zz);
-                        }
+                        if (lps == 8)
+                            colour25<8>(L, c, zz);
+                        else if (lps == 4)
+                            colour25<4>(L, c, zz);
+                        else
+                            colour25<1>(L, c, zz);
                         __syncthreads();
                     }
                     done = true;
@@ -477,9 +693,8 @@ __global__ void __launch_bounds__(kSmallCycleThreads)
                     __syncthreads();
                 }
             } else {
-                const int seq2[4] = {0, 3, 2, 1};
                 for (int ci = 0; ci < 4; ++ci) {
-                    const int c = seq2[dir == 0 ? ci : 3 - ci];
+                    const int c = (int)((0x1230u >> (4 * (dir == 0 ? ci : 3 - ci))) & 0xFu);   // 0, 3, 2, 1
                     const int py = (c >> 1) & 1;
                     const long long items = (long long)((L.n - py + 1) / 2) * nq;
                     for (long long it = threadIdx.x; it < items; it += blockDim.x)
@@ -493,18 +708,29 @@ __global__ void __launch_bounds__(kSmallCycleThreads)
             if (m == 0) break;
             const int dir = (op.w & 3) == 2 ? -1 : (op.w & 3);
             const int dn = (op.w >> 2) & 1;
-            lowrank_v_body<T>(L, P, cs, dir, (unsigned)op.z, dn, z, zp);
+            lowrank_v_body<T>(L, P, cs, dir, (unsigned)op.z, dn, z, zp, off >= 0 ? pre + off : nullptr);
             __syncthreads();
             if (dir >= 0) {
-                for (int k = threadIdx.x; k < m; k += blockDim.x) zp[k] = L.lrv[k];
-                __syncthreads();
-                lowrank_rows<T>(L, m, dir, zp, threadIdx.x, blockDim.x);
-                if (dn) lowrank_dnext<T>(L, m, zp);
+                lowrank_rows<T>(L, m, dir, L.lrv, threadIdx.x, blockDim.x);
+                if (dn) lowrank_dnext<T>(L, m, L.lrv);
             }
             break;
         }
         case kOpRestrict: {
-            for (long long s2 = threadIdx.x; s2 < N; s2 += blockDim.x) residual_site<T, 2>(L, s2);
+            bool done = false;
+            if constexpr (std::is_same<T, double>::value) {
+                if (L.rad == 2) {
+                    if (L.n <= 3)
+                        residual25<8>(L);
+                    else if (L.n <= 7)
+                        residual25<2>(L);
+                    else
+                        residual25<1>(L);
+                    done = true;
+                }
+            }
+            if (!done)
+                for (long long s2 = threadIdx.x; s2 < N; s2 += blockDim.x) residual_site<T, 2>(L, s2);
             __syncthreads();
             const DevLevel<T>& C = lv[op.y - 1];
             const long long Nc = (long long)C.n * C.n;
@@ -515,7 +741,10 @@ __global__ void __launch_bounds__(kSmallCycleThreads)
             for (long long e = threadIdx.x; e < L.alloc; e += blockDim.x) L.x[e] = T(0);
             break;
         case kOpCoarsest:
-            coarsest_slot_body<T>(lv[0], P, cs, chol, n0, (unsigned)op.z, r, g);
+            if (gain && off >= 0)
+                coarsest_gain_body<T>(lv[0], m, gain, n0, pre + off, r);
+            else
+                coarsest_slot_body<T>(lv[0], P, cs, chol, n0, (unsigned)op.z, r, g);
             break;
         case kOpProlong: {
             const DevLevel<T>& C = lv[op.y - 1];
@@ -527,6 +756,9 @@ __global__ void __launch_bounds__(kSmallCycleThreads)
         }
         __syncthreads();
     }
+    const DevLevel<T>& L = lv[top];
+    if (L.x != top_x)
+        for (long long e = threadIdx.x; e < L.alloc; e += blockDim.x) top_x[e] = L.x[e];
 }
 
 __global__ void k_set_cycle(CycleState* cs, unsigned long long seed, unsigned long long cycle, unsigned chain,
@@ -740,10 +972,18 @@ void launch_coarsest_slot(const DevLevel<T>& L, const DevProblem& P, const doubl
 }
 
 template <typename T>
-void launch_cycle_small(const DevLevel<T>* levels_dev, int top, const DevProblem& P, const double* chol, int n0,
-                        const int4* ops, int n_ops, double* zb, cudaStream_t st, int& launches)
+cudaError_t cycle_small_prepare()
 {
-    k_cycle_small<T><<<1, kSmallCycleThreads, 0, st>>>(levels_dev, top, P, chol, n0, ops, n_ops, zb);
+    return cudaFuncSetAttribute(k_cycle_small<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallArena);
+}
+
+template <typename T>
+void launch_cycle_small(const DevLevel<T>* levels_dev, int top, const DevProblem& P, const double* chol,
+                        const double* gain, int n0, const int4* ops, int n_ops, int n_pre, double* zb, cudaStream_t st,
+                        int& launches)
+{
+    k_cycle_small<T><<<1, kSmallCycleThreads, kSmallArena, st>>>(levels_dev, top, P, chol, gain, n0, ops, n_ops, n_pre,
+                                                                 (unsigned)kSmallArena, zb);
     ++launches;
 }
 
@@ -797,8 +1037,9 @@ void launch_resid(const DevLevel<T>& L, const DevProblem& P, double* u, double* 
     template void launch_prolong<T>(const DevLevel<T>&, const DevLevel<T>&, cudaStream_t, int&);                 \
     template void launch_coarsest_slot<T>(const DevLevel<T>&, const DevProblem&, const double*, int, unsigned,     \
                                           cudaStream_t, int&);                                                   \
-    template void launch_cycle_small<T>(const DevLevel<T>*, int, const DevProblem&, const double*, int,            \
-                                        const int4*, int, double*, cudaStream_t, int&);                          \
+    template cudaError_t cycle_small_prepare<T>();                                                                \
+    template void launch_cycle_small<T>(const DevLevel<T>*, int, const DevProblem&, const double*, const double*,  \
+                                        int, const int4*, int, int, double*, cudaStream_t, int&);                \
     template void launch_pack<T>(const DevLevel<T>&, T*, bool, cudaStream_t);                               \
     template void launch_pack_batch<T>(const PackJob<T>*, void* const*, int, int, bool, cudaStream_t);         \
     template void launch_resid<T>(const DevLevel<T>&, const DevProblem&, double*, double*, int, double*,         \

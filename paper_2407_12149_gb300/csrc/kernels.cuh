@@ -23,10 +23,20 @@ enum { kOpSweep = 0, kOpLowrank = 1, kOpRestrict = 2, kOpZero = 3, kOpCoarsest =
 constexpr int kSmallCycleThreads = 512;
 constexpr int kSmallMaxLevels = 16;   // grids 0..top held by the kernel (top < 16)
 constexpr int kSmallMaxOps = 1024;    // phases staged in shared memory (later ones read from global)
-// zb: scratch of n^2 doubles for the largest 25-point grid held (the normals of a sweep)
+constexpr int kSmallSharedN = 15;     // grids up to this size live in shared memory
+constexpr int kSmallPreN = 7;         // grids up to this size have their site normals drawn at the start
+constexpr int kSmallMaxPre = 4096;    // normals drawn at the start, at most
+// dynamic shared memory of the kernel: 227 KB less its static part
+constexpr size_t kSmallArena = 232448 - 36 * 1024;
 template <typename T>
-void launch_cycle_small(const DevLevel<T>* levels_dev, int top, const DevProblem& P, const double* chol, int n0,
-                        const int4* ops, int n_ops, double* zb, cudaStream_t st, int& launches);
+cudaError_t cycle_small_prepare();
+// gain: see setup.hpp (NULL: the coarsest grid is solved with the factor); ops' flags >> 8: 1 + the
+// place of the phase's pre-drawn normals among the n_pre, 0 none.  zb: scratch of n^2 doubles for
+// the largest 25-point grid held (the normals of a sweep)
+template <typename T>
+void launch_cycle_small(const DevLevel<T>* levels_dev, int top, const DevProblem& P, const double* chol,
+                        const double* gain, int n0, const int4* ops, int n_ops, int n_pre, double* zb, cudaStream_t st,
+                        int& launches);
 template <typename T>
 void launch_prolong(const DevLevel<T>& C, const DevLevel<T>& F, cudaStream_t st, int& launches);
 // shared-memory plan of the coarse kernel (coarse.cu), offsets in elements of the path precision
