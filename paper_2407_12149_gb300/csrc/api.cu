@@ -272,7 +272,7 @@ mgmc_status build_device_levels(mgmc_ctx* h, const HostProblem& hp)
             }
             D.coef = upload(h, coef, st);
         }
-        if (sizeof(T) == 8 && (R == 2 || l <= h->top)) {
+        if (sizeof(T) == 8) {
             std::vector<T> aux((size_t)D.alloc * 2, T(0));
             for (long long s2 = 0; s2 < HL.N; ++s2) {
                 const long long e = off(s2);

@@ -64,9 +64,8 @@ struct DevLevel {
     // the squared shifted Laplacian: offsets o = (dx+2) + 5 (dy+2), centre 12, slot t >= 1
     // = a(i, i + o_{12+t}); two halo rows and columns around the interior)
     int rad;
-    // FP64 25-point grids and the grids inside the coarse kernel: 1 / a_ii at [e] and
-    // sqrt(a_ii) at [alloc + e] (rounded once from FP64 on the host), so that a site update
-    // needs neither a division nor a square root
+    // FP64: 1 / a_ii at [e] and sqrt(a_ii) at [alloc + e] (correctly rounded on the host), so
+    // that a site update needs neither a division nor a square root
     const T* isq;
     // B_l rows grouped by grid row (finest level; used by the residual norm)
     const int* brow_ptr;    // [n^(dim-1) + 1]

@@ -2,7 +2,7 @@
 // residual and the grid transfers, shared by all sweep kernels.
 //
 // FP64 uses the plain form x_i <- (f_i + xi_i - sum_{j != i} a_ij x_j) / a_ii
-// (Alg. 3 as a colour-ordered Gauss-Seidel sweep).  FP32 uses the algebraically
+// (Alg. 3 as a colour-ordered Gauss-Seidel sweep; 1/a_ii and sqrt(a_ii) come from the host).  FP32 uses the algebraically
 // identical correction form x_i <- x_i + (f_i + xi_i - (A x)_i) / a_ii (1/a_ii and
 // sqrt(a_ii) from one reciprocal square root) with
 // (A x)_i = rowsum_i x_i + sum_{j != i} a_ij (x_j - x_i): in single precision
@@ -76,10 +76,9 @@ template <int DIM>
 __device__ __forceinline__ double fine_update(const DevLevel<double>& L, long long e, double z)
 {
     const double* x = L.x;
-    double aii = L.diag[e];
     double w = L.woff;
     double acc = L.f ? L.f[e] : 0.0;
-    acc += sqrt(aii) * z;
+    acc += L.isq[L.alloc + e] * z;
     // neighbours in the order (0,0,-1), (0,-1,0), (-1,0,0), (1,0,0), (0,1,0), (0,0,1)
     if (DIM == 3) acc += w * x[e - L.plane];
     acc += w * x[e - L.pitch];
@@ -87,7 +86,7 @@ __device__ __forceinline__ double fine_update(const DevLevel<double>& L, long lo
     acc += w * x[e + 1];
     acc += w * x[e + L.pitch];
     if (DIM == 3) acc += w * x[e + L.plane];
-    return acc / aii;
+    return acc * L.isq[e];
 }
 
 template <int DIM>
@@ -112,15 +111,14 @@ __device__ __forceinline__ double coarse_update(const DevLevel<double>& L, long 
 {
     constexpr int NS = Offsets<DIM>::NS;
     constexpr int C = Offsets<DIM>::C;
-    double aii = L.coef[e];
     double acc = L.f ? L.f[e] : 0.0;
-    acc += sqrt(aii) * z;
+    acc += L.isq[L.alloc + e] * z;
 #pragma unroll
     for (int o = 0; o < NS; ++o) {
         if (o == C) continue;
         acc -= coef_at<DIM>(L, e, o) * L.x[e + off_of<DIM>(o, L.pitch, L.plane)];
     }
-    return acc / aii;
+    return acc * L.isq[e];
 }
 
 template <int DIM>

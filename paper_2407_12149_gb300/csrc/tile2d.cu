@@ -69,7 +69,12 @@ struct TileGeom {
     static constexpr int PAD = (sizeof(T) == 4 && !FINE) ? (BWD ? 12 : 4) : 0;
     static constexpr int SX = SW + PAD;
     static constexpr int SY = TY + 2 * R;
-    static constexpr int NCOEF = FINE ? 1 : 5;
+    // operator fields: a_ii (5-point) or the 5 coefficient slots; FP64 adds 1 / a_ii and
+    // sqrt(a_ii) from the host: an FP64 division and square root are about 20 of the 50 FP64
+    // instructions of a site, and FP64 issues at 1/64 of the FP32 rate (1023^2 FP64 chain, 2 cycles
+    // 1341 -> 1025 us; 9 instead of 7 fields leave two CTAs per SM on the 9-point grids)
+    static constexpr int NST = FINE ? 1 : 5;
+    static constexpr int NCOEF = NST + (sizeof(T) == 8 ? 2 : 0);
     static constexpr int NFLD = 1 + NCOEF + (FINE ? 0 : 1);  // x, coefficients, fdense
     // field stride in elements: every field (a TMA destination) starts on 128 bytes
     static constexpr int FS = (SX * SY * (int)sizeof(T) + 127) / 128 * 128 / (int)sizeof(T);
@@ -85,9 +90,9 @@ struct TileGeom {
     static constexpr int PSZ = (PXA * PY * (int)sizeof(T) + 127) / 128 * 128 / (int)sizeof(T);
     // tensor maps: x source, coefficient fields, fdense (9-point), psi (backward)
     static constexpr int NMAP = NFLD + (BWD ? 1 : 0);
-    // stage buffers: two on the 5-point grid (tile k + 1 is copied while tile k is
-    // computed), one on the 9-point grids (7 fields; three CTAs per SM overlap instead)
-    static constexpr int NSTAGE = FINE ? 2 : 1;
+    // stage buffers: two on the FP32 5-point grid (tile k + 1 is copied while tile k is
+    // computed), one elsewhere (4 to 9 fields; two or three CTAs per SM overlap instead)
+    static constexpr int NSTAGE = (FINE && sizeof(T) == 4) ? 2 : 1;
     static constexpr int STAGE = NFLD * FS + (BWD ? PSZ : 0);  // elements per stage buffer
     // single-stage backward kernels keep a second state buffer: the next tile's state
     // is copied into it while the current tile still stores its own
@@ -103,17 +108,16 @@ struct TileGeom {
 namespace {
 
 // --- per-site arithmetic on the staged tile (same operations as stencil.cuh) ---
+// FP64: iv, sq = 1 / a_ii, sqrt(a_ii) of the site
 template <int SX>
-__device__ __forceinline__ double upd_fine(const double* X, const double* C0, int l, double w, double z)
+__device__ __forceinline__ double upd_fine(const double* X, int l, double w, double z, double iv, double sq)
 {
-    double aii = C0[l];
-    double acc = 0.0;
-    acc += sqrt(aii) * z;
+    double acc = sq * z;
     acc += w * X[l - SX];
     acc += w * X[l - 1];
     acc += w * X[l + 1];
     acc += w * X[l + SX];
-    return acc / aii;
+    return acc * iv;
 }
 
 template <int SX>
@@ -150,17 +154,17 @@ __device__ __forceinline__ float coef9(const float* Cf, int l, int o)
 }
 
 template <int SX, int SXY>
-__device__ __forceinline__ double upd_9(const double* X, const double* Cf, const double* F, int l, double z)
+__device__ __forceinline__ double upd_9(const double* X, const double* Cf, const double* F, int l, double z, double iv,
+                                        double sq)
 {
-    double aii = Cf[l];
     double acc = F[l];
-    acc += sqrt(aii) * z;
+    acc += sq * z;
 #pragma unroll
     for (int o = 0; o < 9; ++o) {
         if (o == 4) continue;
         acc -= coef9<SX, SXY>(Cf, l, o) * X[l + noff<SX>(o)];
     }
-    return acc / aii;
+    return acc * iv;
 }
 
 template <int SX, int SXY>
@@ -402,12 +406,14 @@ __device__ __forceinline__ void tile_phase(const DevLevel<T>& L, const CycleStat
                                             v0, v1);
         } else {
             const int l0 = (dy + G::R) * SX + (dx0 + G::RX);
-            if (FINE) {
-                if (v0) X[l0] = upd_fine<SX>(X, Cf, l0, L.woff, z0);
-                if (v1) X[l0 + 2] = upd_fine<SX>(X, Cf, l0 + 2, L.woff, z1);
+            const T* iv = Cf + G::NST * SXY;   // 1 / a_ii, then sqrt(a_ii)
+            const T* sq = iv + SXY;
+            if constexpr (FINE) {
+                if (v0) X[l0] = upd_fine<SX>(X, l0, L.woff, z0, iv[l0], sq[l0]);
+                if (v1) X[l0 + 2] = upd_fine<SX>(X, l0 + 2, L.woff, z1, iv[l0 + 2], sq[l0 + 2]);
             } else {
-                if (v0) X[l0] = upd_9<SX, SXY>(X, Cf, F, l0, z0);
-                if (v1) X[l0 + 2] = upd_9<SX, SXY>(X, Cf, F, l0 + 2, z1);
+                if (v0) X[l0] = upd_9<SX, SXY>(X, Cf, F, l0, z0, iv[l0], sq[l0]);
+                if (v1) X[l0 + 2] = upd_9<SX, SXY>(X, Cf, F, l0 + 2, z1, iv[l0 + 2], sq[l0 + 2]);
             }
         }
     }
@@ -1136,10 +1142,12 @@ bool make_maps(const DevLevel<T>& L, const DevLevel<T>& C, TileMaps* out)
     if (FINE) {
         ok = ok && encode_field<T>(&out->m[1], L.diag, L.pitch, rows, G::SX, G::SY);
     } else {
-        for (int t = 0; t < G::NCOEF; ++t)
+        for (int t = 0; t < G::NST; ++t)
             ok = ok && encode_field<T>(&out->m[1 + t], L.coef + (long long)t * L.alloc, L.pitch, rows, G::SX, G::SY);
         ok = ok && encode_field<T>(&out->m[1 + G::NCOEF], L.f, L.pitch, rows, G::SX, G::SY);
     }
+    for (int t = G::NST; t < G::NCOEF; ++t)
+        ok = ok && encode_field<T>(&out->m[1 + t], L.isq + (long long)(t - G::NST) * L.alloc, L.pitch, rows, G::SX, G::SY);
     if (BWD) ok = ok && encode_field<T>(&out->m[G::NFLD], C.x, C.pitch, C.n + 2, G::PXA, G::PY);
     return ok;
 }

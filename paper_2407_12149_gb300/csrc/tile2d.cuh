@@ -19,7 +19,7 @@ struct TileJob {
 };
 // TMA descriptors of one tile job: the state source, the operator fields, the
 // dense right-hand side (9-point grids) and, backward, the coarse psi
-constexpr int kTileMaxMaps = 8;
+constexpr int kTileMaxMaps = 10;
 struct TileMaps {  // CUtensorMap is 64-byte aligned
     CUtensorMap m[kTileMaxMaps];
 };
