@@ -116,6 +116,7 @@ struct mgmc_ctx {
     double* gain = nullptr;
     double* e0 = nullptr;
     bool fused = false;   // 2D, nu1 = nu2 = 1: fused tile kernels on the grids above coarse_max_n
+    bool gibbs_fused = false; // 2D Gibbs sampler, nu1 = nu2 = 1: the finest grid's fused sweep kernels
     bool recursive = false;   // W-cycle or radius-2 grids: general kernels, cycle enqueued recursively
     // recursive path, 2D: grids 0..small_top run in one k_cycle_small launch per visit of
     // grid small_top (-1: none); the phase lists of the cycle's visits, in cycle order
@@ -166,6 +167,8 @@ namespace {
 
 template <typename T>
 mgmc_status build_batch_tables(mgmc_ctx* h);
+template <typename T>
+mgmc_status build_gibbs_tables(mgmc_ctx* h);
 void apply_band_min(mgmc_ctx* h);
 
 template <typename T>
@@ -379,6 +382,15 @@ mgmc_status build_device_levels(mgmc_ctx* h, const HostProblem& hp)
             if (hp.m > 0) D.lrv = upload(h, std::vector<double>((size_t)2 * hp.m, 0.0), st);
         }
         if (st != MGMC_OK) return fail(st, "device upload failed");
+    }
+    if (h->gibbs_fused) {   // the state between the two sweeps; no z partials (general low-rank step)
+        DevLevel<T>& D = levels[hp.n_levels - 1];
+        const size_t fbytes = (size_t)D.alloc * sizeof(T);
+        D.x2 = (T*)h->buf.get(fbytes);
+        if (!D.x2) return fail(MGMC_ERR_OOM, "allocator returned NULL");
+        CUDA_TRY(cudaMemsetAsync(D.x2, 0, fbytes, h->buf.stream));
+        const int TX = D.fine ? TileShape<T, true>::TX : TileShape<T, false>::TX;
+        D.ntx = (D.n + TX - 1) / TX;
     }
     // fused tile path: second state buffer, per-tile observation entries, G/H in T, B^T G
     if (h->fused) {
@@ -649,6 +661,30 @@ void enqueue_cycle(mgmc_ctx* h, cudaStream_t s, int& launches)
     const int Lf = h->L - 1;
     const DevProblem& P = h->P;
     const bool prof = h->profile && h->top < Lf;
+    if (h->gibbs_fused) {
+        // the V-cycle's finest-grid kernels: one launch per sweep instead of one per colour.  They
+        // also restrict a residual nobody reads and add the prolongation of a coarse correction
+        // that is zero (nothing writes the coarse state of a Gibbs handle); the low-rank step stays
+        // in the general kernels (G applied in FP64).
+        const DevLevel<T>& D = lv[Lf];
+        DevLevel<T> D2 = D;
+        D2.x = D.x2;
+        for (int dir = 0; dir < 2; ++dir) {
+            if (prof) cudaEventRecordWithFlags(h->ev[2 * dir], s, cudaEventRecordExternal);
+            if (h->stream_fine)
+                launch_stream_fine((const StreamJob*)h->jobs_stream,
+                                   (const StreamMaps*)(dir ? h->maps_sbwd : h->maps_sfwd), h->njob_stream,
+                                   h->stream_strips, h->stream_ctas, dir == 1, s, launches);
+            else
+                launch_tile_batch<T>((const TileJob<T>*)h->jobs_tile[0],
+                                     (const TileMaps*)(dir ? h->maps_bwd[0] : h->maps_fwd[0]), 1, h->per_tile[0],
+                                     h->nblk_tile[0], h->fine0, dir == 1, false, s, launches);
+            if (prof) cudaEventRecordWithFlags(h->ev[2 * dir + 1], s, cudaEventRecordExternal);
+            launch_lowrank<T>(dir ? D : D2, P, dir, (unsigned)dir, false, s, launches);
+        }
+        launch_qoi_batch<T>((const QoiJob<T>*)h->jobs_qoi, 1, h->max_qoi, s, launches);
+        return;
+    }
     if (h->cfg.gibbs) {
         // plain Gibbs sampler (Sec. 5.1.3): the finest grid's sweeps of the V-cycle, no coarse correction
         const DevLevel<T>& D = lv[Lf];
@@ -933,6 +969,7 @@ mgmc_status mgmc_create(const mgmc_config* cfg_in, const mgmc_allocator* alloc, 
     h->n0 = hp.n0;
     h->f_norm = hp.f_norm;
     h->fused = cfg.dim == 2 && cfg.nu1 == 1 && cfg.nu2 == 1 && !cfg.gibbs && !h->recursive;
+    h->gibbs_fused = cfg.dim == 2 && cfg.nu1 == 1 && cfg.nu2 == 1 && cfg.gibbs && !h->recursive;
     auto cleanup = [&](mgmc_status s) {
         h->buf.release();
         delete h;
@@ -1030,6 +1067,10 @@ mgmc_status mgmc_create(const mgmc_config* cfg_in, const mgmc_allocator* alloc, 
         st = h->fp32() ? build_batch_tables<float>(h) : build_batch_tables<double>(h);
         if (st != MGMC_OK) return cleanup(st);
     } else {
+        if (h->gibbs_fused) {
+            st = h->fp32() ? build_gibbs_tables<float>(h) : build_gibbs_tables<double>(h);
+            if (st != MGMC_OK) return cleanup(st);
+        }
         h->max_qoi = h->n_qoi;
         auto job = [&](auto* x) {
             using T = std::remove_pointer_t<decltype(x)>;
@@ -1309,6 +1350,70 @@ void apply_band_min(mgmc_ctx* h)
     for (size_t d = 0; d < h->s9_ok.size(); ++d) h->s9_use[d] = h->s9_ok[d] && h->s9_minn[d] >= band_min;
 }
 
+// the finest grid's FP32 5-point grids of `chains` as streaming jobs
+mgmc_status build_stream_jobs(mgmc_ctx* h, const std::vector<mgmc_ctx*>& chains)
+{
+    mgmc_status st = MGMC_OK;
+    cudaError_t e = stream_prepare();
+    if (e != cudaSuccess) return fail(MGMC_ERR_CUDA, std::string("stream kernel set-up: ") + cudaGetErrorString(e));
+    std::vector<StreamJob> sj;
+    std::vector<StreamMaps> sf, sb;
+    long long strips = 0;
+    for (mgmc_ctx* c : chains) {
+        const int l = c->L - 1;
+        if (l <= c->top) continue;
+        const auto& lv = levels_of<float>(c);
+        StreamJob J{};
+        J.L = lv[l];
+        J.C = lv[l - 1];
+        J.cs = c->cs;
+        J.strip0 = strips;
+        J.spb = (J.L.n + kStreamRows - 1) / kStreamRows;
+        J.nbands = (J.L.n + kStreamBand - 1) / kStreamBand;
+        strips += (long long)J.spb * J.nbands;
+        sj.push_back(J);
+        sf.emplace_back();
+        sb.emplace_back();
+        if (!make_stream_maps(J.L, J.C, false, &sf.back()) || !make_stream_maps(J.L, J.C, true, &sb.back()))
+            return fail(MGMC_ERR_CUDA, "TMA descriptor encoding failed");
+    }
+    h->jobs_stream = upload(h, sj, st);
+    h->maps_sfwd = upload(h, sf, st);
+    h->maps_sbwd = upload(h, sb, st);
+    if (st != MGMC_OK) return fail(st, "stream table upload failed");
+    h->njob_stream = (int)sj.size();
+    h->stream_strips = strips;
+    h->stream_ctas = stream_grid(strips);
+    h->stream_fine = true;
+    return MGMC_OK;
+}
+
+// the sweep kernels' table of a Gibbs handle: its finest grid
+template <typename T>
+mgmc_status build_gibbs_tables(mgmc_ctx* h)
+{
+    const DevLevel<T>& Lh = levels_of<T>(h)[h->L - 1];
+    const DevLevel<T>& Ch = levels_of<T>(h)[h->L - 2];
+    h->fine0 = Lh.fine != 0;
+    if constexpr (std::is_same<T, float>::value)
+        if (h->fine0) return build_stream_jobs(h, {h});
+    mgmc_status st = MGMC_OK;
+    const int TY = Lh.fine ? TileShape<T, true>::TY : TileShape<T, false>::TY;
+    const int tiles = Lh.ntx * ((Lh.n + TY - 1) / TY);
+    TileMaps mf, mb;
+    if (!make_tile_maps<T>(Lh, Ch, false, &mf) || !make_tile_maps<T>(Lh, Ch, true, &mb))
+        return fail(MGMC_ERR_CUDA, "TMA descriptor encoding failed");
+    h->jobs_tile.push_back(upload(h, std::vector<TileJob<T>>{{Lh, Ch, h->P, 0, tiles}}, st));
+    h->maps_fwd.push_back(upload(h, std::vector<TileMaps>{mf}, st));
+    h->maps_bwd.push_back(upload(h, std::vector<TileMaps>{mb}, st));
+    h->per_tile.push_back(tiles);
+    h->nblk_tile.push_back(tiles);
+    if (st != MGMC_OK) return fail(st, "tile table upload failed");
+    cudaError_t e = tile_prepare_batch<T>();
+    if (e != cudaSuccess) return fail(MGMC_ERR_CUDA, std::string("tile kernel set-up: ") + cudaGetErrorString(e));
+    return MGMC_OK;
+}
+
 template <typename T>
 mgmc_status build_batch_tables(mgmc_ctx* h)
 {
@@ -1328,38 +1433,8 @@ mgmc_status build_batch_tables(mgmc_ctx* h)
     h->stream_fine = false;
     if constexpr (std::is_same<T, float>::value) {
         if (depth > 0 && h->fine0) {
-            cudaError_t e = stream_prepare();
-            if (e != cudaSuccess)
-                return fail(MGMC_ERR_CUDA, std::string("stream kernel set-up: ") + cudaGetErrorString(e));
-            std::vector<StreamJob> sj;
-            std::vector<StreamMaps> sf, sb;
-            long long strips = 0;
-            for (mgmc_ctx* c : chains) {
-                const int l = c->L - 1;
-                if (l <= c->top) continue;
-                const auto& lv = levels_of<float>(c);
-                StreamJob J{};
-                J.L = lv[l];
-                J.C = lv[l - 1];
-                J.cs = c->cs;
-                J.strip0 = strips;
-                J.spb = (J.L.n + kStreamRows - 1) / kStreamRows;
-                J.nbands = (J.L.n + kStreamBand - 1) / kStreamBand;
-                strips += (long long)J.spb * J.nbands;
-                sj.push_back(J);
-                sf.emplace_back();
-                sb.emplace_back();
-                if (!make_stream_maps(J.L, J.C, false, &sf.back()) || !make_stream_maps(J.L, J.C, true, &sb.back()))
-                    return fail(MGMC_ERR_CUDA, "TMA descriptor encoding failed");
-            }
-            h->jobs_stream = upload(h, sj, st);
-            h->maps_sfwd = upload(h, sf, st);
-            h->maps_sbwd = upload(h, sb, st);
-            if (st != MGMC_OK) return fail(st, "stream table upload failed");
-            h->njob_stream = (int)sj.size();
-            h->stream_strips = strips;
-            h->stream_ctas = stream_grid(strips);
-            h->stream_fine = true;
+            st = build_stream_jobs(h, chains);
+            if (st != MGMC_OK) return st;
         }
     }
     for (int d = 0; d < depth; ++d) {
