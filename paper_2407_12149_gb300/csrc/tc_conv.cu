@@ -21,9 +21,9 @@
 //
 // Every mbarrier wait is bounded (1 s): a wait that gives up sets *status = 2, the other roles
 // stop, the copies in flight are waited for (bounded), TMEM is freed and the CTA ends.
-// Measured (GB300, 255^2, c0 = 32; im2col + GEMM + col2im before): gradient of 8 samples 17.65 ->
-// 3.34 ms, estimates of 16 samples 6.21 -> 1.72 ms; k_conv alone, without the lines of
-// k_conv_line, 3.73 and 2.10 ms.
+// Measured (GB300, 255^2, c0 = 32; im2col + GEMM + col2im before): gradient of 8 samples 17.7 ->
+// 2.96 ms, estimates of 16 samples 6.21 -> 1.34 ms (3.34 and 1.72 with 64-bit ring counters; 3.73
+// and 2.10 when k_conv ran every layer, without the lines of k_conv_line).
 #include <algorithm>
 #include <cstring>
 
@@ -40,6 +40,21 @@ constexpr int kBM = 128;
 constexpr int kConvThreads = 192;
 constexpr int kMaxStages = 8;
 constexpr size_t kConvSmem = 220 * 1024;   // dynamic shared memory a CTA may use
+
+// position in a ring of n slots: slot and the parity of its current use (32-bit counters: a
+// 64-bit remainder per chunk cost the issuing thread more than the chunk's MMAs)
+struct RingPos {
+    int slot = 0;
+    unsigned par = 0;
+    __device__ __forceinline__ void next(int n)
+    {
+        if (++slot == n) {
+            slot = 0;
+            par ^= 1u;
+        }
+    }
+    __device__ __forceinline__ int ahead(int d, int n) const { return slot + d >= n ? slot + d - n : slot + d; }
+};
 
 struct ConvArgs {
     CUtensorMap x, w;     // pixels (box CK x tw x th x tb), weights (box CK x NT)
@@ -58,18 +73,18 @@ struct ConvArgs {
     int* status;
 };
 
-// Epilogue warps: one tile's accumulations (`units` of them, the u-th on) from TMEM; false if a
-// wait gave up.  TMEM lanes 32 (warp % 4) .. + 31 are the warp's, lane = pixel p0 + that.
+// Epilogue warps: one tile's accumulations (`units` of them, from buffer bp on) from TMEM; false
+// if a wait gave up.  TMEM lanes 32 (warp % 4) .. + 31 are the warp's, lane = pixel p0 + that.
 template <int NT, bool DG, int NBUF, int NTC>
-__device__ __forceinline__ bool conv_epilogue(const ConvArgs& g, long long p0, int n_first, int units, long long& u,
+__device__ __forceinline__ bool conv_epilogue(const ConvArgs& g, long long p0, int n_first, int units, RingPos& bp,
                                               unsigned tmem, unsigned long long* tfull, unsigned long long* tempty)
 {
     const int quarter = (threadIdx.x >> 5) & 3, lane = threadIdx.x & 31;
     const long long p = p0 + quarter * 32 + lane;
     float acc[DG ? NT : 1];
-    for (int a = 0; a < units; ++a, ++u) {
-        const int buf = (int)(u % NBUF);
-        bool ok = mbar_wait(&tfull[buf], (unsigned)((u / NBUF) & 1));
+    for (int a = 0; a < units; ++a, bp.next(NBUF)) {
+        const int buf = bp.slot;
+        bool ok = mbar_wait(&tfull[buf], bp.par);
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) return false;
         tc5::fence_after();
@@ -137,7 +152,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv(const __grid_constant_
     __shared__ unsigned long long full[kMaxStages], empty[kMaxStages], tfull[4], tempty[4], wbar;
     __shared__ unsigned tmem_slot;
     __shared__ volatile int aborted;
-    __shared__ long long issued, consumed;
+    __shared__ int issued, consumed;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int S = g.stages;
     const int items = 9 * g.taps_c;                       // chunks of one tile
@@ -176,17 +191,18 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv(const __grid_constant_
                     tma_load_2d(wres + (t * g.taps_c + c) * B_BYTES, &g.w, t * g.wtap_k + c * g.ck,
                                 t * g.wtap_r + n_first, &wbar);
         }
-        long long k = 0;
+        int k = 0;
+        RingPos rp;
         for (long long mt = blockIdx.x / g.ntiles_n; mt < mtiles && !aborted; mt += step) {
             const long long p0 = mt * kBM;
             const int j0 = (int)(p0 & (g.H - 1)), i0 = (int)((p0 >> g.lgH) & (g.H - 1));
             const int b0 = (int)(p0 >> (2 * g.lgH));
             for (int t = 0; t < 9 && !aborted; ++t) {
                 const int sy = g.sign * (t / 3 - 1), sx = g.sign * (t % 3 - 1);
-                for (int c = 0; c < g.taps_c; ++c, ++k) {
-                    const int s = (int)(k % S);
-                    const long long use = k / S;
-                    if (use > 0 && !mbar_wait(&empty[s], (unsigned)((use - 1) & 1))) {
+                for (int c = 0; c < g.taps_c; ++c, ++k, rp.next(S)) {
+                    const int s = rp.slot;
+                    // a fresh barrier counts as past its phase of parity 1: the first use does not wait
+                    if (!mbar_wait(&empty[s], rp.par ^ 1u)) {
                         aborted = 1;
                         break;
                     }
@@ -201,20 +217,20 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv(const __grid_constant_
         }
     } else if (warp == 1 && lane == 0) {
         const unsigned id = tc5::idesc(NT, false);
-        long long k = 0, u = 0;
+        int k = 0;
+        RingPos rp, bp;
         bool ok = !g.resident || mbar_wait(&wbar, 0u);
         for (long long mt = blockIdx.x / g.ntiles_n; mt < mtiles && ok && !aborted; mt += step)
-            for (int a = 0; a < items && ok; a += unit, ++u) {
-                const int buf = (int)(u % NBUF);
-                const long long use = u / NBUF;
-                if (use > 0 && !mbar_wait(&tempty[buf], (unsigned)((use - 1) & 1))) {
+            for (int a = 0; a < items && ok; a += unit, bp.next(NBUF)) {
+                const int buf = bp.slot;
+                if (!mbar_wait(&tempty[buf], bp.par ^ 1u)) {
                     ok = false;
                     break;
                 }
                 tc5::fence_after();
-                for (int c = 0; c < unit; ++c, ++k) {
-                    const int s = (int)(k % S);
-                    if (!mbar_wait(&full[s], (unsigned)((k / S) & 1))) {
+                for (int c = 0; c < unit; ++c, ++k, rp.next(S)) {
+                    const int s = rp.slot;
+                    if (!mbar_wait(&full[s], rp.par)) {
                         ok = false;
                         break;
                     }
@@ -233,9 +249,9 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv(const __grid_constant_
         if (!ok) aborted = 1;
     } else if (warp >= 2) {
         bool ok = true;
-        long long u = 0;
+        RingPos bp;
         for (long long mt = blockIdx.x / g.ntiles_n; mt < mtiles && ok && !aborted; mt += step)
-            ok = conv_epilogue<NT, DG, NBUF, NTC>(g, mt * kBM, n_first, items / unit, u, tmem, tfull, tempty);
+            ok = conv_epilogue<NT, DG, NBUF, NTC>(g, mt * kBM, n_first, items / unit, bp, tmem, tfull, tempty);
         if (!ok && lane == 0) aborted = 1;
     }
     __syncwarp();
@@ -243,7 +259,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv(const __grid_constant_
     if (threadIdx.x == 0 && aborted) {
         *g.status = 2;
         if (g.resident) mbar_wait(&wbar, 0u);
-        for (long long k = consumed; k < issued; ++k) mbar_wait(&full[k % S], (unsigned)((k / S) & 1));
+        for (int k = consumed; k < issued; ++k) mbar_wait(&full[k % S], (unsigned)((k / S) & 1));
     }
     tc5::fence_before();
     __syncthreads();
@@ -271,7 +287,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
     __shared__ unsigned long long full[kMaxStages], empty[kMaxStages], tfull[4], tempty[4], wbar;
     __shared__ unsigned tmem_slot;
     __shared__ volatile int aborted;
-    __shared__ long long issued, consumed;
+    __shared__ int issued, consumed;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int NL = g.stages;                       // lines of the ring
     const int items = 9 * g.taps_c;
@@ -310,16 +326,16 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
             for (int c = 0; c < g.taps_c; ++c)
                 tma_load_2d(wres + (t * g.taps_c + c) * B_BYTES, &g.w, t * g.wtap_k + c * g.ck, t * g.wtap_r + n_first,
                             &wbar);
-        long long k = 0;
+        int k = 0;
+        RingPos rp;
         for (long long t0 = beg; t0 < end && !aborted;) {
             const long long strip = t0 >> g.lgH;
             const long long t1 = min(end, (strip + 1) << g.lgH);
             const int ia = (int)(t0 & (g.H - 1)), ib = ia + (int)(t1 - t0);
             const int b = (int)(strip / spi), j0 = (int)(strip % spi) << 7;
-            for (int row = ia - 1; row <= ib; ++row, ++k) {
-                const int s = (int)(k % NL);
-                const long long use = k / NL;
-                if (use > 0 && !mbar_wait(&empty[s], (unsigned)((use - 1) & 1))) {
+            for (int row = ia - 1; row <= ib; ++row, ++k, rp.next(NL)) {
+                const int s = rp.slot;
+                if (!mbar_wait(&empty[s], rp.par ^ 1u)) {
                     aborted = 1;
                     break;
                 }
@@ -332,27 +348,26 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
         }
     } else if (warp == 1 && lane == 0) {
         const unsigned id = tc5::idesc(NT, false);
-        long long k = 0, u = 0;   // k: the line above the tile; u: accumulations
-        long long waited = 0;     // lines known to have arrived
+        RingPos kp, wp, bp;       // the line above the tile, the next line to wait for, the accumulator
+        int waited = 0;           // lines known to have arrived
         bool ok = mbar_wait(&wbar, 0u);
         for (long long t0 = beg; t0 < end && ok && !aborted;) {
             const long long strip = t0 >> g.lgH;
             const long long t1 = min(end, (strip + 1) << g.lgH);
-            for (long long t = t0; t < t1 && ok; ++t, ++k) {
-                for (; waited < k + 3 && ok; ++waited)
-                    ok = mbar_wait(&full[waited % NL], (unsigned)((waited / NL) & 1));
+            for (long long t = t0; t < t1 && ok; ++t, kp.next(NL)) {
+                for (int q = t == t0 ? 3 : 1; q > 0 && ok; --q, ++waited, wp.next(NL))
+                    ok = mbar_wait(&full[wp.slot], wp.par);
                 consumed = waited;
                 if (!ok) break;
                 for (int tap = 0; tap < 9 && ok; ++tap) {
-                    const int buf = (int)(u % NBUF);
+                    const int buf = bp.slot;
                     if (DG || tap == 0) {
-                        const long long use = u / NBUF;
-                        if (use > 0) ok = mbar_wait(&tempty[buf], (unsigned)((use - 1) & 1));
+                        ok = mbar_wait(&tempty[buf], bp.par ^ 1u);
                         if (!ok) break;
                         tc5::fence_after();
                     }
                     const int ky = g.sign > 0 ? tap / 3 : 2 - tap / 3, kx = g.sign > 0 ? tap % 3 : 2 - tap % 3;
-                    const unsigned la = smem_addr(ring + ((k + ky) % NL) * line_bytes) + (unsigned)(kx * CKB);
+                    const unsigned la = smem_addr(ring + kp.ahead(ky, NL) * line_bytes) + (unsigned)(kx * CKB);
                     const unsigned lb = smem_addr(wres + tap * g.taps_c * B_BYTES);
                     for (int c = 0; c < g.taps_c; ++c) {
                         const unsigned long long da = tc5::desc(la + c * CHUNK, 16, 8 * CKB, SW);
@@ -364,27 +379,28 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
                     }
                     if (DG || tap == 8) {
                         tc5::commit(&tfull[buf]);
-                        ++u;
+                        bp.next(NBUF);
                     }
                 }
                 // the line above is done with; after the strip's last row all three are
-                tc5::commit(&empty[k % NL]);
+                tc5::commit(&empty[kp.slot]);
                 if (t + 1 == t1) {
-                    tc5::commit(&empty[(k + 1) % NL]);
-                    tc5::commit(&empty[(k + 2) % NL]);
+                    tc5::commit(&empty[kp.ahead(1, NL)]);
+                    tc5::commit(&empty[kp.ahead(2, NL)]);
                 }
             }
-            k += 2;
+            kp.next(NL);
+            kp.next(NL);
             t0 = t1;
         }
         if (!ok) aborted = 1;
     } else if (warp >= 2) {
         bool ok = true;
-        long long u = 0;
+        RingPos bp;
         for (long long t = beg; t < end && ok && !aborted; ++t) {
             const long long strip = t >> g.lgH;
             const long long row = (strip / spi) * g.H + (t & (g.H - 1));
-            ok = conv_epilogue<NT, DG, NBUF, NTC>(g, row * g.H + ((strip % spi) << 7), n_first, DG ? 9 : 1, u, tmem, tfull,
+            ok = conv_epilogue<NT, DG, NBUF, NTC>(g, row * g.H + ((strip % spi) << 7), n_first, DG ? 9 : 1, bp, tmem, tfull,
                                                   tempty);
         }
         if (!ok && lane == 0) aborted = 1;
@@ -394,7 +410,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
     if (threadIdx.x == 0 && aborted) {
         *g.status = 2;
         mbar_wait(&wbar, 0u);
-        for (long long k = consumed; k < issued; ++k) mbar_wait(&full[k % NL], (unsigned)((k / NL) & 1));
+        for (int k = consumed; k < issued; ++k) mbar_wait(&full[k % NL], (unsigned)((k / NL) & 1));
     }
     tc5::fence_before();
     __syncthreads();

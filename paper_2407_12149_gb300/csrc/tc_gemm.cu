@@ -240,6 +240,8 @@ __global__ void k_reduce_splits(const float* __restrict__ part, int splits, long
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < count;
          i += (long long)gridDim.x * blockDim.x) {
         float acc = part[i];
+        // the loads of 16 partials in flight at a time; the sum stays in order
+#pragma unroll 16
         for (int z = 1; z < splits; ++z) acc += part[(long long)z * count + i];
         out[i] = acc;
     }

@@ -431,7 +431,7 @@ __global__ void k_wt_to_flat(const float* __restrict__ part, int splits, int Kp,
         if (k < K && c < Co) {
             const float* p = part + (long long)k * Co + c;
             acc = p[0];
-#pragma unroll 8
+#pragma unroll 16
             for (int z = 1; z < splits; ++z) acc += p[z * count];
         }
         t[r][threadIdx.x] = acc;
