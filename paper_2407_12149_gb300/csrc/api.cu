@@ -630,7 +630,6 @@ void enqueue_level(mgmc_ctx* h, int l, std::vector<int>& visit, cudaStream_t s, 
     }
     if (h->cfg.nu1 == 0) launch_lowrank<T>(D, P, -1, 0u, true, s, launches);
     launch_restrict<T>(D, lv[l - 1], s, launches);
-    cudaMemsetAsync(lv[l - 1].x, 0, (size_t)lv[l - 1].alloc * sizeof(T), s);
     const int calls = l == Lf ? 1 : h->cfg.gamma;
     for (int g = 0; g < calls; ++g) enqueue_level<T>(h, l - 1, visit, s, launches);
     launch_prolong<T>(lv[l - 1], D, s, launches);
@@ -705,7 +704,6 @@ void enqueue_cycle(mgmc_ctx* h, cudaStream_t s, int& launches)
     }
     for (int l = Lf; l > h->top; --l) {
         const DevLevel<T>& D = lv[l];
-        if (l < Lf) cudaMemsetAsync(D.x, 0, (size_t)D.alloc * sizeof(T), s);
         for (int j = 0; j < h->cfg.nu1; ++j) {
             if (prof && l == Lf && j == 0) cudaEventRecordWithFlags(h->ev[0], s, cudaEventRecordExternal);
             launch_sweep<T>(D, P, 0, (unsigned)(2 * j), s, launches);

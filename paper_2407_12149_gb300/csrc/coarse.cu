@@ -153,7 +153,7 @@ __device__ __forceinline__ double upd_s(const Site<double, DIM>& s, const Blk<do
     return (lo + hi) * s.iv;
 }
 
-// FP32: x + (rhs - A x) / a_ii, the operations of fine_update / coarse_update
+// FP32: x + (rhs - A x) / a_ii, the operations of fine_update / CoarseOps
 template <int DIM>
 __device__ __forceinline__ float upd_s(const Site<float, DIM>& s, const Blk<float>& b, int ls)
 {

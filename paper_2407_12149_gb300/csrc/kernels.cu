@@ -26,6 +26,7 @@
 // second read of theta'.
 #include "kernels.cuh"
 
+#include <algorithm>
 #include <type_traits>
 
 namespace mgmc {
@@ -58,36 +59,55 @@ __device__ __forceinline__ bool colour_item(int n, bool redblack, int colour, lo
     return 4 * q + px < n;
 }
 
-template <typename T, int DIM>
-__device__ __forceinline__ void sweep_item(const DevLevel<T>& L, const DevProblem& P, const CycleState& cs,
-                                           bool redblack, int colour, unsigned slot, long long item)
+// the two sites of a half noise block; late(): what has to come before the state is read
+template <typename T, int DIM, bool FINE, typename Late>
+__device__ __forceinline__ void sweep_item(const DevLevel<T>& L, const CycleState& cs, bool redblack, int colour,
+                                           unsigned slot, long long item, Late&& late)
 {
-    int j, k, px, q;
-    if (!colour_item<DIM>(L.n, redblack, colour, item, j, k, px, q)) return;
-    int n = L.n;
-    int nq = (n + 3) >> 2;
-    int i0 = 4 * q + px;
-    bool has1 = i0 + 2 < n;
+    int j = 0, k = 0, px = 0, q = 0;
+    const bool on = colour_item<DIM>(L.n, redblack, colour, item, j, k, px, q);
+    const int n = L.n, nq = (n + 3) >> 2, i0 = 4 * q + px;
+    const bool has1 = on && i0 + 2 < n;
     T z0 = T(0), z1 = T(0);
-    if (cs.noise)  // the block of the group's row, this colour's half of it
+    if (on && cs.noise)  // the block of the group's row, this colour's half of it
         draw_half_ctr<T>(noise_counter(cs, 0u, 0u, L.level, slot), (unsigned)(((long long)k * n + j) * nq + q), px,
                          (unsigned)cs.seed, (unsigned)(cs.seed >> 32), z0, z1);
-    long long e = site_offset(DIM, L.pitch, L.plane, L.base, i0, j, k);
-    if (L.fine) {
-        L.x[e] = fine_update<DIM>(L, e, z0);
+    const long long e = on ? site_offset(DIM, L.pitch, L.plane, L.base, i0, j, k) : 0;
+    if constexpr (FINE) {
+        late();
+        if (on) L.x[e] = fine_update<DIM>(L, e, z0);
         if (has1) L.x[e + 2] = fine_update<DIM>(L, e + 2, z1);
     } else {
-        L.x[e] = coarse_update<DIM>(L, e, z0);
-        if (has1) L.x[e + 2] = coarse_update<DIM>(L, e + 2, z1);
+        CoarseOps<T, DIM> s0, s1;
+        if (on) s0.load(L, e);
+        if (has1) s1.load(L, e + 2);
+        late();
+        // sites of one colour are not neighbours of each other
+        T x0 = T(0), x1 = T(0);
+        if (on) x0 = s0.apply(L, e, z0);
+        if (has1) x1 = s1.apply(L, e + 2, z1);
+        if (on) L.x[e] = x0;
+        if (has1) L.x[e + 2] = x1;
     }
 }
 
-template <typename T, int DIM>
-__global__ void k_sweep_colour(DevLevel<T> L, DevProblem P, int redblack, int colour, unsigned slot)
+// One colour of a sweep.
+// What bounds it: the latency of the launches of a cycle (8 colours a grid in 3D, each too
+// small to fill the chip below 127^3), not their work.  Programmatic launch: what does not
+// depend on earlier launches -- the normals, the stencils of both sites, 1/a_ii, sqrt(a_ii) --
+// is formed before the wait (the cycle state changes only in a cycle's last launch, and the
+// first launch of a cycle has no programmatic predecessor), so that after it one round trip
+// of state and right-hand side is left.
+// Measured (GB300, with the programmatic launches of the low-rank and transfer kernels and 64-thread
+// CTAs on small grids; plain launches before): 127^3 FP32, 2 cycles 1040 -> 617 us; 255^2 squared
+// operator, W-cycle 2532 -> 2431 us; 255^2 Q1 Gibbs, 8 steps 274 -> 233 us.
+template <typename T, int DIM, bool FINE>
+__global__ void __launch_bounds__(256) k_sweep_colour(DevLevel<T> L, DevProblem P, int redblack, int colour, unsigned slot)
 {
+    pdl_launch_dependents();
     const CycleState cs = *P.cs;
-    long long item = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    sweep_item<T, DIM>(L, P, cs, redblack != 0, colour, slot, item);
+    const long long item = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    sweep_item<T, DIM, FINE>(L, cs, redblack != 0, colour, slot, item, [] { pdl_wait(); });
 }
 
 // 25-point grids (squared shifted Laplacian, FP64 2D): colour c = cx + 3 cy is the class
@@ -137,30 +157,31 @@ __device__ __forceinline__ void zero25_pair(const DevLevel<double>& L, double* z
     if (i0 + 2 < L.n) zb[j * L.n + i0 + 2] = 0.0;
 }
 
-__device__ __forceinline__ void sweep25_site(const DevLevel<double>& L, const CycleState& cs, int colour,
-                                             unsigned slot, long long t)
+// as k_sweep_colour: normals (half the FP64 work of a site) and stencils before the wait
+__global__ void __launch_bounds__(256) k_sweep25(DevLevel<double> L, DevProblem P, int colour, unsigned slot)
 {
-    const int n = L.n;
-    int i, j;
-    colour25_site(n, colour, t, i, j);
-    double z = 0.0;
-    if (cs.noise) {
-        double z0, z1;
-        const int nq = (n + 3) >> 2;
-        draw_half_ctr<double>(noise_counter(cs, 0u, 0u, L.level, slot), (unsigned)(j * nq + (i >> 2)), i & 1,
-                              (unsigned)cs.seed, (unsigned)(cs.seed >> 32), z0, z1);
-        z = ((i >> 1) & 1) ? z1 : z0;
-    }
-    const long long e = site_offset(2, L.pitch, L.plane, L.base, i, j, 0);
-    L.x[e] = update25(L, e, z);
-}
-
-__global__ void k_sweep25(DevLevel<double> L, DevProblem P, int colour, unsigned slot)
-{
+    pdl_launch_dependents();
     const CycleState cs = *P.cs;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= colour25_sites(L.n, colour)) return;
-    sweep25_site(L, cs, colour, slot, t);
+    const bool on = t < colour25_sites(L.n, colour);
+    int i = 0, j = 0;
+    double z = 0.0;
+    Ops25 s;
+    long long e = 0;
+    if (on) {
+        colour25_site(L.n, colour, t, i, j);
+        e = site_offset(2, L.pitch, L.plane, L.base, i, j, 0);
+        s.load(L, e);
+        if (cs.noise) {
+            double z0, z1;
+            const int nq = (L.n + 3) >> 2;
+            draw_half_ctr<double>(noise_counter(cs, 0u, 0u, L.level, slot), (unsigned)(j * nq + (i >> 2)), i & 1,
+                                  (unsigned)cs.seed, (unsigned)(cs.seed >> 32), z0, z1);
+            z = ((i >> 1) & 1) ? z1 : z0;
+        }
+    }
+    pdl_wait();
+    if (on) L.x[e] = s.apply(L, e, z);
 }
 
 // Exact coarsest sample theta_0 = A~_0^-1 f_0 + L_0^-T z (Sec. 3.5) with the coarsest
@@ -327,8 +348,12 @@ __global__ void k_lowrank_v(DevLevel<T> L, DevProblem P, int dir, unsigned slot,
 {
     __shared__ double z[kMaxObs];
     __shared__ double zp[kMaxObs];
+    pdl_launch_dependents();
     const CycleState cs = *P.cs;
-    lowrank_v_body<T>(L, P, cs, dir, slot, want_dnext, z, zp);
+    if (dir >= 0 && cs.noise)  // the noise before the wait on the preceding launch
+        for (int k = threadIdx.x; k < P.m; k += blockDim.x) zp[k] = lowrank_normal<T>(cs, L.level, slot, k);
+    pdl_wait();
+    lowrank_v_body<T>(L, P, cs, dir, slot, want_dnext, z, zp, zp);
 }
 
 // theta' = theta*_s - G v on G's rows r0, r0 + stride, ...
@@ -357,16 +382,57 @@ __device__ __forceinline__ void lowrank_dnext(const DevLevel<T>& L, int m, const
 }
 
 // theta' = theta*_s - G v on G's rows, spread over the grid; with want_dnext block 0
-// also forms d_{l-1} = d_l - B^T theta' = d_l - z + (B^T G) v
+// also forms d_{l-1} = d_l - B^T theta' = d_l - z + (B^T G) v.  Four lanes per row (an FP64
+// product costs a warp about 70 cycles, not overlapped with its next one); up to kLrPre
+// of the lane's coefficients are loaded before the wait on the preceding launch.
 template <typename T>
-__global__ void k_lowrank_apply(DevLevel<T> L, DevProblem P, int dir, int want_dnext)
+__global__ void __launch_bounds__(256) k_lowrank_apply(DevLevel<T> L, DevProblem P, int dir, int want_dnext)
 {
+    constexpr int kLrPre = 8;
     __shared__ double v[kMaxObs];
-    const int m = P.m;
+    pdl_launch_dependents();
+    const int m = P.m, rows = L.g_rows[dir], p = threadIdx.x & 3, wr = (threadIdx.x & 31) >> 2;
+    const int r0 = (int)(blockIdx.x * blockDim.x + threadIdx.x) >> 2, stride = (int)(gridDim.x * blockDim.x) >> 2;
+    const double* G = L.g_val[dir];
+    double g[kLrPre];
+    long long s0 = 0;
+    if (r0 < rows) {
+        s0 = L.g_site[dir][r0];
+#pragma unroll
+        for (int q = 0; q < kLrPre; ++q) g[q] = p + 4 * q < m ? G[(long long)r0 * m + p + 4 * q] : 0.0;
+    }
+    pdl_wait();
     for (int k = threadIdx.x; k < m; k += blockDim.x) v[k] = L.lrv[k];
     __syncthreads();
-    lowrank_rows<T>(L, m, dir, v, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
-    if (want_dnext && blockIdx.x == 0) lowrank_dnext<T>(L, m, v);
+    for (int r = r0; r - wr < rows; r += stride) {  // whole warps stay together for the shuffles
+        const bool on = r < rows;
+        double acc = 0.0;
+        if (on) {
+            int t = p;
+            if (r == r0) {
+#pragma unroll
+                for (int q = 0; q < kLrPre; ++q)
+                    if (p + 4 * q < m) acc += g[q] * v[p + 4 * q];
+                t += 4 * kLrPre;
+            }
+            for (; t < m; t += 4) acc += G[(long long)r * m + t] * v[t];
+        }
+        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        if (on && p == 0) {
+            const long long s = r == r0 ? s0 : (long long)L.g_site[dir][r];
+            L.x[s] = (T)((double)L.x[s] - acc);
+        }
+    }
+    if (want_dnext && blockIdx.x == 0)
+        for (int k = threadIdx.x >> 2; k - wr < m; k += blockDim.x >> 2) {
+            double acc = 0.0;
+            if (k < m)
+                for (int t = p; t < m; t += 4) acc += L.BtG[k * m + t] * v[t];
+            acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+            acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+            if (k < m && p == 0) L.dnext[k] = L.d[k] - L.lrv[m + k] + acc;
+        }
 }
 
 // r = f_l - A_l theta at every interior site of the fine grid (the restriction's input)
@@ -381,6 +447,8 @@ __device__ __forceinline__ void residual_site(const DevLevel<T>& F, long long s)
 template <typename T, int DIM>
 __global__ void k_residual(DevLevel<T> F)
 {
+    pdl_launch_dependents();
+    pdl_wait();
     long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     long long N = (long long)F.n * F.n * (DIM == 3 ? F.n : 1);
     if (s >= N) return;
@@ -408,10 +476,15 @@ __device__ __forceinline__ void restrict_site(const DevLevel<T>& F, const DevLev
 template <typename T, int DIM>
 __global__ void k_restrict(DevLevel<T> F, DevLevel<T> C)
 {
+    pdl_launch_dependents();
+    pdl_wait();
     long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     long long N = (long long)C.n * C.n * (DIM == 3 ? C.n : 1);
     if (s >= N) return;
     restrict_site<T, DIM>(F, C, s);
+    // psi_{l-1} = 0 (the ghost ring is never written)
+    int I = (int)(s % C.n), J = (int)((s / C.n) % C.n), K = DIM == 3 ? (int)(s / ((long long)C.n * C.n)) : 0;
+    C.x[site_offset(DIM, C.pitch, C.plane, C.base, I, J, K)] = T(0);
 }
 
 template <typename T, int DIM>
@@ -425,6 +498,8 @@ __device__ __forceinline__ void prolong_add_site(const DevLevel<T>& C, const Dev
 template <typename T, int DIM>
 __global__ void k_prolong(DevLevel<T> C, DevLevel<T> F)
 {
+    pdl_launch_dependents();
+    pdl_wait();
     long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     long long N = (long long)F.n * F.n * (DIM == 3 ? F.n : 1);
     if (s >= N) return;
@@ -689,7 +764,7 @@ __global__ void __launch_bounds__(kSmallCycleThreads)
                     const int colour = dir == 0 ? g2 : 1 - g2;
                     const long long items = (long long)L.n * nq;
                     for (long long it = threadIdx.x; it < items; it += blockDim.x)
-                        sweep_item<T, 2>(L, P, cs, true, colour, slot, it);
+                        sweep_item<T, 2, true>(L, cs, true, colour, slot, it, [] {});
                     __syncthreads();
                 }
             } else {
@@ -698,7 +773,7 @@ __global__ void __launch_bounds__(kSmallCycleThreads)
                     const int py = (c >> 1) & 1;
                     const long long items = (long long)((L.n - py + 1) / 2) * nq;
                     for (long long it = threadIdx.x; it < items; it += blockDim.x)
-                        sweep_item<T, 2>(L, P, cs, false, c, slot, it);
+                        sweep_item<T, 2, false>(L, cs, false, c, slot, it, [] {});
                     __syncthreads();
                 }
             }
@@ -875,11 +950,14 @@ __global__ void k_sum(const double* partial, int n, double* out)
 // ---------------------------------------------------------------------------
 static inline unsigned blocks_for(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
+// Threads per CTA of a launch of `items` threads: 64 while 256 would leave SMs idle, so that
+// a small grid's loads (and its FP64 instructions, which issue per SM) are spread over the chip
+static inline int sweep_threads(long long items) { return items <= 256LL * 304 ? 64 : 256; }
+
 template <typename T>
 void launch_sweep(const DevLevel<T>& L, const DevProblem& P, int dir, unsigned slot, cudaStream_t st, int& launches)
 {
-    const int bs = 256;
-    int nq = (L.n + 3) / 4;
+    const int nq = (L.n + 3) / 4;
     if constexpr (std::is_same<T, double>::value) {
         if (L.rad == 2) {
             // the nine classes in code order forward, reversed backward
@@ -887,37 +965,26 @@ void launch_sweep(const DevLevel<T>& L, const DevProblem& P, int dir, unsigned s
                 const int c = dir == 0 ? ci : 8 - ci;
                 const long long sites = (long long)((L.n - c % 3 + 2) / 3) * ((L.n - c / 3 + 2) / 3);
                 if (sites <= 0) continue;
-                k_sweep25<<<blocks_for(sites, bs), bs, 0, st>>>(L, P, c, slot);
+                const int bs = sweep_threads(sites);
+                launch_pdl(k_sweep25, dim3(blocks_for(sites, bs)), dim3(bs), 0, st, L, P, c, slot);
                 ++launches;
             }
             return;
         }
     }
-    if (L.fine) {
-        long long rows = L.dim == 3 ? (long long)L.n * L.n : L.n;
-        for (int g = 0; g < 2; ++g) {
-            int colour = dir == 0 ? g : 1 - g;
-            unsigned nb = blocks_for(rows * nq, bs);
-            if (L.dim == 2)
-                k_sweep_colour<T, 2><<<nb, bs, 0, st>>>(L, P, 1, colour, slot);
-            else
-                k_sweep_colour<T, 3><<<nb, bs, 0, st>>>(L, P, 1, colour, slot);
-            ++launches;
-        }
-        return;
-    }
     const int seq2[4] = {0, 3, 2, 1};
     const int seq3[8] = {0, 6, 5, 3, 4, 2, 1, 7};
-    int nc = L.dim == 2 ? 4 : 8;
+    const int nc = L.fine ? 2 : (L.dim == 2 ? 4 : 8);
     for (int ci = 0; ci < nc; ++ci) {
-        int c = L.dim == 2 ? seq2[dir == 0 ? ci : nc - 1 - ci] : seq3[dir == 0 ? ci : nc - 1 - ci];
-        int py = (c >> 1) & 1, pz = (c >> 2) & 1;
-        long long rows = (long long)((L.n - py + 1) / 2) * (L.dim == 3 ? (L.n - pz + 1) / 2 : 1);
-        unsigned nb = blocks_for(rows * nq, bs);
-        if (L.dim == 2)
-            k_sweep_colour<T, 2><<<nb, bs, 0, st>>>(L, P, 0, c, slot);
-        else
-            k_sweep_colour<T, 3><<<nb, bs, 0, st>>>(L, P, 0, c, slot);
+        const int at = dir == 0 ? ci : nc - 1 - ci;
+        const int c = L.fine ? at : (L.dim == 2 ? seq2[at] : seq3[at]);
+        const int py = (c >> 1) & 1, pz = (c >> 2) & 1;
+        const long long rows = L.fine ? (L.dim == 3 ? (long long)L.n * L.n : L.n)
+                                      : (long long)((L.n - py + 1) / 2) * (L.dim == 3 ? (L.n - pz + 1) / 2 : 1);
+        const int bs = sweep_threads(rows * nq);
+        auto* kernel = L.dim == 2 ? (L.fine ? k_sweep_colour<T, 2, true> : k_sweep_colour<T, 2, false>)
+                                  : (L.fine ? k_sweep_colour<T, 3, true> : k_sweep_colour<T, 3, false>);
+        launch_pdl(kernel, dim3(blocks_for(rows * nq, bs)), dim3(bs), 0, st, L, P, L.fine ? 1 : 0, c, slot);
         ++launches;
     }
 }
@@ -927,39 +994,32 @@ void launch_lowrank(const DevLevel<T>& L, const DevProblem& P, int dir, unsigned
                     int& launches)
 {
     if (P.m == 0) return;
-    k_lowrank_v<T><<<1, 256, 0, st>>>(L, P, dir, slot, dnext ? 1 : 0);
+    launch_pdl(k_lowrank_v<T>, dim3(1), dim3(256), 0, st, L, P, dir, slot, dnext ? 1 : 0);
     ++launches;
     if (dir < 0) return;
-    const int rows = L.g_rows[dir];
-    int nb = (rows + 255) / 256;
-    nb = nb < 1 ? 1 : (nb > 1024 ? 1024 : nb);
-    k_lowrank_apply<T><<<nb, 256, 0, st>>>(L, P, dir, dnext ? 1 : 0);
+    const unsigned nb = std::min(std::max(blocks_for(4LL * L.g_rows[dir], 256), 1u), 1024u);
+    launch_pdl(k_lowrank_apply<T>, dim3(nb), dim3(256), 0, st, L, P, dir, dnext ? 1 : 0);
     ++launches;
 }
 
+// f_{l-1} = P^T (f_l - A_l theta) and psi_{l-1} = 0
 template <typename T>
 void launch_restrict(const DevLevel<T>& F, const DevLevel<T>& C, cudaStream_t st, int& launches)
 {
-    long long NF = (long long)F.n * F.n * (F.dim == 3 ? F.n : 1);
-    long long N = (long long)C.n * C.n * (C.dim == 3 ? C.n : 1);
-    if (C.dim == 2) {
-        k_residual<T, 2><<<blocks_for(NF, 256), 256, 0, st>>>(F);
-        k_restrict<T, 2><<<blocks_for(N, 256), 256, 0, st>>>(F, C);
-    } else {
-        k_residual<T, 3><<<blocks_for(NF, 256), 256, 0, st>>>(F);
-        k_restrict<T, 3><<<blocks_for(N, 256), 256, 0, st>>>(F, C);
-    }
+    const long long NF = (long long)F.n * F.n * (F.dim == 3 ? F.n : 1);
+    const long long N = (long long)C.n * C.n * (C.dim == 3 ? C.n : 1);
+    const int bf = sweep_threads(NF), bc = sweep_threads(N);
+    launch_pdl(C.dim == 2 ? k_residual<T, 2> : k_residual<T, 3>, dim3(blocks_for(NF, bf)), dim3(bf), 0, st, F);
+    launch_pdl(C.dim == 2 ? k_restrict<T, 2> : k_restrict<T, 3>, dim3(blocks_for(N, bc)), dim3(bc), 0, st, F, C);
     launches += 2;
 }
 
 template <typename T>
 void launch_prolong(const DevLevel<T>& C, const DevLevel<T>& F, cudaStream_t st, int& launches)
 {
-    long long N = (long long)F.n * F.n * (F.dim == 3 ? F.n : 1);
-    if (F.dim == 2)
-        k_prolong<T, 2><<<blocks_for(N, 256), 256, 0, st>>>(C, F);
-    else
-        k_prolong<T, 3><<<blocks_for(N, 256), 256, 0, st>>>(C, F);
+    const long long N = (long long)F.n * F.n * (F.dim == 3 ? F.n : 1);
+    const int bs = sweep_threads(N);
+    launch_pdl(F.dim == 2 ? k_prolong<T, 2> : k_prolong<T, 3>, dim3(blocks_for(N, bs)), dim3(bs), 0, st, C, F);
     ++launches;
 }
 

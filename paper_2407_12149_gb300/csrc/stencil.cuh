@@ -54,21 +54,6 @@ __device__ __forceinline__ double coef25_at(const DevLevel<double>& L, long long
     return L.coef[(long long)(12 - o) * L.alloc + e + off25(o, L.pitch)];
 }
 
-// one Gibbs update of a 25-point site, x_i <- (f_i + sqrt(a_ii) z - sum_{j != i} a_ij x_j) / a_ii
-// with the neighbours in lexicographic offset order; 1 / a_ii and sqrt(a_ii) come from the
-// host (FP64 division and square root are long instruction sequences on this GPU)
-__device__ __forceinline__ double update25(const DevLevel<double>& L, long long e, double z)
-{
-    double acc = L.f ? L.f[e] : 0.0;
-    acc += L.isq[L.alloc + e] * z;
-#pragma unroll
-    for (int o = 0; o < 25; ++o) {
-        if (o == 12) continue;
-        acc -= coef25_at(L, e, o) * L.x[e + off25(o, L.pitch)];
-    }
-    return acc * L.isq[e];
-}
-
 // ---------------------------------------------------------------------------
 // one site update of the Gibbs sweep with right-hand side fdense_i + sqrt(a_ii) z
 // ---------------------------------------------------------------------------
@@ -106,44 +91,6 @@ __device__ __forceinline__ float fine_update(const DevLevel<float>& L, long long
     return xi + (rhs - Ax) * ia;
 }
 
-template <int DIM>
-__device__ __forceinline__ double coarse_update(const DevLevel<double>& L, long long e, double z)
-{
-    constexpr int NS = Offsets<DIM>::NS;
-    constexpr int C = Offsets<DIM>::C;
-    double acc = L.f ? L.f[e] : 0.0;
-    acc += L.isq[L.alloc + e] * z;
-#pragma unroll
-    for (int o = 0; o < NS; ++o) {
-        if (o == C) continue;
-        acc -= coef_at<DIM>(L, e, o) * L.x[e + off_of<DIM>(o, L.pitch, L.plane)];
-    }
-    return acc * L.isq[e];
-}
-
-template <int DIM>
-__device__ __forceinline__ float coarse_update(const DevLevel<float>& L, long long e, float z)
-{
-    constexpr int NS = Offsets<DIM>::NS;
-    constexpr int C = Offsets<DIM>::C;
-    float xi = L.x[e];
-    float s = L.coef[e];
-    float lap = 0.0f, offsum = 0.0f;
-#pragma unroll
-    for (int o = 0; o < NS; ++o) {
-        if (o == C) continue;
-        float a = coef_at<DIM>(L, e, o);
-        lap = fmaf(a, L.x[e + off_of<DIM>(o, L.pitch, L.plane)] - xi, lap);
-        offsum += a;
-    }
-    float aii = s - offsum;
-    float Ax = fmaf(s, xi, lap);
-    float ia, sa;
-    inv_and_sqrt(aii, ia, sa);
-    float rhs = (L.f ? L.f[e] : 0.0f) + sa * z;
-    return xi + (rhs - Ax) * ia;
-}
-
 // One FP32 Gibbs update of a 5-point site from its value xi, its four neighbours,
 // the row-sum part c = s kappa^2_i and the off-diagonal magnitude w (dense
 // right-hand side 0: the finest grid), the same operations as fine_update.
@@ -164,6 +111,79 @@ __device__ __forceinline__ float fine_ax(float xi, float up, float lf, float rt,
     float lap = (xi - up) + (xi - lf) + (xi - rt) + (xi - dn);
     return fmaf(c, xi, w * lap);
 }
+
+// The update of a site of a 9-/27-point (CoarseOps) or 25-point (Ops25) grid in two parts, so
+// that the first can run before the wait on the preceding launch: load() takes what set-up
+// fixed (off-diagonals, 1/a_ii, sqrt(a_ii)) into registers, apply() the state and
+// right-hand side.
+template <typename T, int DIM>
+struct CoarseOps {
+    static constexpr int NS = Offsets<DIM>::NS;
+    static constexpr int C = Offsets<DIM>::C;
+    T a[NS], inv, sq;
+    T s;   // row sum (FP32)
+
+    __device__ __forceinline__ void load(const DevLevel<T>& L, long long e)
+    {
+#pragma unroll
+        for (int o = 0; o < NS; ++o)
+            if (o != C) a[o] = coef_at<DIM>(L, e, o);
+        if constexpr (sizeof(T) == 8) {
+            inv = L.isq[e];
+            sq = L.isq[L.alloc + e];
+        } else {
+            s = L.coef[e];
+            float offsum = 0.0f;
+#pragma unroll
+            for (int o = 0; o < NS; ++o)
+                if (o != C) offsum += a[o];
+            inv_and_sqrt(s - offsum, inv, sq);
+        }
+    }
+
+    __device__ __forceinline__ T apply(const DevLevel<T>& L, long long e, T z) const
+    {
+        if constexpr (sizeof(T) == 8) {
+            double acc = L.f ? L.f[e] : 0.0;
+            acc += sq * z;
+#pragma unroll
+            for (int o = 0; o < NS; ++o)
+                if (o != C) acc -= a[o] * L.x[e + off_of<DIM>(o, L.pitch, L.plane)];
+            return acc * inv;
+        } else {
+            const float xi = L.x[e];
+            float lap = 0.0f;
+#pragma unroll
+            for (int o = 0; o < NS; ++o)
+                if (o != C) lap = fmaf(a[o], L.x[e + off_of<DIM>(o, L.pitch, L.plane)] - xi, lap);
+            const float rhs = (L.f ? L.f[e] : 0.0f) + sq * z;
+            return xi + (rhs - fmaf(s, xi, lap)) * inv;
+        }
+    }
+};
+
+struct Ops25 {
+    double a[25], inv, sq;
+
+    __device__ __forceinline__ void load(const DevLevel<double>& L, long long e)
+    {
+#pragma unroll
+        for (int o = 0; o < 25; ++o)
+            if (o != 12) a[o] = coef25_at(L, e, o);
+        inv = L.isq[e];
+        sq = L.isq[L.alloc + e];
+    }
+
+    __device__ __forceinline__ double apply(const DevLevel<double>& L, long long e, double z) const
+    {
+        double acc = L.f ? L.f[e] : 0.0;
+        acc += sq * z;
+#pragma unroll
+        for (int o = 0; o < 25; ++o)
+            if (o != 12) acc -= a[o] * L.x[e + off25(o, L.pitch)];
+        return acc * inv;
+    }
+};
 
 // (A x)_e of the level (dense part of the operator)
 template <int DIM>
@@ -226,7 +246,7 @@ __device__ __forceinline__ float apply_A(const DevLevel<float>& L, long long e)
 
 // --- FP32 9-point sites of a 4-site group (components 0..3), shared by the tile
 // and the streaming kernels so that both evaluate the same operations in the
-// same order (coarse_update / apply_A of the Galerkin grids).
+// same order (CoarseOps / apply_A of the Galerkin grids).
 // component k of the row (k = -1 and k = 4 are the scalar e outside the group)
 __device__ __forceinline__ float cmp(const float4& v, float e, int k)
 {

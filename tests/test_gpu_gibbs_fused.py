@@ -1,6 +1,6 @@
 """The 2D Gibbs sampler with one sweep before and after (the V-cycle's fused sweep kernels)
 and with two (one launch per colour) against the oracle, over both stencils, both
-precisions, odd and ragged sizes, with and without observations."""
+precisions and several sizes, with and without observations."""
 import numpy as np
 import pytest
 
@@ -11,10 +11,10 @@ from tests.test_gpu_parity import _check32, _check64, _run_gpu
 pytestmark = pytest.mark.gpu
 
 
-# sizes: the smallest grid with two levels, one ragged tile, several tiles, the streamed FP32 range
+# sizes: the smallest grid with two levels, less than a tile, several tiles, the streamed FP32 range
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
 @pytest.mark.parametrize("nu", [1, 2])
-@pytest.mark.parametrize("n,m,disc", [(3, 1, 0), (7, 3, 1), (31, 0, 1), (95, 9, 0), (255, 16, 1), (511, 4, 0)])
+@pytest.mark.parametrize("n,m,disc", [(3, 1, 0), (7, 3, 1), (31, 0, 1), (127, 9, 0), (255, 16, 1), (511, 4, 0)])
 def test_gibbs_matches_oracle(n, m, disc, nu, precision):
     import torch
     from paper_2407_12149_gb300 import build
@@ -29,7 +29,7 @@ def test_gibbs_matches_oracle(n, m, disc, nu, precision):
 
 
 def _oracle(n, m, disc, nu):
-    p = inputs.make_problem("t", 2, n, n_levels=5 if n == 95 else None, kappa2_seed=None if disc else 5, kappa2_const=100.0, m=m,
+    p = inputs.make_problem("t", 2, n, n_levels=None, kappa2_seed=None if disc else 5, kappa2_const=100.0, m=m,
                             obs_seed=4, disc=disc, qoi_cells=(n + 1) // 4)
     o = oracle.Oracle(p.dim, p.n, p.n_levels, kappa2=p.kappa2, kappa2_const=p.kappa2_const, scale_hd=p.scale_hd,
                       disc=disc, nu1=nu, nu2=nu, obs_site=p.obs_site, obs_w=p.obs_w, Gamma=p.Gamma, y=p.y,
