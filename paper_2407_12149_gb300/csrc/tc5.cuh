@@ -78,5 +78,20 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, i
         : "memory");
 }
 
+// position in a ring of n slots: slot and the parity of its current use (32-bit counters: a
+// 64-bit remainder per chunk cost the issuing thread more than the chunk's MMAs)
+struct RingPos {
+    int slot = 0;
+    unsigned par = 0;
+    __device__ __forceinline__ void next(int n)
+    {
+        if (++slot == n) {
+            slot = 0;
+            par ^= 1u;
+        }
+    }
+    __device__ __forceinline__ int ahead(int d, int n) const { return slot + d >= n ? slot + d - n : slot + d; }
+};
+
 }  // namespace tc5
 }  // namespace mgmc

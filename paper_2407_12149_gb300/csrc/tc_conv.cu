@@ -29,32 +29,19 @@
 
 #include "tc5.cuh"
 #include "tc_conv.cuh"
+#include "tc_gemm.cuh"
 
 namespace mgmc {
 
 namespace {
 
 using bf16 = __nv_bfloat16;
+using tc5::RingPos;
 
 constexpr int kBM = 128;
 constexpr int kConvThreads = 192;
 constexpr int kMaxStages = 8;
 constexpr size_t kConvSmem = 220 * 1024;   // dynamic shared memory a CTA may use
-
-// position in a ring of n slots: slot and the parity of its current use (32-bit counters: a
-// 64-bit remainder per chunk cost the issuing thread more than the chunk's MMAs)
-struct RingPos {
-    int slot = 0;
-    unsigned par = 0;
-    __device__ __forceinline__ void next(int n)
-    {
-        if (++slot == n) {
-            slot = 0;
-            par ^= 1u;
-        }
-    }
-    __device__ __forceinline__ int ahead(int d, int n) const { return slot + d >= n ? slot + d - n : slot + d; }
-};
 
 struct ConvArgs {
     CUtensorMap x, w;     // pixels (box CK x tw x th x tb), weights (box CK x NT)
@@ -573,14 +560,6 @@ bool matrix_map(CUtensorMap* m, const bf16* base, int cols, int rows, int ck, in
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<bf16*>(base), dims, strides, box, es,
               CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_mode(2 * ck), CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-int sm_count()
-{
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return 1;
-    return sms;
 }
 
 template <int NT, int CKB, bool DG>

@@ -27,6 +27,9 @@ struct TcGemm {
     int k_per_split;
 };
 
+// multiprocessors of the current device (1 if it cannot be read)
+int sm_count();
+
 // Describe C = A B^T for row-major BF16 A [M][lda] and B [N][ldb] (lda, ldb >= K,
 // multiples of 8 elements; device pointers 16-byte aligned).  splits > 1 only
 // with the FP32 epilogue.  Returns false if the descriptors cannot be encoded.
