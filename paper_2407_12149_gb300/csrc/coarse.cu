@@ -28,7 +28,7 @@
 //  - the code is small (loops over items are not unrolled, the draws are functions): every
 //    launch starts with a cold instruction cache, and an unrolled version of 170 KB spent
 //    30 thousand cycles a launch on instruction fetches.
-// The FP32 arithmetic of a site is that of stencil.cuh, operation by operation.
+// The FP32 arithmetic of a site is that of stencil.cuh, with the update's last product and sum rounded apart.
 // Measured (GB300, against one CTA per chain with operands staged by loads, per-sweep
 // draws and triangular solves): cycle of one 31^2 FP64 chain 137 -> 73 us, of a 255^2 FP32
 // chain 142 -> 97 us, kernel inside a batch of eight 1023^2 chains 95 -> 50 us.  What is left
@@ -153,7 +153,7 @@ __device__ __forceinline__ double upd_s(const Site<double, DIM>& s, const Blk<do
     return (lo + hi) * s.iv;
 }
 
-// FP32: x + (rhs - A x) / a_ii, the operations of fine_update / CoarseOps
+// FP32: x + (rhs - A x) / a_ii
 template <int DIM>
 __device__ __forceinline__ float upd_s(const Site<float, DIM>& s, const Blk<float>& b, int ls)
 {
@@ -173,7 +173,9 @@ __device__ __forceinline__ float upd_s(const Site<float, DIM>& s, const Blk<floa
             if (o != C) lap = fmaf(s.c[o], X[ls + soff<DIM>(o, b.S)] - xi, lap);
         Ax = fmaf(s.c[C], xi, lap);
     }
-    return fmaf(s.rhs - Ax, s.iv, xi);
+    // product and sum rounded apart: the rounding every earlier state of these grids has had
+    // (contracted, the update's error against 64 bits is the same, its bits are not)
+    return __fadd_rn(xi, __fmul_rn(s.rhs - Ax, s.iv));
 }
 
 // (A x) of the dense part at ls
