@@ -297,9 +297,9 @@ mgmc_status mgmc_set_wait_limit(mgmc_handle h, int64_t limit_ns);
 mgmc_status mgmc_set_band_min_n(mgmc_handle h, int band_min_n);
 
 /* Threads per CTA of the 2D coarse-grid kernel (one CTA per chain, all grids with
- * n <= coarse_max_n in shared memory): 0 (default) chooses 1024 while the chains
- * leave SMs free and 256 once several chains share an SM; else a multiple of 32 in
- * [64, 1024].  The kernel's arithmetic does not depend on it (the states are bitwise
+ * n <= coarse_max_n in shared memory): 0 (default) chooses 256, or 512 when
+ * a 63^2 grid is inside; else a multiple of 32 in [64, 1024] (values above the kernel's
+ * limit, 512 in FP32 2D and 256 otherwise, run at the limit).  The kernel's arithmetic does not depend on it (the states are bitwise
  * the same); only the time of its barrier-bound phases does.  The graph is captured
  * again on the next sampling call.  MGMC_ERR_ARG for other values. */
 mgmc_status mgmc_set_coarse_threads(mgmc_handle h, int threads);

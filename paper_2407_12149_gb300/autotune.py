@@ -7,7 +7,7 @@ Three settings change how a cycle runs but not what it computes:
   band_min_n    of the 9-point grids below the finest (FP32), those with
                 n >= band_min_n run in the streaming band kernels, the others in the
                 tile kernels (bitwise identical states);
-  coarse_threads threads per CTA of the coarse kernel (0: by the chain count; the
+  coarse_threads threads per CTA of the coarse kernel (0: by its largest grid; the
                 kernel's arithmetic does not depend on it).
 Which values are fastest depends on the chain count and the grid sizes, so each
 candidate's captured V-cycle is timed with CUDA events over back-to-back cycles

@@ -145,7 +145,7 @@ struct mgmc_ctx {
     int stream_ctas = 0;
     // FP32 9-point grids below the finest: the streaming band kernels (stream9.cu) at the
     // depths whose grids all have n >= band_min_n, per depth
-    int coarse_threads = 0;   // threads of the batched coarse kernel (0: by the chain count)
+    int coarse_threads = 0;   // compute threads of the coarse kernel (0: by the largest grid inside)
     std::vector<char> s9_ok, s9_use;
     std::vector<int> s9_minn;   // smallest grid of the depth
     std::vector<void*> jobs_s9, maps_s9;
@@ -959,7 +959,7 @@ mgmc_status mgmc_create(const mgmc_config* cfg_in, const mgmc_allocator* alloc, 
             h->plan = p;
         }
     }
-    // the Gibbs sampler sweeps the finest grid with the unfused kernels, outside the coarse
+    // the Gibbs sampler sweeps the finest grid alone, outside the coarse
     // kernel; W-cycles and radius-2 grids run every grid above the coarsest on the general
     // path, the cycle enqueued recursively
     h->recursive = cfg.gamma == 2 || cfg.disc == MGMC_SSL;
