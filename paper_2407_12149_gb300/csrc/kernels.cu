@@ -99,8 +99,8 @@ __device__ __forceinline__ void sweep_item(const DevLevel<T>& L, const CycleStat
 // first launch of a cycle has no programmatic predecessor), so that after it one round trip
 // of state and right-hand side is left.
 // Measured (GB300, with the programmatic launches of the low-rank and transfer kernels and 64-thread
-// CTAs on small grids; plain launches before): 127^3 FP32, 2 cycles 1040 -> 617 us; 255^2 squared
-// operator, W-cycle 2532 -> 2431 us; 255^2 Q1 Gibbs, 8 steps 274 -> 233 us.
+// CTAs on small grids; plain launches before): 127^3 FP32, 2 cycles 1040 -> 620 us; 255^2 squared
+// operator, W-cycle 2532 -> 2434 us; 255^2 Q1 Gibbs, 8 steps 274 -> 229 us.
 template <typename T, int DIM, bool FINE>
 __global__ void __launch_bounds__(256) k_sweep_colour(DevLevel<T> L, DevProblem P, int redblack, int colour, unsigned slot)
 {
@@ -952,6 +952,8 @@ static inline unsigned blocks_for(long long n, int bs) { return (unsigned)((n + 
 
 // Threads per CTA of a launch of `items` threads: 64 while 256 would leave SMs idle, so that
 // a small grid's loads (and its FP64 instructions, which issue per SM) are spread over the chip
+// (against 256 everywhere: 127^3 FP32, 2 cycles 667 -> 620 us; 255^2 W-cycle 2437 -> 2408 us);
+// above 304 CTAs of 256 every SM has its two either way
 static inline int sweep_threads(long long items) { return items <= 256LL * 304 ? 64 : 256; }
 
 template <typename T>
