@@ -371,11 +371,20 @@ mgmc_status mgmc_unet_destroy(mgmc_unet_handle u);
  * epilogue: bit 0 add bias (device float [N]), bit 1 ReLU, bit 2 store BF16
  * (else float).  splits > 1 (FP32 output only): the K range is cut into
  * `splits` parts summed in a fixed order (deterministic).  C: device [M][N].
- * Asynchronous on stream; MGMC_ERR_TIMEOUT is reported by the next call that
- * synchronises (a bounded wait inside the kernel gave up).
+ * Asynchronous on stream.  A bounded wait (1 s) inside the kernel that gives up
+ * leaves rows of tiles of C unwritten (splits > 1: C undefined) and is reported by
+ * mgmc_tc_gemm_status.
  * ------------------------------------------------------------------------ */
 mgmc_status mgmc_tc_gemm(const void* A, int lda, const void* B, int ldb, void* C, int M, int N, int K, int splits,
                          int epilogue, const float* bias, void* stream);
+/* Waits for the work on `stream`, then MGMC_ERR_TIMEOUT if a product on the current
+ * device, of this or another thread, has given up since this thread last asked. */
+mgmc_status mgmc_tc_gemm_status(void* stream);
+/* mgmc_tc_gemm with the bound of the kernel's waits in nanoseconds: 0 the default; a
+ * negative value (tests) makes the part that issues the products give up on its first
+ * operands and the others after -wait_ns. */
+mgmc_status mgmc_tc_gemm_bounded(const void* A, int lda, const void* B, int ldb, void* C, int M, int N, int K,
+                                 int splits, int epilogue, const float* bias, void* stream, int64_t wait_ns);
 
 /* Message of the last failing call on this thread; valid until the next call. */
 const char* mgmc_last_error(void);

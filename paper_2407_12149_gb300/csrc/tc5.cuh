@@ -78,6 +78,10 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, i
         : "memory");
 }
 
+// Bound of the waits of the roles beside the MMA issuer, from a kernel's wait_ns (see mbar_wait): a
+// negative bound makes the issuer alone give up at once, so that the others are caught waiting
+__device__ __forceinline__ long long role_limit(long long wait_ns) { return wait_ns < 0 ? -wait_ns : wait_ns; }
+
 // position in a ring of n slots: slot and the parity of its current use (32-bit counters: a
 // 64-bit remainder per chunk cost the issuing thread more than the chunk's MMAs)
 struct RingPos {

@@ -17,8 +17,10 @@
 // the CTAs running together share both operands' tiles in L2.
 // Measured (GB300, one tile per CTA and tiles along M first before): 65536 x 256 x 2304 with bias, ReLU
 // and BF16 output 112 -> 83 us, 8192^3 0.809 -> 0.735 ms; the products are bitwise the same.
-// Every mbarrier wait is bounded (1 s); a wait that gives up sets *status = 2, the other roles
-// stop, the CTA waits (bounded) for its own copies in flight, frees its TMEM and ends.
+// Every mbarrier wait is bounded (1 s).  When one gives up the other roles stop, the accumulator
+// in work is not handed to the epilogue (so what a warp stores, 32 rows of a tile, is always whole), the
+// CTA waits (bounded) for its MMAs and copies in flight, counts the event in *status, frees
+// its TMEM and ends.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -30,6 +32,9 @@
 namespace mgmc {
 
 namespace {
+
+// give-ups of the kernels launched without a status word of their own
+__device__ int g_gave_up;
 
 using tc5::RingPos;
 
@@ -124,7 +129,8 @@ __device__ __forceinline__ void gemm_epilogue(unsigned tmem, const Tile& T, void
 template <int BN>
 __global__ void __launch_bounds__(kThreads, 1)
     k_tc_gemm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, void* C, int M,
-              int N, int K, int k_per_split, long long tiles, int epi, const float* __restrict__ bias, int* status)
+              int N, int K, int k_per_split, long long tiles, int epi, const float* __restrict__ bias, int* status,
+              long long wait_ns)
 {
     constexpr int A_BYTES = kBM * kBK * 2;
     constexpr int STAGE_BYTES = A_BYTES + BN * kBK * 2;
@@ -133,7 +139,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     // 128-byte-swizzled operand tiles start on 1024-byte boundaries
     unsigned char* sm = smem_align_up<1024>(smem_dyn);
-    __shared__ unsigned long long full[S], empty[S], tfull[2], tempty[2];
+    __shared__ unsigned long long full[S], empty[S], tfull[2], tempty[2], drained;
     __shared__ unsigned tmem_slot;
     __shared__ volatile int aborted;
     __shared__ int issued, consumed;
@@ -148,6 +154,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(&tfull[b]);
             mbar_init_count(&tempty[b], 4);
         }
+        mbar_init(&drained);
         fence_mbar_init();
         aborted = 0;
         issued = consumed = 0;
@@ -157,6 +164,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     tc5::fence_after();
     const unsigned tmem = tmem_slot;
+    const long long lim = tc5::role_limit(wait_ns);
 
     if (warp == 0 && lane == 0) {
         int k = 0;
@@ -165,7 +173,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             const Tile T = tile_at<BN>(t, M, N, K, k_per_split);
             for (int kb = 0; kb < T.nkb; ++kb, ++k, rp.next(S)) {
                 // a fresh barrier counts as past its phase of parity 1: the first use does not wait
-                if (!mbar_wait(&empty[rp.slot], rp.par ^ 1u)) {
+                if (!mbar_wait(&empty[rp.slot], rp.par ^ 1u, lim)) {
                     aborted = 1;
                     break;
                 }
@@ -183,13 +191,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         bool ok = true;
         for (long long t = blockIdx.x; t < tiles && ok && !aborted; t += gridDim.x, bp.next(2)) {
             const Tile T = tile_at<BN>(t, M, N, K, k_per_split);
-            if (!mbar_wait(&tempty[bp.slot], bp.par ^ 1u)) {
+            if (!mbar_wait(&tempty[bp.slot], bp.par ^ 1u, lim)) {
                 ok = false;
                 break;
             }
             tc5::fence_after();
             for (int kb = 0; kb < T.nkb; ++kb, ++k, rp.next(S)) {
-                if (!mbar_wait(&full[rp.slot], rp.par)) {
+                if (!mbar_wait(&full[rp.slot], rp.par, wait_ns)) {
                     ok = false;
                     break;
                 }
@@ -203,14 +211,17 @@ __global__ void __launch_bounds__(kThreads, 1)
                 tc5::commit(&empty[rp.slot]);
                 consumed = k + 1;
             }
+            if (!ok) break;   // an incomplete accumulator never reaches the epilogue
             tc5::commit(&tfull[bp.slot]);
         }
         if (!ok) aborted = 1;
     } else if (warp >= 2) {
         bool ok = true;
         RingPos bp;
-        for (long long t = blockIdx.x; t < tiles && !aborted; t += gridDim.x, bp.next(2)) {
-            ok = mbar_wait(&tfull[bp.slot], bp.par);
+        for (long long t = blockIdx.x; t < tiles; t += gridDim.x, bp.next(2)) {
+            // the lanes leave the loop together: tcgen05.ld is a warp's
+            if (__any_sync(0xffffffffu, aborted)) break;
+            ok = mbar_wait(&tfull[bp.slot], bp.par, lim);
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc5::fence_after();
@@ -223,10 +234,16 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     __syncwarp();
     __syncthreads();
-    if (threadIdx.x == 0 && aborted) {
-        *status = 2;
-        // copies issued but never consumed may still be in flight: wait for them (bounded)
-        for (int k = consumed; k < issued; ++k) mbar_wait(&full[k % S], (unsigned)((k / S) & 1));
+    if (aborted) {
+        // MMAs issued and copies never consumed may still be in flight: wait for them (bounded)
+        if (threadIdx.x == 32) {
+            tc5::commit(&drained);
+            mbar_wait(&drained, 0u);
+        }
+        if (threadIdx.x == 0) {
+            for (int k = consumed; k < issued; ++k) mbar_wait(&full[k % S], (unsigned)((k / S) & 1));
+            atomicAdd(status ? status : &g_gave_up, 1);
+        }
     }
     tc5::fence_before();
     __syncthreads();
@@ -259,7 +276,8 @@ bool encode_bf16(CUtensorMap* m, const void* base, int ld, int rows, int cols, i
 }
 
 template <int BN>
-cudaError_t launch(const TcGemm& g, void* C, int epi, const float* bias, int* status, cudaStream_t st)
+cudaError_t launch(const TcGemm& g, void* C, int epi, const float* bias, int* status, long long wait_ns,
+                   cudaStream_t st)
 {
     static bool prepared = false;  // per process (one device in use at a time)
     if (!prepared) {
@@ -271,7 +289,7 @@ cudaError_t launch(const TcGemm& g, void* C, int epi, const float* bias, int* st
     const long long tiles = (long long)((g.M + kBM - 1) / kBM) * ((g.N + BN - 1) / BN) * g.splits;
     const unsigned grid = (unsigned)std::min<long long>(tiles, sm_count());
     k_tc_gemm<BN><<<grid, kThreads, gemm_smem<BN>(), st>>>(g.a, g.b, C, g.M, g.N, g.K, g.k_per_split, tiles, epi, bias,
-                                                          status);
+                                                          status, wait_ns);
     return cudaGetLastError();
 }
 
@@ -315,15 +333,22 @@ bool tc_gemm_plan(TcGemm* g, const void* A, int lda, const void* B, int ldb, int
     return encode_bf16(&g->a, A, lda, M, K, kBM) && encode_bf16(&g->b, B, ldb, N, K, g->bn);
 }
 
-cudaError_t tc_gemm_run(const TcGemm& g, void* C, int epilogue, const float* bias, int* status, cudaStream_t st)
+cudaError_t tc_gemm_run(const TcGemm& g, void* C, int epilogue, const float* bias, int* status, long long wait_ns,
+                        cudaStream_t st)
 {
     if (g.splits > 1 && epilogue != kEpiF32) return cudaErrorInvalidValue;
     switch (g.bn) {
-        case 32: return launch<32>(g, C, epilogue, bias, status, st);
-        case 64: return launch<64>(g, C, epilogue, bias, status, st);
-        case 128: return launch<128>(g, C, epilogue, bias, status, st);
-        default: return launch<256>(g, C, epilogue, bias, status, st);
+        case 32: return launch<32>(g, C, epilogue, bias, status, wait_ns, st);
+        case 64: return launch<64>(g, C, epilogue, bias, status, wait_ns, st);
+        case 128: return launch<128>(g, C, epilogue, bias, status, wait_ns, st);
+        default: return launch<256>(g, C, epilogue, bias, status, wait_ns, st);
     }
+}
+
+cudaError_t tc_gemm_gave_up(int* count, cudaStream_t st)
+{
+    cudaError_t e = cudaMemcpyFromSymbolAsync(count, g_gave_up, sizeof(int), 0, cudaMemcpyDeviceToHost, st);
+    return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
 }
 
 cudaError_t tc_reduce_splits(const float* part, int splits, long long count, float* out, cudaStream_t st)

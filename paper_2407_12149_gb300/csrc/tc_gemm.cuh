@@ -35,8 +35,13 @@ int sm_count();
 // with the FP32 epilogue.  Returns false if the descriptors cannot be encoded.
 bool tc_gemm_plan(TcGemm* g, const void* A, int lda, const void* B, int ldb, int M, int N, int K, int splits);
 // Launch; C is float or __nv_bfloat16 [M][N] (row-major), bias float [N] or NULL.
-// status: device int set to 2 if a bounded wait inside the kernel gave up.
-cudaError_t tc_gemm_run(const TcGemm& g, void* C, int epilogue, const float* bias, int* status, cudaStream_t st);
+// status: device int that counts the CTAs in which a bounded wait gave up (NULL: a counter of
+// the device, see tc_gemm_gave_up).  wait_ns: bound of the waits (0: 1 s; < 0, a test of the
+// give-up path: the MMA issuer gives up on its first operands, the other roles after -wait_ns).
+cudaError_t tc_gemm_run(const TcGemm& g, void* C, int epilogue, const float* bias, int* status, long long wait_ns,
+                        cudaStream_t st);
+// The current device's counter of such CTAs once the work on `st` is done (synchronises it).
+cudaError_t tc_gemm_gave_up(int* count, cudaStream_t st);
 // Sum of `splits` FP32 partials [splits][count] into out [count] (fixed order).
 cudaError_t tc_reduce_splits(const float* part, int splits, long long count, float* out, cudaStream_t st);
 

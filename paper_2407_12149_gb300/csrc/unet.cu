@@ -28,6 +28,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <map>
 #include <string>
 #include <vector>
 
@@ -616,7 +617,7 @@ mgmc_status gemm(UnetCtx* u, const void* A, int lda, const void* B, int ldb, voi
     if (g.splits > 1 && (size_t)g.splits * M * N > u->wpart_elems)
         return unet_fail(MGMC_ERR_STATE, "split-K scratch too small");
     void* out = g.splits > 1 ? (void*)u->wpart : C;
-    UNET_CUDA(tc_gemm_run(g, out, epi, bias, u->status, u->stream));
+    UNET_CUDA(tc_gemm_run(g, out, epi, bias, u->status, 0, u->stream));
     if (g.splits > 1) UNET_CUDA(tc_reduce_splits(u->wpart, g.splits, M * N, (float*)C, u->stream));
     return MGMC_OK;
 }
@@ -778,7 +779,7 @@ mgmc_status check_status(UnetCtx* u)
     int s = 0;
     UNET_CUDA(cudaStreamSynchronize(u->stream));
     UNET_CUDA(cudaMemcpy(&s, u->status, sizeof(int), cudaMemcpyDeviceToHost));
-    if (s == 2) return unet_fail(MGMC_ERR_TIMEOUT, "a tensor-core GEMM's bounded wait gave up");
+    if (s != 0) return unet_fail(MGMC_ERR_TIMEOUT, "a bounded wait inside a tensor-core kernel gave up");
     return MGMC_OK;
 }
 
@@ -1061,9 +1062,27 @@ mgmc_status mgmc_unet_destroy(mgmc_unet_handle u)
 mgmc_status mgmc_tc_gemm(const void* A, int lda, const void* B, int ldb, void* C, int M, int N, int K, int splits,
                          int epilogue, const float* bias, void* stream)
 {
+    return mgmc_tc_gemm_bounded(A, lda, B, ldb, C, M, N, K, splits, epilogue, bias, stream, 0);
+}
+
+mgmc_status mgmc_tc_gemm_status(void* stream)
+{
+    // the counter of every device as this thread last saw it
+    static thread_local std::map<int, int> seen;
+    int dev = 0, count = 0;
+    UNET_CUDA(cudaGetDevice(&dev));
+    UNET_CUDA(tc_gemm_gave_up(&count, (cudaStream_t)stream));
+    int& last = seen[dev];
+    if (count == last) return MGMC_OK;
+    last = count;
+    return unet_fail(MGMC_ERR_TIMEOUT, "mgmc_tc_gemm: a bounded wait inside the kernel gave up");
+}
+
+mgmc_status mgmc_tc_gemm_bounded(const void* A, int lda, const void* B, int ldb, void* C, int M, int N, int K,
+                                 int splits, int epilogue, const float* bias, void* stream, int64_t wait_ns)
+{
     static thread_local float* part = nullptr;
     static thread_local size_t part_bytes = 0;
-    static thread_local int* status = nullptr;
     if (!A || !B || !C || M <= 0 || N <= 0 || K <= 0 || splits < 1 || (epilogue & ~7) ||
         ((epilogue & kEpiBias) && !bias))
         return unet_fail(MGMC_ERR_ARG, "mgmc_tc_gemm: bad arguments");
@@ -1073,10 +1092,6 @@ mgmc_status mgmc_tc_gemm(const void* A, int lda, const void* B, int ldb, void* C
     TcGemm g;
     if (!tc_gemm_plan(&g, A, lda, B, ldb, M, N, K, splits))
         return unet_fail(MGMC_ERR_ARG, "mgmc_tc_gemm: TMA descriptor encoding failed (alignment, lda/ldb)");
-    if (!status) {
-        UNET_CUDA(cudaMalloc(&status, sizeof(int)));
-        UNET_CUDA(cudaMemset(status, 0, sizeof(int)));
-    }
     void* out = C;
     if (g.splits > 1) {
         const size_t need = sizeof(float) * (size_t)g.splits * M * N;
@@ -1089,7 +1104,7 @@ mgmc_status mgmc_tc_gemm(const void* A, int lda, const void* B, int ldb, void* C
         }
         out = part;
     }
-    UNET_CUDA(tc_gemm_run(g, out, epilogue, bias, status, st));
+    UNET_CUDA(tc_gemm_run(g, out, epilogue, bias, nullptr, (long long)wait_ns, st));
     if (g.splits > 1) UNET_CUDA(tc_reduce_splits(part, g.splits, (long long)M * N, (float*)C, st));
     return MGMC_OK;
 }

@@ -75,7 +75,7 @@ _lib = None
 EXPORTS = ("mgmc_config_default", "mgmc_create", "mgmc_point_obs_rows", "mgmc_sample", "mgmc_mean_solve",
            "mgmc_qoi_stats", "mgmc_qoi_stats_noalloc", "mgmc_info", "mgmc_level_n", "mgmc_launches_per_cycle", "mgmc_set_profiling",
            "mgmc_profile_times", "mgmc_set_band_min_n", "mgmc_set_coarse_threads", "mgmc_create_batch", "mgmc_sample_batch", "mgmc_get_state", "mgmc_destroy",
-           "mgmc_tc_gemm", "mgmc_unet_create", "mgmc_unet_n_params", "mgmc_unet_get_params",
+           "mgmc_tc_gemm", "mgmc_tc_gemm_status", "mgmc_tc_gemm_bounded", "mgmc_unet_create", "mgmc_unet_n_params", "mgmc_unet_get_params",
            "mgmc_unet_set_params", "mgmc_unet_inputs", "mgmc_unet_gradient", "mgmc_unet_train",
            "mgmc_unet_predict", "mgmc_unet_destroy", "mgmc_check_status", "mgmc_set_wait_limit",
            "mgmc_fine_operator",
@@ -120,6 +120,8 @@ def load():
     L.mgmc_tc_gemm.argtypes = [ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p, ctypes.c_int, ctypes.c_void_p,
                                ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_void_p,
                                ctypes.c_void_p]
+    L.mgmc_tc_gemm_bounded.argtypes = L.mgmc_tc_gemm.argtypes + [ctypes.c_int64]
+    L.mgmc_tc_gemm_status.argtypes = [ctypes.c_void_p]
     L.mgmc_unet_create.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_uint64,
                                    ctypes.POINTER(mgmc_allocator), ctypes.c_void_p, ctypes.POINTER(ctypes.c_void_p)]
     L.mgmc_unet_n_params.argtypes = [ctypes.c_void_p, ctypes.POINTER(ctypes.c_int64)]
@@ -256,19 +258,27 @@ def mgmc_create(dim, n, *, n_levels=0, nu1=1, nu2=1, precision=MGMC_FP64, scale_
 EPI_BIAS, EPI_RELU, EPI_BF16 = 1, 2, 4
 
 
-def tc_gemm(A, B, out=None, splits=1, epilogue=0, bias=None, stream=None):
+def tc_gemm(A, B, out=None, splits=1, epilogue=0, bias=None, stream=None, wait_ns=0):
     """C = A B^T on the tensor cores: A [M][K], B [N][K] bfloat16 CUDA tensors
-    (row strides multiples of 8); returns C [M][N] float32 (bfloat16 with EPI_BF16)."""
+    (row strides multiples of 8); returns C [M][N] float32 (bfloat16 with EPI_BF16).
+    Asynchronous; tc_gemm_status reports a product that gave up.  wait_ns: bound of the
+    kernel's waits (mgmc_tc_gemm_bounded; 0 the default)."""
     torch = _torch()
     M, K = A.shape
     N = B.shape[0]
     if out is None:
         out = torch.empty(M, N, dtype=torch.bfloat16 if epilogue & EPI_BF16 else torch.float32, device=A.device)
-    _check(load().mgmc_tc_gemm(ctypes.c_void_p(A.data_ptr()), A.stride(0), ctypes.c_void_p(B.data_ptr()),
-                               B.stride(0), ctypes.c_void_p(out.data_ptr()), M, N, K, splits, epilogue,
-                               ctypes.c_void_p(bias.data_ptr()) if bias is not None else None,
-                               _stream_handle(stream)))
+    _check(load().mgmc_tc_gemm_bounded(ctypes.c_void_p(A.data_ptr()), A.stride(0), ctypes.c_void_p(B.data_ptr()),
+                                       B.stride(0), ctypes.c_void_p(out.data_ptr()), M, N, K, splits, epilogue,
+                                       ctypes.c_void_p(bias.data_ptr()) if bias is not None else None,
+                                       _stream_handle(stream), int(wait_ns)))
     return out
+
+
+def tc_gemm_status(stream=None):
+    """Wait for the stream's work and raise MGMCError if a product on the device has given up
+    since this thread last asked (mgmc_tc_gemm_status)."""
+    _check(load().mgmc_tc_gemm_status(_stream_handle(stream)))
 
 
 def mgmc_get_state(h, chain, x_ptr, stream=None):
