@@ -360,6 +360,11 @@ mgmc_status mgmc_unet_train(mgmc_unet_handle u, int64_t n_samples, const void* i
  * or FP64 (precision = MGMC_FP32 / MGMC_FP64) */
 mgmc_status mgmc_unet_predict(mgmc_unet_handle u, int64_t n_samples, const void* inputs_bf16, void* x_out,
                               int precision);
+/* Bound of the staging waits of the handle's tensor-core kernels in later calls, as
+ * mgmc_tc_gemm_bounded's wait_ns (0, the default: 1 s).  A call in which one gave up
+ * returns MGMC_ERR_TIMEOUT; its outputs, and after mgmc_unet_train the parameters, are
+ * then undefined. */
+mgmc_status mgmc_unet_set_wait_limit(mgmc_unet_handle u, int64_t limit_ns);
 mgmc_status mgmc_unet_destroy(mgmc_unet_handle u);
 
 /* ------------------------------------------------------------------------

@@ -19,8 +19,9 @@
 // read pixel-major, i.e. MN-major tiles (64 pixels x 64 or 32 channels), so nothing is
 // transposed; the pixel range is cut into splits summed in a fixed order.
 //
-// Every mbarrier wait is bounded (1 s): a wait that gives up sets *status = 2, the other roles
-// stop, the copies in flight are waited for (bounded), TMEM is freed and the CTA ends.
+// Every mbarrier wait is bounded (1 s): when one gives up the other roles stop, the accumulator in
+// work is not handed to the epilogue, MMAs and copies in flight are waited for (bounded), the
+// event is counted in *status, TMEM is freed and the CTA ends.
 // Measured (GB300, 255^2, c0 = 32; im2col + GEMM + col2im before): gradient of 8 samples 17.7 ->
 // 2.96 ms, estimates of 16 samples 6.21 -> 1.34 ms (3.34 and 1.72 with 64-bit ring counters; 3.73
 // and 2.10 when k_conv ran every layer, without the lines of k_conv_line).
@@ -58,6 +59,7 @@ struct ConvArgs {
     const float* bias;
     void* out;
     int* status;
+    long long wait_ns;    // bound of the waits (tc_gemm.cuh)
 };
 
 // Epilogue warps: one tile's accumulations (`units` of them, from buffer bp on) from TMEM; false
@@ -71,7 +73,7 @@ __device__ __forceinline__ bool conv_epilogue(const ConvArgs& g, long long p0, i
     float acc[DG ? NT : 1];
     for (int a = 0; a < units; ++a, bp.next(NBUF)) {
         const int buf = bp.slot;
-        bool ok = mbar_wait(&tfull[buf], bp.par);
+        bool ok = mbar_wait(&tfull[buf], bp.par, tc5::role_limit(g.wait_ns));
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) return false;
         tc5::fence_after();
@@ -125,6 +127,23 @@ __device__ __forceinline__ bool conv_epilogue(const ConvArgs& g, long long p0, i
     return true;
 }
 
+// After a wait gave up, all threads: the MMAs issued (by thread 32) and the copies never consumed
+// (stages consumed .. issued - 1 of the ring of n, the weights) may still be in flight and are
+// waited for (bounded)
+__device__ __forceinline__ void conv_drain(unsigned long long* full, int n, int consumed, int issued,
+                                           unsigned long long* wbar, unsigned long long* drained, int* status)
+{
+    if (threadIdx.x == 32) {
+        tc5::commit(drained);
+        mbar_wait(drained, 0u);
+    }
+    if (threadIdx.x == 0) {
+        if (wbar) mbar_wait(wbar, 0u);
+        for (int k = consumed; k < issued; ++k) mbar_wait(&full[k % n], (unsigned)((k / n) & 1));
+        atomicAdd(status, 1);
+    }
+}
+
 // NT: output channels of a tile; CKB: bytes of a chunk's row; DG: data gradient
 template <int NT, int CKB, bool DG>
 __global__ void __launch_bounds__(kConvThreads, 1) k_conv(const __grid_constant__ ConvArgs g)
@@ -136,7 +155,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv(const __grid_constant_
     constexpr unsigned SW = tc5::swizzle_of(CKB);
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     unsigned char* sm = smem_align_up<1024>(smem_dyn);
-    __shared__ unsigned long long full[kMaxStages], empty[kMaxStages], tfull[4], tempty[4], wbar;
+    __shared__ unsigned long long full[kMaxStages], empty[kMaxStages], tfull[4], tempty[4], wbar, drained;
     __shared__ unsigned tmem_slot;
     __shared__ volatile int aborted;
     __shared__ int issued, consumed;
@@ -157,6 +176,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv(const __grid_constant_
             mbar_init_count(&tempty[b], 4);
         }
         mbar_init(&wbar);
+        mbar_init(&drained);
         fence_mbar_init();
         aborted = 0;
         issued = consumed = 0;
@@ -166,6 +186,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv(const __grid_constant_
     __syncthreads();
     tc5::fence_after();
     const unsigned tmem = tmem_slot;
+    const long long lim = tc5::role_limit(g.wait_ns);
     const int n_first = (int)(blockIdx.x % g.ntiles_n) * NT;   // a CTA keeps its N tile (grid is a multiple)
     const long long step = gridDim.x / g.ntiles_n;
     const long long mtiles = g.tiles / g.ntiles_n;
@@ -189,7 +210,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv(const __grid_constant_
                 for (int c = 0; c < g.taps_c; ++c, ++k, rp.next(S)) {
                     const int s = rp.slot;
                     // a fresh barrier counts as past its phase of parity 1: the first use does not wait
-                    if (!mbar_wait(&empty[s], rp.par ^ 1u)) {
+                    if (!mbar_wait(&empty[s], rp.par ^ 1u, lim)) {
                         aborted = 1;
                         break;
                     }
@@ -210,14 +231,14 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv(const __grid_constant_
         for (long long mt = blockIdx.x / g.ntiles_n; mt < mtiles && ok && !aborted; mt += step)
             for (int a = 0; a < items && ok; a += unit, bp.next(NBUF)) {
                 const int buf = bp.slot;
-                if (!mbar_wait(&tempty[buf], bp.par ^ 1u)) {
+                if (!mbar_wait(&tempty[buf], bp.par ^ 1u, lim)) {
                     ok = false;
                     break;
                 }
                 tc5::fence_after();
                 for (int c = 0; c < unit; ++c, ++k, rp.next(S)) {
                     const int s = rp.slot;
-                    if (!mbar_wait(&full[s], rp.par)) {
+                    if (!mbar_wait(&full[s], rp.par, g.wait_ns)) {
                         ok = false;
                         break;
                     }
@@ -231,23 +252,21 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv(const __grid_constant_
                     tc5::commit(&empty[s]);
                     consumed = k + 1;
                 }
+                if (!ok) break;   // an incomplete accumulator never reaches the epilogue
                 tc5::commit(&tfull[buf]);
             }
         if (!ok) aborted = 1;
     } else if (warp >= 2) {
         bool ok = true;
         RingPos bp;
-        for (long long mt = blockIdx.x / g.ntiles_n; mt < mtiles && ok && !aborted; mt += step)
+        // the lanes leave the loop together: tcgen05.ld is a warp's
+        for (long long mt = blockIdx.x / g.ntiles_n; mt < mtiles && ok && !__any_sync(0xffffffffu, aborted); mt += step)
             ok = conv_epilogue<NT, DG, NBUF, NTC>(g, mt * kBM, n_first, items / unit, bp, tmem, tfull, tempty);
         if (!ok && lane == 0) aborted = 1;
     }
     __syncwarp();
     __syncthreads();
-    if (threadIdx.x == 0 && aborted) {
-        *g.status = 2;
-        if (g.resident) mbar_wait(&wbar, 0u);
-        for (int k = consumed; k < issued; ++k) mbar_wait(&full[k % S], (unsigned)((k / S) & 1));
-    }
+    if (aborted) conv_drain(full, S, consumed, issued, g.resident ? &wbar : nullptr, &drained, g.status);
     tc5::fence_before();
     __syncthreads();
     if (warp == 0) tc5::dealloc(tmem, TCOLS);
@@ -271,7 +290,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
     constexpr unsigned SW = tc5::swizzle_of(CKB);
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     unsigned char* sm = smem_align_up<1024>(smem_dyn);
-    __shared__ unsigned long long full[kMaxStages], empty[kMaxStages], tfull[4], tempty[4], wbar;
+    __shared__ unsigned long long full[kMaxStages], empty[kMaxStages], tfull[4], tempty[4], wbar, drained;
     __shared__ unsigned tmem_slot;
     __shared__ volatile int aborted;
     __shared__ int issued, consumed;
@@ -291,6 +310,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
             mbar_init_count(&tempty[b], 4);
         }
         mbar_init(&wbar);
+        mbar_init(&drained);
         fence_mbar_init();
         aborted = 0;
         issued = consumed = 0;
@@ -300,6 +320,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
     __syncthreads();
     tc5::fence_after();
     const unsigned tmem = tmem_slot;
+    const long long lim = tc5::role_limit(g.wait_ns);
     const int n_first = (int)(blockIdx.x % g.ntiles_n) * NT;
     const long long ctas = gridDim.x / g.ntiles_n, cta = blockIdx.x / g.ntiles_n;
     const long long mtiles = g.tiles / g.ntiles_n;
@@ -322,7 +343,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
             const int b = (int)(strip / spi), j0 = (int)(strip % spi) << 7;
             for (int row = ia - 1; row <= ib; ++row, ++k, rp.next(NL)) {
                 const int s = rp.slot;
-                if (!mbar_wait(&empty[s], rp.par ^ 1u)) {
+                if (!mbar_wait(&empty[s], rp.par ^ 1u, lim)) {
                     aborted = 1;
                     break;
                 }
@@ -342,14 +363,16 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
             const long long strip = t0 >> g.lgH;
             const long long t1 = min(end, (strip + 1) << g.lgH);
             for (long long t = t0; t < t1 && ok; ++t, kp.next(NL)) {
-                for (int q = t == t0 ? 3 : 1; q > 0 && ok; --q, ++waited, wp.next(NL))
-                    ok = mbar_wait(&full[wp.slot], wp.par);
+                for (int q = t == t0 ? 3 : 1; q > 0; --q, ++waited, wp.next(NL)) {
+                    ok = mbar_wait(&full[wp.slot], wp.par, g.wait_ns);
+                    if (!ok) break;   // `waited` counts the lines that have arrived
+                }
                 consumed = waited;
                 if (!ok) break;
                 for (int tap = 0; tap < 9 && ok; ++tap) {
                     const int buf = bp.slot;
                     if (DG || tap == 0) {
-                        ok = mbar_wait(&tempty[buf], bp.par ^ 1u);
+                        ok = mbar_wait(&tempty[buf], bp.par ^ 1u, lim);
                         if (!ok) break;
                         tc5::fence_after();
                     }
@@ -369,6 +392,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
                         bp.next(NBUF);
                     }
                 }
+                if (!ok) break;
                 // the line above is done with; after the strip's last row all three are
                 tc5::commit(&empty[kp.slot]);
                 if (t + 1 == t1) {
@@ -384,7 +408,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
     } else if (warp >= 2) {
         bool ok = true;
         RingPos bp;
-        for (long long t = beg; t < end && ok && !aborted; ++t) {
+        for (long long t = beg; t < end && ok && !__any_sync(0xffffffffu, aborted); ++t) {
             const long long strip = t >> g.lgH;
             const long long row = (strip / spi) * g.H + (t & (g.H - 1));
             ok = conv_epilogue<NT, DG, NBUF, NTC>(g, row * g.H + ((strip % spi) << 7), n_first, DG ? 9 : 1, bp, tmem, tfull,
@@ -394,11 +418,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
     }
     __syncwarp();
     __syncthreads();
-    if (threadIdx.x == 0 && aborted) {
-        *g.status = 2;
-        mbar_wait(&wbar, 0u);
-        for (int k = consumed; k < issued; ++k) mbar_wait(&full[k % NL], (unsigned)((k / NL) & 1));
-    }
+    if (aborted) conv_drain(full, NL, consumed, issued, &wbar, &drained, g.status);
     tc5::fence_before();
     __syncthreads();
     if (warp == 0) tc5::dealloc(tmem, TCOLS);
@@ -411,6 +431,7 @@ struct WgradArgs {
     int cin, nout;
     float* out;              // [splits][9 cin][nout]
     int* status;
+    long long wait_ns;
 };
 constexpr int kWgStages = 4;
 
@@ -452,7 +473,7 @@ __global__ void __launch_bounds__(128, 1) k_wgrad(const __grid_constant__ WgradA
         int kb = 0;
         for (; kb < nkb; ++kb) {
             const int s = kb % kWgStages, use = kb / kWgStages;
-            if (use > 0 && !mbar_wait(&empty[s], (unsigned)((use - 1) & 1))) {
+            if (use > 0 && !mbar_wait(&empty[s], (unsigned)((use - 1) & 1), tc5::role_limit(g.wait_ns))) {
                 aborted = 1;
                 break;
             }
@@ -473,7 +494,7 @@ __global__ void __launch_bounds__(128, 1) k_wgrad(const __grid_constant__ WgradA
         int kb = 0;
         for (; kb < nkb; ++kb) {
             const int s = kb % kWgStages;
-            if (!mbar_wait(&full[s], (unsigned)((kb / kWgStages) & 1))) {
+            if (!mbar_wait(&full[s], (unsigned)((kb / kWgStages) & 1), g.wait_ns)) {
                 aborted = 1;
                 break;
             }
@@ -510,7 +531,7 @@ __global__ void __launch_bounds__(128, 1) k_wgrad(const __grid_constant__ WgradA
                                                               __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]));
     }
     if (threadIdx.x == 0 && !good && nkb > 0) {
-        *g.status = 2;
+        atomicAdd(g.status, 1);
         for (int kb = consumed; kb < issued; ++kb) mbar_wait(&full[kb % kWgStages], (unsigned)((kb / kWgStages) & 1));
     }
     tc5::fence_before();
@@ -628,7 +649,7 @@ cudaError_t run_wgrad_a(const WgradArgs& g, int ua, int splits, cudaStream_t st)
 }  // namespace
 
 cudaError_t tc_conv_fwd(const bf16* X, int B, int H, int cin, const bf16* W, int cout, const float* bias, bf16* Y,
-                        int* status, cudaStream_t st)
+                        int* status, long long wait_ns, cudaStream_t st)
 {
     ConvArgs g;
     std::memset(&g, 0, sizeof(g));
@@ -645,6 +666,7 @@ cudaError_t tc_conv_fwd(const bf16* X, int B, int H, int cin, const bf16* W, int
     g.bias = bias;
     g.out = Y;
     g.status = status;
+    g.wait_ns = wait_ns;
     switch (nt) {
         case 32: return run_conv_n<32, false>(g, X, B, st);
         case 64: return run_conv_n<64, false>(g, X, B, st);
@@ -654,7 +676,7 @@ cudaError_t tc_conv_fwd(const bf16* X, int B, int H, int cin, const bf16* W, int
 }
 
 cudaError_t tc_conv_dgrad(const bf16* dZ, int B, int H, int cin, const bf16* Wt, int cout, float* dX, int* status,
-                          cudaStream_t st)
+                          long long wait_ns, cudaStream_t st)
 {
     ConvArgs g;
     std::memset(&g, 0, sizeof(g));
@@ -670,6 +692,7 @@ cudaError_t tc_conv_dgrad(const bf16* dZ, int B, int H, int cin, const bf16* Wt,
     g.nout = cin;
     g.out = dX;
     g.status = status;
+    g.wait_ns = wait_ns;
     switch (nt) {
         case 32: return run_conv_n<32, true>(g, dZ, B, st);
         case 64: return run_conv_n<64, true>(g, dZ, B, st);
@@ -679,7 +702,7 @@ cudaError_t tc_conv_dgrad(const bf16* dZ, int B, int H, int cin, const bf16* Wt,
 }
 
 cudaError_t tc_conv_wgrad(const bf16* X, const bf16* dZ, int B, int H, int cin, int cout, int splits,
-                          long long k_per_split, float* part, int* status, cudaStream_t st)
+                          long long k_per_split, float* part, int* status, long long wait_ns, cudaStream_t st)
 {
     WgradArgs g;
     std::memset(&g, 0, sizeof(g));
@@ -693,6 +716,7 @@ cudaError_t tc_conv_wgrad(const bf16* X, const bf16* dZ, int B, int H, int cin, 
     g.nout = cout;
     g.out = part;
     g.status = status;
+    g.wait_ns = wait_ns;
     switch (cout) {
         case 16: return run_wgrad_a<16, 32>(g, ua, splits, st);
         case 32: return run_wgrad_a<32, 64>(g, ua, splits, st);

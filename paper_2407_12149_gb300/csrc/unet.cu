@@ -550,6 +550,7 @@ struct UnetCtx {
     float *du = nullptr, *dp = nullptr;
     long long* idx = nullptr;
     int* status = nullptr;
+    long long wait_ns = 0;   // bound of the tensor-core kernels' waits (tc_gemm.cuh)
     size_t wpart_elems = 0;
     mgmc_allocator alloc{};
     bool use_alloc = false;
@@ -617,7 +618,7 @@ mgmc_status gemm(UnetCtx* u, const void* A, int lda, const void* B, int ldb, voi
     if (g.splits > 1 && (size_t)g.splits * M * N > u->wpart_elems)
         return unet_fail(MGMC_ERR_STATE, "split-K scratch too small");
     void* out = g.splits > 1 ? (void*)u->wpart : C;
-    UNET_CUDA(tc_gemm_run(g, out, epi, bias, u->status, 0, u->stream));
+    UNET_CUDA(tc_gemm_run(g, out, epi, bias, u->status, u->wait_ns, u->stream));
     if (g.splits > 1) UNET_CUDA(tc_reduce_splits(u->wpart, g.splits, M * N, (float*)C, u->stream));
     return MGMC_OK;
 }
@@ -666,7 +667,7 @@ mgmc_status forward(UnetCtx* u, int B, const bf16* input)
                                                        u->u0);
         if (tc_conv_ok(D.cin, D.cout)) {
             if (tc_conv_fwd(u->layer_in(l), B, Hs, D.cin, u->Wb[l], D.cout, u->theta + u->boff[l], u->act[l], u->status,
-                            st) != cudaSuccess)
+                            u->wait_ns, st) != cudaSuccess)
                 rc = unet_fail(MGMC_ERR_CUDA, "convolution launch failed");
             continue;
         }
@@ -701,10 +702,11 @@ mgmc_status conv_backward(UnetCtx* u, int l, int B, const bf16* input, float* dx
         const int ns = (int)((kb + per - 1) / per);
         if ((size_t)ns * u->Kp[l] * D.cout > u->wpart_elems)
             return unet_fail(MGMC_ERR_STATE, "split-K scratch too small");
-        UNET_CUDA(tc_conv_wgrad(u->layer_in(l), u->dz, B, Hs, D.cin, D.cout, ns, per * 64, u->wpart, u->status, st));
+        UNET_CUDA(tc_conv_wgrad(u->layer_in(l), u->dz, B, Hs, D.cin, D.cout, ns, per * 64, u->wpart, u->status,
+                                u->wait_ns, st));
         k_wt_to_flat<<<dim3((unsigned)((u->K[l] + 31) / 32), (unsigned)((D.cout + 31) / 32)), dim3(32, 32), 0, st>>>(
             u->wpart, ns, u->Kp[l], u->K[l], D.cout, u->grad + u->woff[l]);
-        if (dx) UNET_CUDA(tc_conv_dgrad(u->dz, B, Hs, D.cin, u->Wt[l], D.cout, dx, u->status, st));
+        if (dx) UNET_CUDA(tc_conv_dgrad(u->dz, B, Hs, D.cin, u->Wt[l], D.cout, dx, u->status, u->wait_ns, st));
         UNET_CUDA(cudaGetLastError());
         return MGMC_OK;
     }
@@ -940,6 +942,13 @@ mgmc_status mgmc_unet_set_params(mgmc_unet_handle u, const float* host_in)
     mgmc_status rc = refresh_bf16(u);
     if (rc != MGMC_OK) return rc;
     UNET_CUDA(cudaStreamSynchronize(u->stream));
+    return MGMC_OK;
+}
+
+mgmc_status mgmc_unet_set_wait_limit(mgmc_unet_handle u, int64_t limit_ns)
+{
+    if (!u) return unet_fail(MGMC_ERR_ARG, "bad arguments");
+    u->wait_ns = (long long)limit_ns;
     return MGMC_OK;
 }
 

@@ -77,7 +77,7 @@ EXPORTS = ("mgmc_config_default", "mgmc_create", "mgmc_point_obs_rows", "mgmc_sa
            "mgmc_profile_times", "mgmc_set_band_min_n", "mgmc_set_coarse_threads", "mgmc_create_batch", "mgmc_sample_batch", "mgmc_get_state", "mgmc_destroy",
            "mgmc_tc_gemm", "mgmc_tc_gemm_status", "mgmc_tc_gemm_bounded", "mgmc_unet_create", "mgmc_unet_n_params", "mgmc_unet_get_params",
            "mgmc_unet_set_params", "mgmc_unet_inputs", "mgmc_unet_gradient", "mgmc_unet_train",
-           "mgmc_unet_predict", "mgmc_unet_destroy", "mgmc_check_status", "mgmc_set_wait_limit",
+           "mgmc_unet_predict", "mgmc_unet_set_wait_limit", "mgmc_unet_destroy", "mgmc_check_status", "mgmc_set_wait_limit",
            "mgmc_fine_operator",
            "mgmc_last_error")
 
@@ -135,6 +135,7 @@ def load():
                                   ctypes.c_int, ctypes.c_float, ctypes.c_uint64, ctypes.c_void_p]
     L.mgmc_unet_predict.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int]
     L.mgmc_unet_destroy.argtypes = [ctypes.c_void_p]
+    L.mgmc_unet_set_wait_limit.argtypes = [ctypes.c_void_p, ctypes.c_int64]
     L.mgmc_destroy.argtypes = [ctypes.c_void_p]
     L.mgmc_check_status.argtypes = [ctypes.c_void_p, ctypes.c_void_p]
     L.mgmc_fine_operator.argtypes = [ctypes.POINTER(mgmc_config), _F64P, ctypes.c_double, _F64P]
@@ -615,6 +616,10 @@ class Unet:
                                         ctypes.c_void_p(out.data_ptr()),
                                         MGMC_FP32 if precision == "fp32" else MGMC_FP64))
         return out
+
+    def set_wait_limit(self, limit_ns: int):
+        """Bound of the tensor-core kernels' waits (mgmc_unet_set_wait_limit; tests)."""
+        _check(load().mgmc_unet_set_wait_limit(self.h, int(limit_ns)))
 
     def close(self):
         if getattr(self, "h", None):
