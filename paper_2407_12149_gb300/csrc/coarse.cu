@@ -1018,11 +1018,11 @@ __global__ void k_qoi_batch(const QoiJob<T>* __restrict__ jobs)
     // the QoI sites and weights never change: the first kQoiPre of each thread are loaded
     // before the wait on the preceding launch, the state after it (same summation order)
     constexpr int kQoiPre = 4;
-    const QoiJob<T> J = jobs[blockIdx.y];
+    const QoiJob<T> J = jobs[blockIdx.x];
     // the chain's own number of CTAs: its sum does not depend on the other chains of a launch
     const int nb = qoi_ctas(J.n_qoi);
-    if ((int)blockIdx.x >= nb) return;
-    const int t0 = blockIdx.x * blockDim.x + threadIdx.x, st = nb * blockDim.x;
+    if ((int)blockIdx.y >= nb) return;
+    const int t0 = blockIdx.y * blockDim.x + threadIdx.x, st = nb * blockDim.x;
     long long site[kQoiPre];
     double w[kQoiPre];
 #pragma unroll
@@ -1046,7 +1046,7 @@ __global__ void k_qoi_batch(const QoiJob<T>* __restrict__ jobs)
     if (threadIdx.x != 0) return;
     double q = part[0];
     if (nb > 1) {
-        J.part[blockIdx.x] = q;
+        J.part[blockIdx.y] = q;
         __threadfence();
         if (atomicAdd(J.ticket, 1) != nb - 1) return;
         __threadfence();
@@ -1109,7 +1109,8 @@ void launch_coarse(const CoarseJob<T>* jobs, int n, int dim, int threads, size_t
 template <typename T>
 void launch_qoi_batch(const QoiJob<T>* jobs, int n, int max_qoi, cudaStream_t st, int& launches)
 {
-    launch_pdl(k_qoi_batch<T>, dim3((unsigned)qoi_ctas(max_qoi), (unsigned)n), dim3(256), 0, st, jobs);
+    // chains along x: a batch may hold 65 536, one more than gridDim.y takes
+    launch_pdl(k_qoi_batch<T>, dim3((unsigned)n, (unsigned)qoi_ctas(max_qoi)), dim3(256), 0, st, jobs);
     ++launches;
 }
 
