@@ -24,6 +24,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 
 #include "tc5.cuh"
@@ -279,12 +280,16 @@ template <int BN>
 cudaError_t launch(const TcGemm& g, void* C, int epi, const float* bias, int* status, long long wait_ns,
                    cudaStream_t st)
 {
-    static bool prepared = false;  // per process (one device in use at a time)
-    if (!prepared) {
-        cudaError_t e = cudaFuncSetAttribute(k_tc_gemm<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)gemm_smem<BN>());
+    // the shared-memory opt-in, once per device (each of the first 64 has a bit)
+    static std::atomic<unsigned long long> prepared{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (!(prepared.load() & bit)) {
+        e = cudaFuncSetAttribute(k_tc_gemm<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gemm_smem<BN>());
         if (e != cudaSuccess) return e;
-        prepared = true;
+        prepared.fetch_or(bit);
     }
     const long long tiles = (long long)((g.M + kBM - 1) / kBM) * ((g.N + BN - 1) / BN) * g.splits;
     const unsigned grid = (unsigned)std::min<long long>(tiles, sm_count());

@@ -29,6 +29,7 @@
 #include <cstdint>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -796,6 +797,40 @@ float host_loss(UnetCtx* u, int B)
     return (float)(s / ((double)B * u->n * u->n));
 }
 
+// Partial sums of split products are stream-ordered memory of one pool per device: products of
+// several streams and threads never share them, and the pool keeps at most kSplitKeep bytes
+// between calls (memory given back at every synchronisation costs a mapping in the next call).
+constexpr unsigned long long kSplitKeep = 512ull << 20;
+cudaError_t split_pool(cudaMemPool_t* pool)
+{
+    static std::mutex mu;
+    static std::map<int, cudaMemPool_t> pools;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = pools.find(dev);
+    if (it == pools.end()) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t p = nullptr;
+        e = cudaMemPoolCreate(&p, &props);
+        if (e != cudaSuccess) return e;
+        unsigned long long keep = kSplitKeep;
+        e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e != cudaSuccess) {
+            cudaMemPoolDestroy(p);
+            return e;
+        }
+        it = pools.emplace(dev, p).first;
+    }
+    *pool = it->second;
+    return cudaSuccess;
+}
+
 }  // namespace
 }  // namespace mgmc
 
@@ -1090,8 +1125,6 @@ mgmc_status mgmc_tc_gemm_status(void* stream)
 mgmc_status mgmc_tc_gemm_bounded(const void* A, int lda, const void* B, int ldb, void* C, int M, int N, int K,
                                  int splits, int epilogue, const float* bias, void* stream, int64_t wait_ns)
 {
-    static thread_local float* part = nullptr;
-    static thread_local size_t part_bytes = 0;
     if (!A || !B || !C || M <= 0 || N <= 0 || K <= 0 || splits < 1 || (epilogue & ~7) ||
         ((epilogue & kEpiBias) && !bias))
         return unet_fail(MGMC_ERR_ARG, "mgmc_tc_gemm: bad arguments");
@@ -1101,20 +1134,19 @@ mgmc_status mgmc_tc_gemm_bounded(const void* A, int lda, const void* B, int ldb,
     TcGemm g;
     if (!tc_gemm_plan(&g, A, lda, B, ldb, M, N, K, splits))
         return unet_fail(MGMC_ERR_ARG, "mgmc_tc_gemm: TMA descriptor encoding failed (alignment, lda/ldb)");
-    void* out = C;
-    if (g.splits > 1) {
-        const size_t need = sizeof(float) * (size_t)g.splits * M * N;
-        if (need > part_bytes) {
-            if (part) cudaFree(part);
-            part = nullptr;
-            part_bytes = 0;
-            UNET_CUDA(cudaMalloc(&part, need));
-            part_bytes = need;
-        }
-        out = part;
+    if (g.splits == 1) {
+        UNET_CUDA(tc_gemm_run(g, C, epilogue, bias, nullptr, (long long)wait_ns, st));
+        return MGMC_OK;
     }
-    UNET_CUDA(tc_gemm_run(g, out, epilogue, bias, nullptr, (long long)wait_ns, st));
-    if (g.splits > 1) UNET_CUDA(tc_reduce_splits(part, g.splits, (long long)M * N, (float*)C, st));
+    cudaMemPool_t pool;
+    float* part = nullptr;
+    UNET_CUDA(split_pool(&pool));
+    UNET_CUDA(cudaMallocFromPoolAsync((void**)&part, sizeof(float) * (size_t)g.splits * M * N, pool, st));
+    cudaError_t e = tc_gemm_run(g, part, epilogue, bias, nullptr, (long long)wait_ns, st);
+    if (e == cudaSuccess) e = tc_reduce_splits(part, g.splits, (long long)M * N, (float*)C, st);
+    const cudaError_t ef = cudaFreeAsync(part, st);
+    UNET_CUDA(e);
+    UNET_CUDA(ef);
     return MGMC_OK;
 }
 
