@@ -375,7 +375,8 @@ mgmc_status mgmc_unet_destroy(mgmc_unet_handle u);
  * (lda, ldb >= K and multiples of 8; base addresses 16-byte aligned).
  * epilogue: bit 0 add bias (device float [N]), bit 1 ReLU, bit 2 store BF16
  * (else float).  splits > 1 (FP32 output only): the K range is cut into
- * `splits` parts summed in a fixed order (deterministic).  C: device [M][N].
+ * `splits` parts summed in a fixed order (deterministic).  C: device [M][N], aligned
+ * to its elements (it may be a view; 16-byte stores are used where its rows allow).
  * Asynchronous on stream.  A bounded wait (1 s) inside the kernel that gives up
  * leaves rows of tiles of C unwritten (splits > 1: C undefined) and is reported by
  * mgmc_tc_gemm_status.

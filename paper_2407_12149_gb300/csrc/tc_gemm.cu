@@ -77,10 +77,10 @@ __device__ __forceinline__ Tile tile_at(long long t, int M, int N, int K, int k_
     return T;
 }
 
-// one tile from the accumulator at `tmem`: this warp's 32 rows
+// one tile from the accumulator at `tmem`: this warp's 32 rows; vec: the rows of C start on 16 bytes
 template <int BN>
 __device__ __forceinline__ void gemm_epilogue(unsigned tmem, const Tile& T, void* C, int M, int N, int epi,
-                                              const float* __restrict__ bias)
+                                              bool vec, const float* __restrict__ bias)
 {
     const int quarter = (threadIdx.x >> 5) & 3;   // TMEM lanes 32 (warp % 4) .. + 31 are the warp's
     const int row = T.m0 + quarter * 32 + (int)(threadIdx.x & 31);
@@ -99,7 +99,7 @@ __device__ __forceinline__ void gemm_epilogue(unsigned tmem, const Tile& T, void
         }
         if (epi & kEpiBF16) {
             __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(C) + (long long)row * N + col0;
-            if (col0 + 32 <= N && ((N & 7) == 0)) {
+            if (vec && col0 + 32 <= N) {
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
                     __nv_bfloat162 h[4];
@@ -114,7 +114,7 @@ __device__ __forceinline__ void gemm_epilogue(unsigned tmem, const Tile& T, void
             }
         } else {
             float* out = reinterpret_cast<float*>(C) + (long long)T.z * M * N + (long long)row * N + col0;
-            if (col0 + 32 <= N && ((N & 3) == 0)) {
+            if (vec && col0 + 32 <= N) {
 #pragma unroll
                 for (int q = 0; q < 8; ++q)
                     *reinterpret_cast<float4*>(out + 4 * q) = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
@@ -130,7 +130,7 @@ __device__ __forceinline__ void gemm_epilogue(unsigned tmem, const Tile& T, void
 template <int BN>
 __global__ void __launch_bounds__(kThreads, 1)
     k_tc_gemm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, void* C, int M,
-              int N, int K, int k_per_split, long long tiles, int epi, const float* __restrict__ bias, int* status,
+              int N, int K, int k_per_split, long long tiles, int epi, int vec, const float* __restrict__ bias, int* status,
               long long wait_ns)
 {
     constexpr int A_BYTES = kBM * kBK * 2;
@@ -226,7 +226,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc5::fence_after();
-            gemm_epilogue<BN>(tmem + (unsigned)(bp.slot * BN), tile_at<BN>(t, M, N, K, k_per_split), C, M, N, epi, bias);
+            gemm_epilogue<BN>(tmem + (unsigned)(bp.slot * BN), tile_at<BN>(t, M, N, K, k_per_split), C, M, N, epi, vec != 0,
+                              bias);
             tc5::fence_before();
             __syncwarp();
             if (lane == 0) tc5::arrive(&tempty[bp.slot]);
@@ -293,8 +294,11 @@ cudaError_t launch(const TcGemm& g, void* C, int epi, const float* bias, int* st
     }
     const long long tiles = (long long)((g.M + kBM - 1) / kBM) * ((g.N + BN - 1) / BN) * g.splits;
     const unsigned grid = (unsigned)std::min<long long>(tiles, sm_count());
-    k_tc_gemm<BN><<<grid, kThreads, gemm_smem<BN>(), st>>>(g.a, g.b, C, g.M, g.N, g.K, g.k_per_split, tiles, epi, bias,
-                                                          status, wait_ns);
+    // 16-byte stores where every row starts on 16 bytes: C and the row pitch (C may be a view)
+    const size_t elem = (epi & kEpiBF16) ? 2 : 4;
+    const int vec = (reinterpret_cast<uintptr_t>(C) & 15) == 0 && ((size_t)g.N * elem & 15) == 0;
+    k_tc_gemm<BN><<<grid, kThreads, gemm_smem<BN>(), st>>>(g.a, g.b, C, g.M, g.N, g.K, g.k_per_split, tiles, epi, vec,
+                                                          bias, status, wait_ns);
     return cudaGetLastError();
 }
 

@@ -1130,6 +1130,8 @@ mgmc_status mgmc_tc_gemm_bounded(const void* A, int lda, const void* B, int ldb,
         return unet_fail(MGMC_ERR_ARG, "mgmc_tc_gemm: bad arguments");
     if (splits > 1 && epilogue != kEpiF32)
         return unet_fail(MGMC_ERR_ARG, "mgmc_tc_gemm: split-K needs the plain FP32 epilogue");
+    if (reinterpret_cast<uintptr_t>(C) % ((epilogue & kEpiBF16) ? 2 : 4) || reinterpret_cast<uintptr_t>(bias) % 4)
+        return unet_fail(MGMC_ERR_ARG, "mgmc_tc_gemm: C or bias is not aligned to its elements");
     cudaStream_t st = (cudaStream_t)stream;
     TcGemm g;
     if (!tc_gemm_plan(&g, A, lda, B, ldb, M, N, K, splits))
