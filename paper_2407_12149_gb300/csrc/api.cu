@@ -129,11 +129,18 @@ struct mgmc_ctx {
     // batch handle: per-chain handles and the job tables of the batched launches
     std::vector<mgmc_ctx*> sub;
     int n_depth = 0;
-    std::vector<void*> jobs_tile, jobs_lrd, jobs_lru;
+    std::vector<void*> jobs_tile;
     std::vector<void*> maps_fwd, maps_bwd;   // TileMaps per tile job, per depth
-    std::vector<int> njob_tile, nblk_tile, njob_lrd, nblk_lrd, njob_lru, nblk_lru;
-    std::vector<int> per_tile, per_lrd, per_lru;
-    std::vector<int> cl_lrd, cl_lru;   // cluster size of the low-rank launches (1: none)
+    std::vector<int> njob_tile, nblk_tile, per_tile;
+    // low-rank launches per depth, forward and backward: [0] after the tile kernels (z partials),
+    // [1] after the streaming kernels (the state is read)
+    struct LowrankTable {
+        void* jobs = nullptr;
+        int njobs = 0, per = 0, nblocks = 0;
+        int cluster = 1;   // CTAs of a job launched as one cluster
+    };
+    std::vector<LowrankTable> lr_d[2], lr_u[2];
+    bool streamed(int d) const { return (d == 0 && stream_fine) || s9_use[d]; }
     // FP32 finest grids: the streaming kernels (stream2d.cu) instead of depth-0 tiles
     bool stream_fine = false;
     bool fine0 = true;    // the depth-0 grids have the 5-point finite-difference form
@@ -513,8 +520,8 @@ void enqueue_cycle_batch(mgmc_ctx* h, cudaStream_t s, int& launches)
                                  h->njob_tile[d], h->per_tile[d], h->nblk_tile[d], d == 0 && h->fine0, false, d > 0,
                                  s, launches);
         if (prof && d == 0) cudaEventRecordWithFlags(h->ev[1], s, cudaEventRecordExternal);
-        launch_lowrank_batch<T>((const LowrankJob<T>*)h->jobs_lrd[d], h->njob_lrd[d], h->per_lrd[d], h->nblk_lrd[d],
-                                h->cl_lrd[d], true, s, launches);
+        const auto& lr = h->lr_d[h->streamed(d)][d];
+        launch_lowrank_batch<T>((const LowrankJob<T>*)lr.jobs, lr.njobs, lr.per, lr.nblocks, lr.cluster, true, s, launches);
     }
     launch_coarse<T>((const CoarseJob<T>*)h->jobs_coarse, nc, 2, coarse_cta(h), h->batch_coarse_smem, s, launches);
     for (int d = h->n_depth - 1; d >= 0; --d) {
@@ -530,8 +537,8 @@ void enqueue_cycle_batch(mgmc_ctx* h, cudaStream_t s, int& launches)
                                  h->njob_tile[d], h->per_tile[d], h->nblk_tile[d], d == 0 && h->fine0, true, false, s,
                                  launches);
         if (prof && d == 0) cudaEventRecordWithFlags(h->ev[3], s, cudaEventRecordExternal);
-        launch_lowrank_batch<T>((const LowrankJob<T>*)h->jobs_lru[d], h->njob_lru[d], h->per_lru[d], h->nblk_lru[d],
-                                h->cl_lru[d], false, s, launches);
+        const auto& lr = h->lr_u[h->streamed(d)][d];
+        launch_lowrank_batch<T>((const LowrankJob<T>*)lr.jobs, lr.njobs, lr.per, lr.nblocks, lr.cluster, false, s, launches);
     }
     launch_qoi_batch<T>((const QoiJob<T>*)h->jobs_qoi, nc, h->max_qoi, s, launches);
 }
@@ -1412,6 +1419,47 @@ mgmc_status build_gibbs_tables(mgmc_ctx* h)
     return MGMC_OK;
 }
 
+// common block count of the jobs of one launch (0: they differ)
+template <typename V, typename F>
+int common_count(const V& v, F count)
+{
+    const int per = v.empty() ? 0 : count(v[0]);
+    for (const auto& j : v)
+        if (count(j) != per) return 0;
+    return per;
+}
+
+// The low-rank launch of depth d.  state: after the streaming kernels, which leave no z partials --
+// the blocks of a job then read the state and are one cluster, of one size for all jobs.  The
+// partials are the same products, added in the same order: the same bits either way.  After the
+// tile kernels of a depth that could also stream they are used (32 FP32 chains of 63^2 to 511^2, 4
+// cycles 889 -> 881 us; 127^2 with ball observations 17 -> 9 us a launch).
+template <typename T>
+mgmc_ctx::LowrankTable lowrank_table(mgmc_ctx* h, const std::vector<mgmc_ctx*>& chains, int d, bool down, bool state,
+                                     mgmc_status& st)
+{
+    mgmc_ctx::LowrankTable t;
+    std::vector<LowrankJob<T>> jobs;
+    auto rows_of = [&](const DevLevel<T>& L) { return down ? std::max(L.g_rows[0], L.h_rows) : L.g_rows[1]; };
+    auto has = [&](const mgmc_ctx* c) { return c->L - 1 - d > c->top && c->m > 0; };
+    if (state)
+        for (mgmc_ctx* c : chains)
+            if (has(c)) t.cluster = std::max(t.cluster, lowrank_cluster(rows_of(levels_of<T>(c)[c->L - 1 - d])));
+    for (mgmc_ctx* c : chains) {
+        if (!has(c)) continue;
+        const auto& lv = levels_of<T>(c);
+        DevLevel<T> L = lv[c->L - 1 - d];
+        if (state) L.zparts = nullptr;
+        const int nb = state ? t.cluster : lowrank_blocks(rows_of(L));
+        jobs.push_back({L, lv[c->L - 2 - d], c->P, t.nblocks, nb});
+        t.nblocks += nb;
+    }
+    t.njobs = (int)jobs.size();
+    t.per = common_count(jobs, [](const LowrankJob<T>& j) { return j.nblocks; });
+    t.jobs = upload(h, jobs, st);
+    return t;
+}
+
 template <typename T>
 mgmc_status build_batch_tables(mgmc_ctx* h)
 {
@@ -1438,12 +1486,10 @@ mgmc_status build_batch_tables(mgmc_ctx* h)
     for (int d = 0; d < depth; ++d) {
         std::vector<TileJob<T>> tj;
         std::vector<TileMaps> mf, mb;
-        std::vector<LowrankJob<T>> ld, lu;
-        int tiles = 0, bd = 0, bu = 0;
+        int tiles = 0;
         // FP32 9-point grids below the finest: the streaming band kernels can take this
         // depth (which of the two kernel families runs is set by band_min_n, see
-        // apply_band_min); the low-rank steps then read the state at the observation
-        // entries, whichever family wrote it
+        // apply_band_min); the low-rank steps then read the state at the observation entries
         bool s9 = false;
         int s9_minn = 0;
         if constexpr (std::is_same<T, float>::value) {
@@ -1498,16 +1544,10 @@ mgmc_status build_batch_tables(mgmc_ctx* h)
                 h->s9_grid.back() = stream9_grid(strips);
             }
         }
-        // grids without z partials: the blocks of a low-rank job are one cluster, of one size
-        // for all jobs of the launch
-        const bool zst = (d == 0 && h->stream_fine) || s9;
-        int cld = 1, clu = 1;
-        for (mgmc_ctx* c : chains) {
-            const int l = c->L - 1 - d;
-            if (l <= c->top || c->m == 0) continue;
-            const DevLevel<T>& Lh = levels_of<T>(c)[l];
-            cld = std::max(cld, lowrank_cluster(std::max(Lh.g_rows[0], Lh.h_rows)));
-            clu = std::max(clu, lowrank_cluster(Lh.g_rows[1]));
+        for (int f = 0; f < 2; ++f) {
+            const bool have = f ? (d == 0 && h->stream_fine) || s9 : !(d == 0 && h->stream_fine);
+            h->lr_d[f].push_back(have ? lowrank_table<T>(h, chains, d, true, f == 1, st) : mgmc_ctx::LowrankTable{});
+            h->lr_u[f].push_back(have ? lowrank_table<T>(h, chains, d, false, f == 1, st) : mgmc_ctx::LowrankTable{});
         }
         for (mgmc_ctx* c : chains) {
             const int l = c->L - 1 - d;
@@ -1523,40 +1563,13 @@ mgmc_status build_batch_tables(mgmc_ctx* h)
             mb.emplace_back();
             if (!make_tile_maps<T>(Lh, Ch, false, &mf.back()) || !make_tile_maps<T>(Lh, Ch, true, &mb.back()))
                 return fail(MGMC_ERR_CUDA, "TMA descriptor encoding failed");
-            if (c->m > 0) {
-                DevLevel<T> Lz = Lh;
-                if (zst) Lz.zparts = nullptr;   // the low-rank kernel reads the state
-                const int nd = zst ? cld : lowrank_blocks(std::max(Lh.g_rows[0], Lh.h_rows));
-                const int nu = zst ? clu : lowrank_blocks(Lh.g_rows[1]);
-                ld.push_back({Lz, Ch, c->P, bd, nd});
-                bd += nd;
-                lu.push_back({Lz, Ch, c->P, bu, nu});
-                bu += nu;
-            }
         }
-        h->cl_lrd.push_back(zst ? cld : 1);
-        h->cl_lru.push_back(zst ? clu : 1);
-        // common block count of the jobs of one launch (0: they differ)
-        auto common = [](const auto& v, auto count) {
-            int per = v.empty() ? 0 : count(v[0]);
-            for (const auto& j : v)
-                if (count(j) != per) return 0;
-            return per;
-        };
-        h->per_tile.push_back(common(tj, [](const TileJob<T>& j) { return j.ntiles; }));
-        h->per_lrd.push_back(common(ld, [](const LowrankJob<T>& j) { return j.nblocks; }));
-        h->per_lru.push_back(common(lu, [](const LowrankJob<T>& j) { return j.nblocks; }));
+        h->per_tile.push_back(common_count(tj, [](const TileJob<T>& j) { return j.ntiles; }));
         h->jobs_tile.push_back(upload(h, tj, st));
         h->maps_fwd.push_back(upload(h, mf, st));
         h->maps_bwd.push_back(upload(h, mb, st));
         h->njob_tile.push_back((int)tj.size());
         h->nblk_tile.push_back(tiles);
-        h->jobs_lrd.push_back(upload(h, ld, st));
-        h->njob_lrd.push_back((int)ld.size());
-        h->nblk_lrd.push_back(bd);
-        h->jobs_lru.push_back(upload(h, lu, st));
-        h->njob_lru.push_back((int)lu.size());
-        h->nblk_lru.push_back(bu);
     }
     std::vector<CoarseJob<T>> cj;
     std::vector<QoiJob<T>> qj;
