@@ -116,7 +116,7 @@ struct mgmc_ctx {
     double* gain = nullptr;
     double* e0 = nullptr;
     bool fused = false;   // 2D, nu1 = nu2 = 1: fused tile kernels on the grids above coarse_max_n
-    bool gibbs_fused = false; // 2D Gibbs sampler, nu1 = nu2 = 1: the finest grid's fused sweep kernels
+    bool gibbs_fused = false; // Gibbs sampler on an FP32 9-point grid: the fused sweep kernels (mgmc_create)
     bool recursive = false;   // W-cycle or radius-2 grids: general kernels, cycle enqueued recursively
     // recursive path, 2D: grids 0..small_top run in one k_cycle_small launch per visit of
     // grid small_top (-1: none); the phase lists of the cycle's visits, in cycle order
@@ -174,7 +174,6 @@ namespace {
 
 template <typename T>
 mgmc_status build_batch_tables(mgmc_ctx* h);
-template <typename T>
 mgmc_status build_gibbs_tables(mgmc_ctx* h);
 void apply_band_min(mgmc_ctx* h);
 
@@ -396,8 +395,7 @@ mgmc_status build_device_levels(mgmc_ctx* h, const HostProblem& hp)
         D.x2 = (T*)h->buf.get(fbytes);
         if (!D.x2) return fail(MGMC_ERR_OOM, "allocator returned NULL");
         CUDA_TRY(cudaMemsetAsync(D.x2, 0, fbytes, h->buf.stream));
-        const int TX = D.fine ? TileShape<T, true>::TX : TileShape<T, false>::TX;
-        D.ntx = (D.n + TX - 1) / TX;
+        D.ntx = (D.n + TileShape<T, false>::TX - 1) / TileShape<T, false>::TX;
     }
     // fused tile path: second state buffer, per-tile observation entries, G/H in T, B^T G
     if (h->fused) {
@@ -677,14 +675,9 @@ void enqueue_cycle(mgmc_ctx* h, cudaStream_t s, int& launches)
         D2.x = D.x2;
         for (int dir = 0; dir < 2; ++dir) {
             if (prof) cudaEventRecordWithFlags(h->ev[2 * dir], s, cudaEventRecordExternal);
-            if (h->stream_fine)
-                launch_stream_fine((const StreamJob*)h->jobs_stream,
-                                   (const StreamMaps*)(dir ? h->maps_sbwd : h->maps_sfwd), h->njob_stream,
-                                   h->stream_strips, h->stream_ctas, dir == 1, s, launches);
-            else
-                launch_tile_batch<T>((const TileJob<T>*)h->jobs_tile[0],
-                                     (const TileMaps*)(dir ? h->maps_bwd[0] : h->maps_fwd[0]), 1, h->per_tile[0],
-                                     h->nblk_tile[0], h->fine0, dir == 1, false, s, launches);
+            launch_tile_batch<T>((const TileJob<T>*)h->jobs_tile[0],
+                                 (const TileMaps*)(dir ? h->maps_bwd[0] : h->maps_fwd[0]), 1, h->per_tile[0],
+                                 h->nblk_tile[0], false, dir == 1, false, s, launches);
             if (prof) cudaEventRecordWithFlags(h->ev[2 * dir + 1], s, cudaEventRecordExternal);
             launch_lowrank<T>(dir ? D : D2, P, dir, (unsigned)dir, false, s, launches);
         }
@@ -974,7 +967,13 @@ mgmc_status mgmc_create(const mgmc_config* cfg_in, const mgmc_allocator* alloc, 
     h->n0 = hp.n0;
     h->f_norm = hp.f_norm;
     h->fused = cfg.dim == 2 && cfg.nu1 == 1 && cfg.nu2 == 1 && !cfg.gibbs && !h->recursive;
-    h->gibbs_fused = cfg.dim == 2 && cfg.nu1 == 1 && cfg.nu2 == 1 && cfg.gibbs && !h->recursive;
+    // Gibbs sampler: one launch per colour, or the tile kernels' fused sweeps where those are faster
+    // (us a step, 8 observations, per colour / fused; one box): FP32 9-point 15^2 27.0 / 25.0, 31^2 27.0 / 25.0,
+    // 127^2 27.0 / 27.0, 255^2 29.7 / 29.0, 511^2 33.5 / 33.2, 1023^2 49.9 / 61.9; FP32 5-point (streaming
+    // kernels) 31^2 18.8 / 25.0, 255^2 24.5 / 29.1, 1023^2 37.6 / 44.3; FP64 5-point 31^2 20.9 / 43.4,
+    // 1023^2 109 / 206; FP64 9-point 31^2 31.1 / 43.4, 1023^2 125 / 327
+    h->gibbs_fused = cfg.dim == 2 && cfg.nu1 == 1 && cfg.nu2 == 1 && cfg.gibbs && !h->recursive &&
+                     cfg.precision == MGMC_FP32 && cfg.disc == MGMC_Q1 && cfg.n <= 255;
     auto cleanup = [&](mgmc_status s) {
         h->buf.release();
         delete h;
@@ -1073,7 +1072,7 @@ mgmc_status mgmc_create(const mgmc_config* cfg_in, const mgmc_allocator* alloc, 
         if (st != MGMC_OK) return cleanup(st);
     } else {
         if (h->gibbs_fused) {
-            st = h->fp32() ? build_gibbs_tables<float>(h) : build_gibbs_tables<double>(h);
+            st = build_gibbs_tables(h);
             if (st != MGMC_OK) return cleanup(st);
         }
         h->max_qoi = h->n_qoi;
@@ -1355,7 +1354,7 @@ void apply_band_min(mgmc_ctx* h)
     for (size_t d = 0; d < h->s9_ok.size(); ++d) h->s9_use[d] = h->s9_ok[d] && h->s9_minn[d] >= band_min;
 }
 
-// the finest grid's FP32 5-point grids of `chains` as streaming jobs
+// the FP32 5-point finest grids of `chains` as streaming jobs
 mgmc_status build_stream_jobs(mgmc_ctx* h, const std::vector<mgmc_ctx*>& chains)
 {
     mgmc_status st = MGMC_OK;
@@ -1393,28 +1392,24 @@ mgmc_status build_stream_jobs(mgmc_ctx* h, const std::vector<mgmc_ctx*>& chains)
     return MGMC_OK;
 }
 
-// the sweep kernels' table of a Gibbs handle: its finest grid
-template <typename T>
+// the tile kernels' table of a Gibbs handle: its finest grid
 mgmc_status build_gibbs_tables(mgmc_ctx* h)
 {
-    const DevLevel<T>& Lh = levels_of<T>(h)[h->L - 1];
-    const DevLevel<T>& Ch = levels_of<T>(h)[h->L - 2];
-    h->fine0 = Lh.fine != 0;
-    if constexpr (std::is_same<T, float>::value)
-        if (h->fine0) return build_stream_jobs(h, {h});
+    const DevLevel<float>& Lh = h->lf[h->L - 1];
+    const DevLevel<float>& Ch = h->lf[h->L - 2];
     mgmc_status st = MGMC_OK;
-    const int TY = Lh.fine ? TileShape<T, true>::TY : TileShape<T, false>::TY;
+    constexpr int TY = TileShape<float, false>::TY;
     const int tiles = Lh.ntx * ((Lh.n + TY - 1) / TY);
     TileMaps mf, mb;
-    if (!make_tile_maps<T>(Lh, Ch, false, &mf) || !make_tile_maps<T>(Lh, Ch, true, &mb))
+    if (!make_tile_maps<float>(Lh, Ch, false, &mf) || !make_tile_maps<float>(Lh, Ch, true, &mb))
         return fail(MGMC_ERR_CUDA, "TMA descriptor encoding failed");
-    h->jobs_tile.push_back(upload(h, std::vector<TileJob<T>>{{Lh, Ch, h->P, 0, tiles}}, st));
+    h->jobs_tile.push_back(upload(h, std::vector<TileJob<float>>{{Lh, Ch, h->P, 0, tiles}}, st));
     h->maps_fwd.push_back(upload(h, std::vector<TileMaps>{mf}, st));
     h->maps_bwd.push_back(upload(h, std::vector<TileMaps>{mb}, st));
     h->per_tile.push_back(tiles);
     h->nblk_tile.push_back(tiles);
     if (st != MGMC_OK) return fail(st, "tile table upload failed");
-    cudaError_t e = tile_prepare_batch<T>();
+    cudaError_t e = tile_prepare_batch<float>();
     if (e != cudaSuccess) return fail(MGMC_ERR_CUDA, std::string("tile kernel set-up: ") + cudaGetErrorString(e));
     return MGMC_OK;
 }
