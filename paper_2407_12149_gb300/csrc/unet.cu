@@ -576,7 +576,7 @@ struct UnetCtx {
     void* get(size_t bytes)
     {
         void* p = nullptr;
-        bytes = (bytes + 255) / 256 * 256;
+        bytes = (std::max<size_t>(bytes, 1) + 255) / 256 * 256;
         if (use_alloc)
             p = alloc.alloc(bytes, stream, alloc.ctx);
         else if (cudaMalloc(&p, bytes) != cudaSuccess)
@@ -905,7 +905,9 @@ mgmc_status mgmc_unet_create(int n, int c0, int max_batch, uint64_t seed, const 
     cudaMemsetAsync(u->status, 0, sizeof(int), u->stream);
     // buffers for max_batch samples
     const int B = max_batch;
-    size_t col_elems = 0, dact_max = 0, dz_max = 0, dwt_max = 0;
+    // im2col forms (col, colT, dzT, dwt, dcol): only the layers that tc_conv.cu does not take, dcol
+    // only where a gradient goes further down
+    size_t col_elems = 0, dcol_elems = 0, dact_max = 0, dz_max = 0, dzt_max = 0, dwt_max = 0;
     for (int l = 0; l < kLayers; ++l) {
         const long long P = u->Ps(u->L[l].level, B);
         u->Wb[l] = (bf16*)u->get(sizeof(bf16) * (size_t)u->L[l].cout * u->Kp[l]);
@@ -913,9 +915,12 @@ mgmc_status mgmc_unet_create(int n, int c0, int max_batch, uint64_t seed, const 
         u->act[l] = (bf16*)u->get(sizeof(bf16) * (size_t)P * u->L[l].cout);
         u->dact[l] = (float*)u->get(sizeof(float) * (size_t)P * u->L[l].cout);
         if (!u->Wb[l] || !u->Wt[l] || !u->act[l] || !u->dact[l]) return fail_all(MGMC_ERR_OOM, "allocation failed");
-        col_elems = std::max(col_elems, (size_t)P * u->Kp[l]);
         dact_max = std::max(dact_max, (size_t)P * u->L[l].cin);
         dz_max = std::max(dz_max, (size_t)P * u->L[l].cout);
+        if (tc_conv_ok(u->L[l].cin, u->L[l].cout)) continue;
+        col_elems = std::max(col_elems, (size_t)P * u->Kp[l]);
+        if (l > 0) dcol_elems = std::max(dcol_elems, (size_t)P * u->Kp[l]);
+        dzt_max = std::max(dzt_max, (size_t)P * u->L[l].cout);
         dwt_max = std::max(dwt_max, (size_t)u->Kp[l] * u->L[l].cout);
     }
     // split-K partials: splits <= 304 / ceil(Kp / 128), so splits * Kp * cout <= 304 * 128 * 256
@@ -933,9 +938,9 @@ mgmc_status mgmc_unet_create(int n, int c0, int max_batch, uint64_t seed, const 
     u->tgt = (float*)u->get(sizeof(float) * (size_t)B * n * n);
     u->col = (bf16*)u->get(sizeof(bf16) * col_elems);
     u->colT = (bf16*)u->get(sizeof(bf16) * col_elems);
-    u->dcol = (float*)u->get(sizeof(float) * col_elems);
+    u->dcol = (float*)u->get(sizeof(float) * dcol_elems);
     u->dz = (bf16*)u->get(sizeof(bf16) * dz_max);
-    u->dzT = (bf16*)u->get(sizeof(bf16) * dz_max);
+    u->dzT = (bf16*)u->get(sizeof(bf16) * dzt_max);
     u->dwt = (float*)u->get(sizeof(float) * dwt_max);
     u->wpart = (float*)u->get(sizeof(float) * u->wpart_elems);
     u->part = (float*)u->get(sizeof(float) * (kLossOff + kRedBlocks));
