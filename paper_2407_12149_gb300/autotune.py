@@ -28,7 +28,8 @@ from typing import Callable, Dict, Iterable, Optional, Sequence, Tuple
 # a band threshold above every grid: the tile kernels only
 TILES_ONLY = 1 << 20
 DEFAULTS = {"coarse_max_n": 31, "band_min_n": 0, "coarse_threads": 0}
-COARSE_THREADS = (0, 128, 256, 512, 1024)
+# up to the kernel's limit (512 in FP32, 256 in FP64, where 512 runs as 256; see mgmc_set_coarse_threads)
+COARSE_THREADS = (0, 128, 256, 512)
 
 
 def pick_fastest(timings: Dict[int, float]) -> int:
@@ -230,7 +231,8 @@ def autotune(problems: Sequence, precision: str = "fp32", coarse_candidates: Ite
         s = make_sampler(problems, c)
         try:
             b, ms = tune_band_min_n(s, band_candidates(problems, c), timer=timer)
-            t, tms = tune_coarse_threads(s, timer=timer)
+            threads = [k for k in COARSE_THREADS if precision == "fp32" or k <= 256]
+            t, tms = tune_coarse_threads(s, threads, timer=timer)
         finally:
             s.close()
         for k, v in ms.items():

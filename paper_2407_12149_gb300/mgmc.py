@@ -520,7 +520,7 @@ class BatchSampler:
         mgmc_set_band_min_n(self.h, band_min_n)
 
     def set_coarse_threads(self, threads: int):
-        """Threads per CTA of the coarse-grid kernel (mgmc_set_coarse_threads; 0 = by chain count)."""
+        """Threads per CTA of the coarse-grid kernel (mgmc_set_coarse_threads; 0 = by its largest grid)."""
         mgmc_set_coarse_threads(self.h, threads)
 
     def get_state(self, c, x, stream=None):
