@@ -65,7 +65,9 @@ typedef struct mgmc_ctx* mgmc_handle;
 
 /* Device-memory provider.  alloc(bytes, stream, ctx) returns device memory
  * or NULL; free(ptr, stream, ctx) returns it.  Both are called only from
- * mgmc_create / mgmc_destroy on the caller's thread. */
+ * mgmc_create / mgmc_destroy on the caller's thread.  Memory that does not start
+ * on a 256-byte boundary is given back at once and asked for again with 255 bytes
+ * of room. */
 typedef struct {
     void* (*alloc)(size_t bytes, void* stream, void* ctx);
     void (*free)(void* ptr, void* stream, void* ctx);

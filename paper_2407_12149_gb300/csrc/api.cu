@@ -57,9 +57,15 @@ struct Buffers {
             if (cudaMalloc(&p, bytes) != cudaSuccess) p = nullptr;
         } else {
             p = alloc.alloc(bytes, (void*)stream, alloc.ctx);
+            if (reinterpret_cast<uintptr_t>(p) & 255) {
+                // bulk and TMA copies start on 16-byte boundaries: room to align in
+                alloc.free(p, (void*)stream, alloc.ctx);
+                p = alloc.alloc(bytes + 255, (void*)stream, alloc.ctx);
+            }
         }
-        if (p) list.push_back(p);
-        return p;
+        if (!p) return nullptr;
+        list.push_back(p);
+        return (void*)((reinterpret_cast<uintptr_t>(p) + 255) & ~(uintptr_t)255);
     }
     void release()
     {

@@ -577,12 +577,19 @@ struct UnetCtx {
     {
         void* p = nullptr;
         bytes = (std::max<size_t>(bytes, 1) + 255) / 256 * 256;
-        if (use_alloc)
+        if (use_alloc) {
             p = alloc.alloc(bytes, stream, alloc.ctx);
-        else if (cudaMalloc(&p, bytes) != cudaSuccess)
+            if (reinterpret_cast<uintptr_t>(p) & 255) {
+                // TMA copies and 16-byte loads start on 16-byte boundaries: room to align in
+                alloc.free(p, stream, alloc.ctx);
+                p = alloc.alloc(bytes + 255, stream, alloc.ctx);
+            }
+        } else if (cudaMalloc(&p, bytes) != cudaSuccess) {
             p = nullptr;
-        if (p) blocks.push_back(p);
-        return p;
+        }
+        if (!p) return nullptr;
+        blocks.push_back(p);
+        return (void*)((reinterpret_cast<uintptr_t>(p) + 255) & ~(uintptr_t)255);
     }
     void release()
     {
