@@ -301,9 +301,10 @@ mgmc_status mgmc_set_band_min_n(mgmc_handle h, int band_min_n);
 /* Threads per CTA of the 2D coarse-grid kernel (one CTA per chain, all grids with
  * n <= coarse_max_n in shared memory): 0 (default) chooses 256, or 512 when
  * a 63^2 grid is inside; else a multiple of 32 in [64, 1024] (values above the kernel's
- * limit, 512 in FP32 2D and 256 otherwise, run at the limit).  The kernel's arithmetic does not depend on it (the states are bitwise
- * the same); only the time of its barrier-bound phases does.  The graph is captured
- * again on the next sampling call.  MGMC_ERR_ARG for other values. */
+ * limit, 512 in FP32 2D and 256 otherwise, run at the limit).  The kernel's arithmetic
+ * does not depend on it (the states are bitwise the same); only the time of its
+ * barrier-bound phases does.  The graph is captured again on the next sampling call.
+ * MGMC_ERR_ARG for other values. */
 mgmc_status mgmc_set_coarse_threads(mgmc_handle h, int threads);
 
 /* Benchmark timing: with enable != 0 the captured cycle records CUDA events
@@ -388,9 +389,10 @@ mgmc_status mgmc_tc_gemm(const void* A, int lda, const void* B, int ldb, void* C
 /* Waits for the work on `stream`, then MGMC_ERR_TIMEOUT if a product on the current
  * device, of this or another thread, has given up since this thread last asked. */
 mgmc_status mgmc_tc_gemm_status(void* stream);
-/* mgmc_tc_gemm with the bound of the kernel's waits in nanoseconds: 0 the default; a
- * negative value (tests) makes the part that issues the products give up on its first
- * operands and the others after -wait_ns. */
+/* mgmc_tc_gemm with a bound in nanoseconds for the kernel's waits, for tests of what
+ * happens when they give up: > 0 bounds the waits of the parts that copy operands in
+ * and results out, < 0 also makes the part that issues the products give up at once
+ * (the others after -wait_ns); 0 is mgmc_tc_gemm. */
 mgmc_status mgmc_tc_gemm_bounded(const void* A, int lda, const void* B, int ldb, void* C, int M, int N, int K,
                                  int splits, int epilogue, const float* bias, void* stream, int64_t wait_ns);
 

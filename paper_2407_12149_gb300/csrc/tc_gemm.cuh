@@ -36,8 +36,8 @@ int sm_count();
 bool tc_gemm_plan(TcGemm* g, const void* A, int lda, const void* B, int ldb, int M, int N, int K, int splits);
 // Launch; C is float or __nv_bfloat16 [M][N] (row-major), bias float [N] or NULL.
 // status: device int that counts the CTAs in which a bounded wait gave up (NULL: a counter of
-// the device, see tc_gemm_gave_up).  wait_ns: bound of the waits (0: 1 s; < 0, a test of the
-// give-up path: the MMA issuer gives up on its first operands, the other roles after -wait_ns).
+// the device, see tc_gemm_gave_up).  wait_ns, for tests of the give-up path: bound of the waits
+// beside the MMA issuer's (0: 1 s); < 0: the issuer gives up at once, the others after -wait_ns.
 cudaError_t tc_gemm_run(const TcGemm& g, void* C, int epilogue, const float* bias, int* status, long long wait_ns,
                         cudaStream_t st);
 // The current device's counter of such CTAs once the work on `st` is done (synchronises it).

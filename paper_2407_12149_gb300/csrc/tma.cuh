@@ -55,8 +55,8 @@ constexpr unsigned long long kWaitNs = 1000000000ull;
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity, long long limit_ns = 0)
 {
     if (limit_ns < 0) return false;
-    const unsigned long long bound = limit_ns > 0 ? (unsigned long long)limit_ns : kWaitNs;
     if (mbar_test(bar, parity)) return true;
+    const unsigned long long bound = limit_ns > 0 ? (unsigned long long)limit_ns : kWaitNs;
     const unsigned long long t0 = global_ns();
     for (unsigned it = 1; it < (1u << 30); ++it) {
         if (mbar_test(bar, parity)) return true;

@@ -269,10 +269,10 @@ def tc_gemm(A, B, out=None, splits=1, epilogue=0, bias=None, stream=None, wait_n
     N = B.shape[0]
     if out is None:
         out = torch.empty(M, N, dtype=torch.bfloat16 if epilogue & EPI_BF16 else torch.float32, device=A.device)
-    _check(load().mgmc_tc_gemm_bounded(ctypes.c_void_p(A.data_ptr()), A.stride(0), ctypes.c_void_p(B.data_ptr()),
-                                       B.stride(0), ctypes.c_void_p(out.data_ptr()), M, N, K, splits, epilogue,
-                                       ctypes.c_void_p(bias.data_ptr()) if bias is not None else None,
-                                       _stream_handle(stream), int(wait_ns)))
+    args = (ctypes.c_void_p(A.data_ptr()), A.stride(0), ctypes.c_void_p(B.data_ptr()), B.stride(0),
+            ctypes.c_void_p(out.data_ptr()), M, N, K, splits, epilogue,
+            ctypes.c_void_p(bias.data_ptr()) if bias is not None else None, _stream_handle(stream))
+    _check(load().mgmc_tc_gemm_bounded(*args, int(wait_ns)) if wait_ns else load().mgmc_tc_gemm(*args))
     return out
 
 
