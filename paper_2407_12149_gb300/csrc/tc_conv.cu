@@ -227,18 +227,18 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv(const __grid_constant_
         const unsigned id = tc5::idesc(NT, false);
         int k = 0;
         RingPos rp, bp;
-        bool ok = !g.resident || mbar_wait(&wbar, 0u);
+        bool ok = g.wait_ns >= 0 && (!g.resident || mbar_wait(&wbar, 0u));
         for (long long mt = blockIdx.x / g.ntiles_n; mt < mtiles && ok && !aborted; mt += step)
             for (int a = 0; a < items && ok; a += unit, bp.next(NBUF)) {
                 const int buf = bp.slot;
-                if (!mbar_wait(&tempty[buf], bp.par ^ 1u, lim)) {
+                if (!mbar_wait(&tempty[buf], bp.par ^ 1u)) {
                     ok = false;
                     break;
                 }
                 tc5::fence_after();
                 for (int c = 0; c < unit; ++c, ++k, rp.next(S)) {
                     const int s = rp.slot;
-                    if (!mbar_wait(&full[s], rp.par, g.wait_ns)) {
+                    if (!mbar_wait(&full[s], rp.par)) {
                         ok = false;
                         break;
                     }
@@ -358,13 +358,13 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
         const unsigned id = tc5::idesc(NT, false);
         RingPos kp, wp, bp;       // the line above the tile, the next line to wait for, the accumulator
         int waited = 0;           // lines known to have arrived
-        bool ok = mbar_wait(&wbar, 0u);
+        bool ok = g.wait_ns >= 0 && mbar_wait(&wbar, 0u);
         for (long long t0 = beg; t0 < end && ok && !aborted;) {
             const long long strip = t0 >> g.lgH;
             const long long t1 = min(end, (strip + 1) << g.lgH);
             for (long long t = t0; t < t1 && ok; ++t, kp.next(NL)) {
                 for (int q = t == t0 ? 3 : 1; q > 0; --q, ++waited, wp.next(NL)) {
-                    ok = mbar_wait(&full[wp.slot], wp.par, g.wait_ns);
+                    ok = mbar_wait(&full[wp.slot], wp.par);
                     if (!ok) break;   // `waited` counts the lines that have arrived
                 }
                 consumed = waited;
@@ -372,7 +372,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_line(const __grid_cons
                 for (int tap = 0; tap < 9 && ok; ++tap) {
                     const int buf = bp.slot;
                     if (DG || tap == 0) {
-                        ok = mbar_wait(&tempty[buf], bp.par ^ 1u, lim);
+                        ok = mbar_wait(&tempty[buf], bp.par ^ 1u);
                         if (!ok) break;
                         tc5::fence_after();
                     }
@@ -491,10 +491,12 @@ __global__ void __launch_bounds__(128, 1) k_wgrad(const __grid_constant__ WgradA
         issued = kb;
     } else if (warp == 1 && lane == 0) {
         const unsigned id = tc5::idesc(NT, true);
+        const int n = g.wait_ns < 0 ? 0 : nkb;
+        if (g.wait_ns < 0) aborted = 1;
         int kb = 0;
-        for (; kb < nkb; ++kb) {
+        for (; kb < n; ++kb) {
             const int s = kb % kWgStages;
-            if (!mbar_wait(&full[s], (unsigned)((kb / kWgStages) & 1), g.wait_ns)) {
+            if (!mbar_wait(&full[s], (unsigned)((kb / kWgStages) & 1))) {
                 aborted = 1;
                 break;
             }
