@@ -6,14 +6,17 @@
 //  - -2 ln u: table-driven (P. T. P. Tang, "Table-driven implementation of the logarithm
 //    function in IEEE floating-point arithmetic", ACM TOMS 16, 1990): u = 2^e z, z in
 //    [0.6875, 1.375), z inv_i = 1 + r with |r| < 2^-7.4 and the Taylor series of log(1 + r); the
-//    cell next to 1 has inv = 1, so a small logarithm keeps its relative accuracy;
+//    cell next to 1 has inv = 1, so a small logarithm keeps its relative accuracy.  Cell and exponent
+//    come from the high word less 0x3fe60000, its top mantissa bits and an arithmetic shift, as in
+//    the log of Arm's Optimized Routines (table and polynomial are not that one's);
 //  - its square root: Newton's iteration from the hardware reciprocal square root;
 //  - sine and cosine of 2 pi u: the nearest odd multiple of 2 pi / 256 from a table, Taylor
 //    series of the remainder, angle addition.
-// 38 FP64 instructions a pair instead of about 70 (log, sqrt, sincospi and the integer
-// conversions).  Error relative to the radius against 113-bit arithmetic over 10^6 draws with
-// uniforms next to 0 and 1 among them: rms 5.8e-17 (library functions 5.9e-17), largest 3.3e-16
-// (3.0e-16); 53-bit pairs rms 6.0e-17 (18e-17: their angle was rounded before the call).
+// 38 FP64 instructions a pair (14 + 6 + 2 + 16 below) instead of about 70 (log, sqrt, sincospi and
+// the integer conversions).  Error relative to the radius against extended precision over 10^6 draws: rms
+// 5.8e-17 (library functions 5.9e-17), largest 3.4e-16 (3.0e-16); 53-bit pairs rms 6.0e-17 and 3.7e-16
+// (18e-17: their angle was rounded before the call).  tests/test_normal64_host.py bounds it by five
+// roundings at the ends of every cell, next to 0 and 1, at ties and at the carry to u = 1.
 // Measured (GB300): 31^2 FP64 chain, 8 cycles 584 -> 418 us; 1023^2 FP64, 2 cycles 1883 -> 1470 us.
 #pragma once
 #include <cuda_runtime.h>
