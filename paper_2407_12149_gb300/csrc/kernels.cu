@@ -583,16 +583,20 @@ __device__ __forceinline__ void residual25(const DevLevel<double>& L)
         const long long e = on ? site_offset(2, L.pitch, L.plane, L.base, t % L.n, t / L.n, 0) : 0;
         double acc = 0.0;
         if (on) {
-            if (lane == 0) acc = fma(-L.coef[e], L.x[e], L.f ? L.f[e] : 0.0);
 #pragma unroll
-            for (int q = 0; q < 24 / LPS; ++q) {
-                const int u = lane + LPS * q, o = u + (u >= 12 ? 1 : 0);
-                acc = fma(-coef25_at(L, e, o), L.x[e + off25(o, L.pitch)], acc);
+            for (int q = 0; q < PER; ++q) {
+                const int u = lane * PER + q;
+                if (LPS == 1 && q == 12) acc = fma(L.coef[e], L.x[e], acc);
+                acc = fma(coef25_at(L, e, u + (u >= 12 ? 1 : 0)), L.x[e + off25(u + (u >= 12 ? 1 : 0), L.pitch)], acc);
             }
         }
 #pragma unroll
-        for (int s = 1; s < LPS; s <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
-        if (on && lane == 0) L.res[e] = acc;
+        for (int s = 1; s < H; s <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, s);
+        if (LPS > 1) {
+            if (on && lane < H) acc = fma(L.coef[e], L.x[e], acc);
+            acc += __shfl_xor_sync(0xffffffffu, acc, H);
+        }
+        if (on && lane == 0) L.res[e] = (L.f ? L.f[e] : 0.0) - acc;
     }
 }
 
@@ -1048,8 +1052,12 @@ void launch_cycle_small(const DevLevel<T>* levels_dev, int top, const DevProblem
                         const double* gain, int n0, const int4* ops, int n_ops, int n_pre, double* zb, cudaStream_t st,
                         int& launches)
 {
-    k_cycle_small<T><<<1, kSmallCycleThreads, kSmallArena, st>>>(levels_dev, top, P, chol, gain, n0, ops, n_ops, n_pre,
-                                                                 (unsigned)kSmallArena, zb);
+    // a visit of few phases does not earn the copies of its grids (FP32 W-cycle with 8 observations, us, with
+    // / without copies: 3^2, 8 phases 31.3 / 27.1; 7^2, 16 phases 51.7 / 45.6; 15^2 has 32): room for the
+    // drawn normals only, and every field stays in global memory
+    const size_t arena = n_ops >= kSmallStageOps ? kSmallArena : ((size_t)n_pre * sizeof(double) + 15) / 16 * 16;
+    k_cycle_small<T><<<1, kSmallCycleThreads, arena, st>>>(levels_dev, top, P, chol, gain, n0, ops, n_ops, n_pre,
+                                                           (unsigned)arena, zb);
     ++launches;
 }
 

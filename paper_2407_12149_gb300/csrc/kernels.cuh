@@ -24,6 +24,7 @@ constexpr int kSmallCycleThreads = 512;
 constexpr int kSmallMaxLevels = 16;   // grids 0..top held by the kernel (top < 16)
 constexpr int kSmallMaxOps = 1024;    // phases staged in shared memory (later ones read from global)
 constexpr int kSmallSharedN = 15;     // grids up to this size live in shared memory
+constexpr int kSmallStageOps = 24;    // .. if the visit has at least as many phases
 constexpr int kSmallPreN = 7;         // grids up to this size have their site normals drawn at the start
 constexpr int kSmallMaxPre = 4096;    // normals drawn at the start, at most
 // dynamic shared memory of the kernel: 227 KB less its static part
