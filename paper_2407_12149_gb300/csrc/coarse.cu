@@ -516,58 +516,53 @@ __device__ __forceinline__ void s_coarsest(const CoarseJob<T>& J, int m, const B
         tm.sync();
         return;
     }
-    // larger coarsest grids: two triangular solves, the CTA updating the remaining unknowns.  While
-    // they are more than the threads, a thread's four loads of the factor are in flight together,
-    // and thread 0's next diagonal entry is loaded a step ahead (a cycle with 961 / 343 / 225 coarsest
-    // unknowns, FP64: 1520 / 465 / 285 us; one load at a time 2000 / 552 / 320).  256 threads at most:
-    // with the 512 of a 63^2 grid a step takes longer (961 unknowns, FP32: 1770 against 1680 us)
+    // larger coarsest grids: two triangular solves, the CTA updating the remaining unknowns.  Thread 0's
+    // next diagonal entry is loaded a step ahead, a thread's loads of the factor two at a time (a cycle
+    // with 961 coarsest unknowns in FP64 / FP32, 225 in FP64: 1657 / 1565 / 324 us; one load after the other
+    // 2060 / 1774 / 345.  Four at a time: 83 registers in FP32, and one CTA per SM instead of two)
     double* r = vec;
     const double* chol = J.chol;
-    const int tid = threadIdx.x, nt = tm.nt;
-    const int ns = min(nt, 256);
 #pragma unroll 1
-    for (int s = tid; s < n0; s += nt) {
+    for (int s = threadIdx.x; s < n0; s += tm.nt) {
         double acc = (double)b.F[at(s)];
 #pragma unroll 4
         for (int k = 0; k < m; ++k) acc += J.e0[(long long)k * n0 + s] * d[k];   // (B_0 Gamma^-1 d)_s
         r[s] = acc;
     }
     tm.sync();
-    // r[first ..] of `left` unknowns, minus yi times the entries col[0], col[ld], ..
-    auto update = [&](int first, int left, const double* col, long long ld, double yi) {
-        if (tid >= ns) return;
-        if (left <= ns) {
-            if (tid < left) r[first + tid] -= col[tid * ld] * yi;
-            return;
-        }
-        double c[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) c[q] = tid + q * ns < left ? col[(tid + q * ns) * ld] : 0.0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (tid + q * ns < left) r[first + tid + q * ns] -= c[q] * yi;
-#pragma unroll 1
-        for (int t = tid + 4 * ns; t < left; t += ns) r[first + t] -= col[t * ld] * yi;
-    };
-    double diag = chol[0];
+    double diag = chol[0];   // thread 0 divides
 #pragma unroll 1
     for (int i = 0; i < n0; ++i) {
-        if (tid == 0) r[i] = r[i] / diag;
+        if (threadIdx.x == 0) r[i] = r[i] / diag;
         tm.sync();
-        if (tid == 0 && i + 1 < n0) diag = chol[(long long)(i + 1) * (n0 + 1)];
-        update(i + 1, n0 - i - 1, chol + (long long)(i + 1) * n0 + i, n0, r[i]);
+        if (threadIdx.x == 0 && i + 1 < n0) diag = chol[(i + 1) * (n0 + 1)];
+        const double yi = r[i];
+#pragma unroll 1
+        for (int t = i + 1 + threadIdx.x; t < n0; t += 2 * tm.nt) {
+            const int u = t + tm.nt;
+            const double ct = chol[t * n0 + i], cu = u < n0 ? chol[u * n0 + i] : 0.0;
+            r[t] -= ct * yi;
+            if (u < n0) r[u] -= cu * yi;
+        }
         tm.sync();
     }
 #pragma unroll 1
-    for (int s = tid; s < n0; s += nt) r[s] += zc[s];
+    for (int s = threadIdx.x; s < n0; s += tm.nt) r[s] += zc[s];
     tm.sync();
-    diag = chol[(long long)(n0 - 1) * (n0 + 1)];
+    diag = chol[n0 * n0 - 1];
 #pragma unroll 1
     for (int i = n0 - 1; i >= 0; --i) {
-        if (tid == 0) r[i] = r[i] / diag;
+        if (threadIdx.x == 0) r[i] = r[i] / diag;
         tm.sync();
-        if (tid == 0 && i > 0) diag = chol[(long long)(i - 1) * (n0 + 1)];
-        update(0, i, chol + (long long)i * n0, 1, r[i]);
+        if (threadIdx.x == 0 && i > 0) diag = chol[(i - 1) * (n0 + 1)];
+        const double xi = r[i];
+#pragma unroll 1
+        for (int t = threadIdx.x; t < i; t += 2 * tm.nt) {
+            const int u = t + tm.nt;
+            const double ct = chol[i * n0 + t], cu = u < i ? chol[i * n0 + u] : 0.0;
+            r[t] -= ct * xi;
+            if (u < i) r[u] -= cu * xi;
+        }
         tm.sync();
     }
 #pragma unroll 1
@@ -683,7 +678,8 @@ __global__ void k_coarse_image(const CoarseJob<T>* __restrict__ job, unsigned ch
 }
 
 // One CTA per chain (2D batches) or the one chain of a handle; blockDim.x - kHelp compute
-// threads.  Their number never changes the arithmetic.
+// threads.  Their number never changes the arithmetic.  At 80 registers two CTAs of 256 + 128 threads
+// share an SM (at 88 one does: 2000 chains of 7^2 in FP32 245 -> 313 us a cycle).
 template <typename T, int DIM>
 __global__ void __launch_bounds__(coarse_max_threads<T, DIM>() + kHelp) k_coarse_cycle(const CoarseJob<T>* __restrict__ jobs)
 {
