@@ -570,9 +570,10 @@ __device__ __forceinline__ void colour25(const DevLevel<double>& L, int c, Z&& z
 // r = f - A x of a 25-point grid, LPS lanes per site.  The couplings before and after the centre sum
 // to about minus the centre's product: it joins the first half before the second half is added, so
 // that no partial sum exceeds half of it (all lanes' sums first, the centre's product among them,
-// had 2.8 times the error of the state against extended precision: 63^2, six W-cycles, 7.6e-14 -> 2.1e-13)
+// had 2.8 times the error of the state against extended precision: 63^2, six W-cycles, 7.6e-14 -> 2.1e-13).
+// Not inlined: its registers cost the kernel's other phases (64 observations, W-cycles 5 %).
 template <int LPS>
-__device__ __forceinline__ void residual25(const DevLevel<double>& L)
+__device__ __noinline__ void residual25(const DevLevel<double>& L)
 {
     constexpr int H = LPS > 1 ? LPS / 2 : 1, PER = LPS > 1 ? 12 / H : 24;   // lanes of a half, couplings of a lane
     const int N = L.n * L.n, lane = threadIdx.x & (LPS - 1);
