@@ -1146,8 +1146,15 @@ mgmc_status mgmc_tc_gemm_bounded(const void* A, int lda, const void* B, int ldb,
         return unet_fail(MGMC_ERR_ARG, "mgmc_tc_gemm: C or bias is not aligned to its elements");
     cudaStream_t st = (cudaStream_t)stream;
     TcGemm g;
-    if (!tc_gemm_plan(&g, A, lda, B, ldb, M, N, K, splits))
-        return unet_fail(MGMC_ERR_ARG, "mgmc_tc_gemm: TMA descriptor encoding failed (alignment, lda/ldb)");
+    bool planned = tc_gemm_plan(&g, A, lda, B, ldb, M, N, K, splits);
+    if (!planned) {
+        // the encoder needs a current context, which a thread's first CUDA call does not find
+        int dev = 0;
+        UNET_CUDA(cudaGetDevice(&dev));
+        UNET_CUDA(cudaSetDevice(dev));
+        planned = tc_gemm_plan(&g, A, lda, B, ldb, M, N, K, splits);
+    }
+    if (!planned) return unet_fail(MGMC_ERR_ARG, "mgmc_tc_gemm: TMA descriptor encoding failed (alignment, lda/ldb)");
     if (g.splits == 1) {
         UNET_CUDA(tc_gemm_run(g, C, epilogue, bias, nullptr, (long long)wait_ns, st));
         return MGMC_OK;
