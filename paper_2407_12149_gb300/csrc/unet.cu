@@ -804,38 +804,94 @@ float host_loss(UnetCtx* u, int B)
     return (float)(s / ((double)B * u->n * u->n));
 }
 
-// Partial sums of split products are stream-ordered memory of one pool per device: products of
-// several streams and threads never share them, and the pool keeps at most kSplitKeep bytes
-// between calls (memory given back at every synchronisation costs a mapping in the next call).
+// Partial sums of split products.  A stream keeps its scratch for its next product (stream order
+// keeps them apart, and the caller holds the lock over its two launches, so that two threads on one
+// stream do not mix theirs); streams are known by their ids, which no later stream has again.  Under
+// capture, and beyond kSplitStreams streams or kSplitKeep bytes kept, the memory is the call's alone.
+// All of it is stream-ordered memory of one pool per device.  (Allocated and released by every call, a
+// small product took 22 -> 28 us with a wait after each.)
 constexpr unsigned long long kSplitKeep = 512ull << 20;
-cudaError_t split_pool(cudaMemPool_t* pool)
-{
-    static std::mutex mu;
-    static std::map<int, cudaMemPool_t> pools;
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = pools.find(dev);
-    if (it == pools.end()) {
-        cudaMemPoolProps props{};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.handleTypes = cudaMemHandleTypeNone;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = dev;
-        cudaMemPool_t p = nullptr;
-        e = cudaMemPoolCreate(&p, &props);
-        if (e != cudaSuccess) return e;
-        unsigned long long keep = kSplitKeep;
-        e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
-        if (e != cudaSuccess) {
-            cudaMemPoolDestroy(p);
-            return e;
+constexpr size_t kSplitStreams = 64;
+struct SplitScratch {
+    struct Slot {
+        int dev;
+        unsigned long long stream;
+        float* part;
+        size_t bytes;
+    };
+    std::mutex mu;
+    std::map<int, cudaMemPool_t> pools;
+    std::vector<Slot> slots;
+    size_t kept = 0;
+
+    cudaError_t pool(int dev, cudaMemPool_t* out)
+    {
+        auto it = pools.find(dev);
+        if (it == pools.end()) {
+            cudaMemPoolProps props{};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.handleTypes = cudaMemHandleTypeNone;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            cudaMemPool_t p = nullptr;
+            cudaError_t e = cudaMemPoolCreate(&p, &props);
+            if (e != cudaSuccess) return e;
+            unsigned long long keep = kSplitKeep;
+            e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+            if (e != cudaSuccess) {
+                cudaMemPoolDestroy(p);
+                return e;
+            }
+            it = pools.emplace(dev, p).first;
         }
-        it = pools.emplace(dev, p).first;
+        *out = it->second;
+        return cudaSuccess;
     }
-    *pool = it->second;
-    return cudaSuccess;
+
+    // `bytes` for work on `st` (lock held); *own: the caller releases them behind its work
+    cudaError_t take(size_t bytes, cudaStream_t st, float** part, bool* own)
+    {
+        int dev = 0;
+        unsigned long long id = 0;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e == cudaSuccess) e = cudaStreamIsCapturing(st, &cap);
+        if (e != cudaSuccess) return e;
+        Slot* slot = nullptr;
+        if (cap == cudaStreamCaptureStatusNone) {
+            e = cudaStreamGetId(st, &id);
+            if (e != cudaSuccess) return e;
+            for (Slot& s : slots)
+                if (s.dev == dev && s.stream == id) slot = &s;
+        }
+        *own = false;
+        if (slot && slot->bytes >= bytes) {
+            *part = slot->part;
+            return cudaSuccess;
+        }
+        cudaMemPool_t p;
+        e = pool(dev, &p);
+        if (e == cudaSuccess) e = cudaMallocFromPoolAsync((void**)part, bytes, p, st);
+        if (e != cudaSuccess) return e;
+        const size_t had = slot ? slot->bytes : 0;
+        *own = cap != cudaStreamCaptureStatusNone || (!slot && slots.size() >= kSplitStreams) ||
+               kept - had + bytes > kSplitKeep;
+        if (*own) return cudaSuccess;
+        kept += bytes - had;
+        if (!slot) {
+            slots.push_back({dev, id, *part, bytes});
+            return cudaSuccess;
+        }
+        e = cudaFreeAsync(slot->part, st);   // behind the stream's earlier products
+        slot->part = *part;
+        slot->bytes = bytes;
+        return e;
+    }
+};
+SplitScratch& split_scratch()
+{
+    static SplitScratch* s = new SplitScratch;   // not destroyed: a thread may still be in a call at exit
+    return *s;
 }
 
 }  // namespace
@@ -1159,13 +1215,14 @@ mgmc_status mgmc_tc_gemm_bounded(const void* A, int lda, const void* B, int ldb,
         UNET_CUDA(tc_gemm_run(g, C, epilogue, bias, nullptr, (long long)wait_ns, st));
         return MGMC_OK;
     }
-    cudaMemPool_t pool;
+    SplitScratch& scratch = split_scratch();
+    std::lock_guard<std::mutex> lock(scratch.mu);
     float* part = nullptr;
-    UNET_CUDA(split_pool(&pool));
-    UNET_CUDA(cudaMallocFromPoolAsync((void**)&part, sizeof(float) * (size_t)g.splits * M * N, pool, st));
+    bool own = false;
+    UNET_CUDA(scratch.take(sizeof(float) * (size_t)g.splits * M * N, st, &part, &own));
     cudaError_t e = tc_gemm_run(g, part, epilogue, bias, nullptr, (long long)wait_ns, st);
     if (e == cudaSuccess) e = tc_reduce_splits(part, g.splits, (long long)M * N, (float*)C, st);
-    const cudaError_t ef = cudaFreeAsync(part, st);
+    const cudaError_t ef = own ? cudaFreeAsync(part, st) : cudaSuccess;
     UNET_CUDA(e);
     UNET_CUDA(ef);
     return MGMC_OK;
