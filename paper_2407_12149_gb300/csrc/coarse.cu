@@ -29,11 +29,12 @@
 //    launch starts with a cold instruction cache, and an unrolled version of 170 KB spent
 //    30 thousand cycles a launch on instruction fetches.
 // The FP32 arithmetic of a site is that of stencil.cuh, with the update's last product and sum rounded apart.
-// Measured (GB300, against one CTA per chain with operands staged by loads, per-sweep
-// draws and triangular solves): cycle of one 31^2 FP64 chain 137 -> 73 us, of a 255^2 FP32
-// chain 142 -> 97 us, kernel inside a batch of eight 1023^2 chains 95 -> 50 us.  What is left
-// is the phases' own latency (about 600 cycles a colour, 2000 a low-rank step); grids with a
-// compile-time size or only four warps on the smallest ones measured no faster.
+// Measured (GB300, against one CTA per chain with operands staged by loads, per-sweep draws and
+// triangular solves): cycle of one 31^2 FP64 chain 137 -> 73 us (52 with the normals of
+// normal64.cuh), of a 255^2 FP32 chain 142 -> 97 us (90 with the low-rank launches of tile2d.cu),
+// cold launch inside a batch of 32 1023^2 chains 97 -> 38 us.  What is left is the phases' own
+// latency (about 600 cycles a colour, 2000 a low-rank step); grids with a compile-time size or
+// only four warps on the smallest ones measured no faster.
 #include <algorithm>
 
 #include "kernels.cuh"
